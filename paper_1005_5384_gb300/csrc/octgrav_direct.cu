@@ -5,6 +5,11 @@
 // in shared memory and reused by a block of 256 targets; the sources are cut
 // into fixed chunks whose partial sums are added in chunk order, so results
 // do not depend on scheduling.
+//
+// Bound by the FP64 pipe (about 1.6 lane operations per clock and SM, 17 of
+// them per pair): only the number of SMs that hold a block matters. The
+// chunks are therefore sized by the grid, not by the sources alone
+// (direct_chunks).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -41,7 +46,7 @@ __global__ void __launch_bounds__(TB) k_direct(const double* __restrict__ pos, c
     for (int k = 0; k < m; ++k) {
       if (base + k == ti) continue;  // self term excluded
       const double dx = sx[k] - xi, dy = sy[k] - yi, dz = sz[k] - zi;
-      const double r2 = ((dx * dx + dy * dy) + dz * dz) + eps2;
+      const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
       const double ri = rsqrt(r2);
       const double mr = sm[k] * ri;
       const double mr3 = mr * ri * ri;
@@ -60,31 +65,42 @@ __global__ void __launch_bounds__(TB) k_direct(const double* __restrict__ pos, c
   }
 }
 
+// One thread per target and component adds the chunks' partial sums in order;
+// eight loads are in flight at a time (there may be a few hundred chunks).
 __global__ void k_direct_sum(const double* __restrict__ part, int64_t nt, int nchunks, double G,
                              double* __restrict__ acc, double* __restrict__ pot) {
-  const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (t >= nt) return;
-  double s[4] = {0, 0, 0, 0};
-  for (int c = 0; c < nchunks; ++c)
-    for (int k = 0; k < 4; ++k) s[k] += part[4 * (c * nt + t) + k];
-  acc[3 * t] = G * s[0];
-  acc[3 * t + 1] = G * s[1];
-  acc[3 * t + 2] = G * s[2];
-  pot[t] = G * s[3];
+  const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (i >= 4 * nt) return;
+  double s = 0;
+#pragma unroll 8
+  for (int c = 0; c < nchunks; ++c) s += part[4 * c * nt + i];
+  const int64_t t = i >> 2;
+  const int k = static_cast<int>(i & 3);
+  if (k < 3) acc[3 * t + k] = G * s;
+  else pot[t] = G * s;
 }
 
 }  // namespace
 
-int64_t direct_chunks(int64_t n) { return std::max<int64_t>(1, std::min<int64_t>(64, (n + 16383) / 16384)); }
+// Source chunks: at most 16384 sources each (up to 64 chunks; a chunk is one
+// sequential FP64 sum), and as many as it takes for (target blocks) x chunks
+// to fill the 152 SMs with two blocks each: two keep the FP64 pipe busy and a
+// single wave of them has no ragged end. With the first limit alone 1024
+// targets of 300,000 particles ran on 76 SMs: 21.6 ms a call, 10.5 ms now.
+int64_t direct_chunks(int64_t n, int64_t nt) {
+  const int64_t blocks = std::max<int64_t>(1, (nt + TB - 1) / TB);
+  const int64_t sums = std::min<int64_t>(64, (n + 16383) / 16384), fill = std::min<int64_t>(2 * 152 / blocks, (n + TB - 1) / TB);
+  return std::max<int64_t>(1, std::max(sums, fill));
+}
 
 cudaError_t direct_sum(const double* pos, const double* mass, int64_t n, const int64_t* targets, int64_t nt,
                        double eps, double G, double* part, double* acc, double* pot, cudaStream_t st) {
   if (nt <= 0) return cudaSuccess;
-  const int64_t nch = direct_chunks(n);
+  const int64_t nch = direct_chunks(n, nt);
   const int64_t chunk = (n + nch - 1) / nch;
   dim3 grid(static_cast<unsigned>((nt + TB - 1) / TB), static_cast<unsigned>(nch));
   k_direct<<<grid, TB, 0, st>>>(pos, mass, n, targets, nt, eps * eps, chunk, part);
-  k_direct_sum<<<static_cast<unsigned>((nt + 255) / 256), 256, 0, st>>>(part, nt, static_cast<int>(nch), G, acc, pot);
+  k_direct_sum<<<static_cast<unsigned>((4 * nt + 255) / 256), 256, 0, st>>>(part, nt, static_cast<int>(nch), G, acc, pot);
   return cudaGetLastError();
 }
 

@@ -913,7 +913,7 @@ int octgrav_direct(const double* pos, const double* mass, int64_t n, const int64
   DevBuf dp, dm, dt, dpart, da, dpot;
   int rc;
   if ((rc = dp.reserve(24 * n)) || (rc = dm.reserve(8 * n)) || (rc = dt.reserve(targets ? 8 * nt : 8)) ||
-      (rc = dpart.reserve(32 * og::direct_chunks(n) * nt)) || (rc = da.reserve(24 * nt)) || (rc = dpot.reserve(8 * nt)))
+      (rc = dpart.reserve(32 * og::direct_chunks(n, nt) * nt)) || (rc = da.reserve(24 * nt)) || (rc = dpot.reserve(8 * nt)))
     return rc;
   CUDA_TRY(cudaMemcpyAsync(dp.p, pos, 24 * n, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dm.p, mass, 8 * n, cudaMemcpyHostToDevice, st));
