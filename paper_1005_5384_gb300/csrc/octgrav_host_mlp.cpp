@@ -208,27 +208,48 @@ static double splitmix_uniform(uint64_t& s) {
   return static_cast<double>(z >> 11) * (1.0 / 9007199254740992.0);
 }
 
+}  // extern "C"
+
+namespace {
+
+// One allocation for a call's device arrays, given back when the call ends.
+struct Scratch {
+  DevBuf buf;
+  size_t used = 0;
+  ~Scratch() { buf.release(); }
+  static size_t room(size_t floats) { return (4 * floats + 255) & ~static_cast<size_t>(255); }
+  float* take(size_t floats) {
+    float* at = reinterpret_cast<float*>(static_cast<char*>(buf.p) + used);
+    used += room(floats);
+    return at;
+  }
+};
+
+}  // namespace
+
+extern "C" {
+
 int octgrav_mlp_grad(const float* params, const float* x, const float* target, int64_t n, float* grad, float* loss,
                      void* stream) {
   if (!params || !x || !target || n < 1 || n > (1 << 30) || !grad) return fail(OCTGRAV_ERR_ARG, "bad argument");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  DevBuf bw, bx, bt, bg, bl;
-  int rc;
-  if ((rc = bw.reserve(4 * og::MLP_NPARAM)) || (rc = bx.reserve(4 * og::MLP_NF * n)) || (rc = bt.reserve(4 * n)) ||
-      (rc = bg.reserve(4 * og::MLP_NPARAM)) || (rc = bl.reserve(4)))
-    return rc;
-  CUDA_TRY(cudaMemcpyAsync(bw.p, params, 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(bx.p, x, 4 * og::MLP_NF * n, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(bt.p, target, 4 * n, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemsetAsync(bg.p, 0, 4 * og::MLP_NPARAM, st));
-  CUDA_TRY(cudaMemsetAsync(bl.p, 0, 4, st));
-  cudaError_t e = og::mlp_grad(static_cast<float*>(bw.p), static_cast<float*>(bx.p), static_cast<float*>(bt.p),
-                               static_cast<int>(n), static_cast<int>(n), 0, 0, true, static_cast<float*>(bg.p),
-                               static_cast<float*>(bl.p), st);
+  const int B = static_cast<int>(n);
+  const size_t nx = static_cast<size_t>(og::MLP_NF) * B, np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
+  Scratch S;
+  int rc = S.buf.reserve(2 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + Scratch::room(B) + Scratch::room(np) +
+                         Scratch::room(1));
+  if (rc) return rc;
+  float *w = S.take(og::MLP_NPARAM), *g = S.take(og::MLP_NPARAM), *dx = S.take(nx), *dt = S.take(B), *part = S.take(np),
+        *dl = S.take(1);
+  CUDA_TRY(cudaMemcpyAsync(w, params, 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dx, x, 4 * nx, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dt, target, 4 * n, cudaMemcpyHostToDevice, st));
+  cudaError_t e = og::mlp_grad(w, dx, dt, B, B, 0, 0, true, part, st);
+  if (e == cudaSuccess) e = og::mlp_gradient(part, B, g, dl, st);
   if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "gradient kernel failed: %s", cudaGetErrorString(e));
-  CUDA_TRY(cudaMemcpyAsync(grad, bg.p, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
   float l = 0;
-  CUDA_TRY(cudaMemcpyAsync(&l, bl.p, 4, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(grad, g, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(&l, dl, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   if (loss) *loss = l;
   return OCTGRAV_OK;
@@ -269,32 +290,26 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   float* w3 = W2 + NH * NH + NH;
   for (int k = 0; k < NH; ++k) w3[k] = static_cast<float>((2 * splitmix_uniform(rs) - 1) * std::sqrt(3.0 / NH));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  DevBuf bx, by, bw, bm, bv, bg, bl;
-  int rc;
-  if ((rc = bx.reserve(4 * X.size())) || (rc = by.reserve(4 * n)) || (rc = bw.reserve(4 * og::MLP_NPARAM)) ||
-      (rc = bm.reserve(4 * og::MLP_NPARAM)) || (rc = bv.reserve(4 * og::MLP_NPARAM)) ||
-      (rc = bg.reserve(4 * og::MLP_NPARAM)) || (rc = bl.reserve(4)))
-    return rc;
-  CUDA_TRY(cudaMemcpyAsync(bx.p, X.data(), 4 * X.size(), cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(by.p, y.data(), 4 * n, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(bw.p, w.data(), 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemsetAsync(bm.p, 0, 4 * og::MLP_NPARAM, st));
-  CUDA_TRY(cudaMemsetAsync(bv.p, 0, 4 * og::MLP_NPARAM, st));
   const int B = static_cast<int>(std::min<int64_t>(batch, n));
+  const size_t np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
+  Scratch S;
+  int rc = S.buf.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(X.size()) + Scratch::room(n) +
+                         Scratch::room(np) + Scratch::room(1));
+  if (rc) return rc;
+  float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(X.size()),
+        *dy = S.take(n), *part = S.take(np), *dl = S.take(1);
+  CUDA_TRY(cudaMemcpyAsync(dx, X.data(), 4 * X.size(), cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dy, y.data(), 4 * n, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dw, w.data(), 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemsetAsync(dm, 0, 2 * Scratch::room(og::MLP_NPARAM), st));  // dm and dv follow each other
   for (int k = 1; k <= steps; ++k) {
-    CUDA_TRY(cudaMemsetAsync(bg.p, 0, 4 * og::MLP_NPARAM, st));
-    CUDA_TRY(cudaMemsetAsync(bl.p, 0, 4, st));
-    cudaError_t e = og::mlp_grad(static_cast<float*>(bw.p), static_cast<float*>(bx.p), static_cast<float*>(by.p),
-                                 static_cast<int>(n), B, k, seed, false, static_cast<float*>(bg.p),
-                                 static_cast<float*>(bl.p), st);
-    if (e == cudaSuccess)
-      e = og::mlp_adam(static_cast<float*>(bw.p), static_cast<float*>(bm.p), static_cast<float*>(bv.p),
-                       static_cast<float*>(bg.p), static_cast<float>(lr), k, st);
+    cudaError_t e = og::mlp_grad(dw, dx, dy, static_cast<int>(n), B, k, seed, false, part, st);
+    if (e == cudaSuccess) e = og::mlp_adam(part, B, dw, dm, dv, static_cast<float>(lr), k, dl, st);
     if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "training kernels failed: %s", cudaGetErrorString(e));
   }
   float l = 0;
-  CUDA_TRY(cudaMemcpyAsync(w.data(), bw.p, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(&l, bl.p, 4, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(w.data(), dw, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(&l, dl, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
   // The range limits are the training extremes widened by kRangeMargin standard
   // deviations: an input equal to an extreme is in range however it is

@@ -157,11 +157,17 @@ struct MlpSampleArgs {
 };
 cudaError_t mlp_sample_features(const MlpSampleArgs& a, cudaStream_t st);
 cudaError_t mlp_sample_labels(const MlpSampleArgs& a, cudaStream_t st);
-// One training step's gradient (grad and loss accumulated, zero them first);
-// use_all: the B samples are X[0..B) instead of B counter-based draws.
+// A training step's gradient in two launches. mlp_grad writes the shares of
+// mlp_blocks(B) blocks to part (MLP_PART floats each); use_all: the B samples
+// are X[0..B) instead of B counter-based draws. mlp_gradient adds them into
+// grad and loss; mlp_adam adds them and updates the parameters, and writes the
+// step's loss.
+int mlp_blocks(int B);
 cudaError_t mlp_grad(const float* w, const float* X, const float* t, int n_total, int B, int step, uint64_t seed,
-                     bool use_all, float* grad, float* loss, cudaStream_t st);
-cudaError_t mlp_adam(float* w, float* m, float* v, const float* g, float lr, int step, cudaStream_t st);
+                     bool use_all, float* part, cudaStream_t st);
+cudaError_t mlp_gradient(const float* part, int B, float* grad, float* loss, cudaStream_t st);
+cudaError_t mlp_adam(const float* part, int B, float* w, float* m, float* v, float lr, int step, float* loss,
+                     cudaStream_t st);
 
 // Encode the 2-D tensor map over a cell-record array (n_cells rows of 64 B)
 // used by the gather4 staging. Returns cudaSuccess or an error.

@@ -100,130 +100,245 @@ __device__ __forceinline__ int sample_index(uint64_t seed, int step, int b, int 
   return static_cast<int>(z % static_cast<uint64_t>(n));
 }
 
-constexpr int TB = 32;  // samples per block in the gradient kernel
+constexpr int TB = 32;             // samples per tile: one per lane
+constexpr int GT = 256;            // threads of the gradient kernel (8 warps, 8 hidden units each)
+constexpr int RS = MLP_NH + 4;     // row stride of the activations: 16-byte rows, 8 rows on distinct banks
+constexpr int XS = MLP_NF + 8;     // row stride of the inputs
 
-// Gradient of L = sum_b (y_b - t_b)^2 / (2B) for the samples of one block,
-// added to grad; L added to loss. Dense layer algebra written out per sample
-// row and hidden unit, everything in shared memory.
-__global__ void __launch_bounds__(256) grad_kernel(const float* __restrict__ w, const float* __restrict__ X,
-                                                    const float* __restrict__ t, int n_total, int B, int step,
-                                                    uint64_t seed, int use_all, float* grad, float* loss) {
-  __shared__ float W[MLP_NPARAM];
-  __shared__ float xs[TB][MLP_NF + 1];
-  __shared__ float ts[TB];
-  __shared__ float h1[TB][MLP_NH + 1];  // relu(z1); sign of z1 kept as h1 > 0
-  __shared__ float z2[TB][MLP_NH + 1];  // becomes dz2
-  __shared__ float d1[TB][MLP_NH + 1];  // dz1
-  __shared__ float dy[TB];
-  const int tid = threadIdx.x;
-  const float* W1 = W;
-  const float* b1 = W1 + MLP_NH * MLP_NF;
+struct GradSmem {
+  float4 w1t[MLP_NF][MLP_NH / 4];  // W1 transposed: 8 consecutive units of one input are two 16-byte words
+  float4 w2t[MLP_NH][MLP_NH / 4];  // W2 transposed (layer 2) ...
+  float4 w2[MLP_NH][RS / 4];       // ... and as it is (back through layer 2)
+  float4 xs[TB][XS / 4];
+  float4 h1[TB][RS / 4];           // relu(z1); z1 > 0 iff h1 > 0
+  float4 dz2[TB][RS / 4];
+  float4 d1[TB][RS / 4];           // dz1
+  float b1[MLP_NH], b2[MLP_NH], w3[MLP_NH];
+  float ypart[GT / 32][TB];        // warps' shares of the output
+  float ts[TB];
+  float dy[2];                     // sums over the tile: dy and L
+  float gw3[MLP_NH];               // and w3's gradient
+  float b3;
+};
+
+__device__ __forceinline__ void fma8(float* z, const float4* w, float x) {
+  const float4 a = w[0], b = w[1];
+  z[0] = fmaf(a.x, x, z[0]);
+  z[1] = fmaf(a.y, x, z[1]);
+  z[2] = fmaf(a.z, x, z[2]);
+  z[3] = fmaf(a.w, x, z[3]);
+  z[4] = fmaf(b.x, x, z[4]);
+  z[5] = fmaf(b.y, x, z[5]);
+  z[6] = fmaf(b.z, x, z[6]);
+  z[7] = fmaf(b.w, x, z[7]);
+}
+
+// One block's share of the gradient of L = sum_b (y_b - t_b)^2 / (2B), written
+// to part[block] (MLP_PART floats: the parameters, then L).
+//
+// FP32 FMAs and shared-memory reads bound it (6 x 5057 flops a sample), so the
+// layout is made for the reads. Layers: lane = sample, warp w = units 8w ..
+// 8w + 7; a weight row's 8 values are the same for the whole warp (two
+// broadcast 16-byte reads for 8 FMAs), a sample's activations are read 16
+// bytes at a time from rows 8 of which lie on distinct banks. Weight
+// gradients: a 4 x 4 tile of (unit, input) per thread, summed over the
+// samples in registers and over the block's tiles, and written once: no
+// atomics, so a step's result does not depend on scheduling. One output per thread with
+// W2[j][i] read at a stride of 64 floats put all 32 lanes on one bank:
+// 43 us a step at B = 4096, 17 us now (both with the parameter update).
+__global__ void __launch_bounds__(GT) grad_kernel(const float* __restrict__ w, const float* __restrict__ X,
+                                                   const float* __restrict__ t, int n_total, int B, int step,
+                                                   uint64_t seed, int use_all, float* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  GradSmem& S = *reinterpret_cast<GradSmem*>(smem);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const float* b1 = w + MLP_NH * MLP_NF;
   const float* W2 = b1 + MLP_NH;
   const float* b2 = W2 + MLP_NH * MLP_NH;
   const float* w3 = b2 + MLP_NH;
-  for (int k = tid; k < MLP_NPARAM; k += blockDim.x) W[k] = w[k];
-  const int base = blockIdx.x * TB;
-  const int nb = min(TB, B - base);
-  for (int k = tid; k < TB * MLP_NF; k += blockDim.x) {
-    const int r = k / MLP_NF, f = k % MLP_NF;
-    float v = 0.f;
-    if (r < nb) {
-      const int sidx = use_all ? base + r : sample_index(seed, step, base + r, n_total);
-      v = X[static_cast<size_t>(sidx) * MLP_NF + f];
-      if (f == 0) ts[r] = t[sidx];
-    }
-    xs[r][f] = v;
-  }
+  float* w1t = reinterpret_cast<float*>(S.w1t);
+  float* w2t = reinterpret_cast<float*>(S.w2t);
+  float* w2s = reinterpret_cast<float*>(S.w2);
+  for (int k = tid; k < MLP_NH * MLP_NF; k += GT) w1t[(k % MLP_NF) * MLP_NH + k / MLP_NF] = w[k];
+  for (int k = tid; k < MLP_NH * MLP_NH; k += GT) w2s[(k / MLP_NH) * RS + k % MLP_NH] = W2[k];
   __syncthreads();
-  const float b3 = w3[MLP_NH];
+  for (int k = tid; k < MLP_NH * MLP_NH; k += GT) w2t[k] = w2s[(k % MLP_NH) * RS + k / MLP_NH];
+  if (tid < MLP_NH) {
+    S.b1[tid] = b1[tid];
+    S.b2[tid] = b2[tid];
+    S.w3[tid] = w3[tid];
+  }
+  if (tid == 0) S.b3 = w3[MLP_NH];
   const float invB = 1.f / static_cast<float>(B);
-  // layer 1
-  for (int k = tid; k < TB * MLP_NH; k += blockDim.x) {
-    const int r = k / MLP_NH, j = k % MLP_NH;
-    float z = b1[j];
-    for (int i = 0; i < MLP_NF; ++i) z = fmaf(W1[j * MLP_NF + i], xs[r][i], z);
-    h1[r][j] = fmaxf(z, 0.f);
+  const int u0 = 8 * wp;                                // this warp's units
+  const int ja = 4 * (tid >> 4), ib = 4 * (tid & 15);   // this thread's 4 x 4 tile of W2's gradient
+  const int jc = tid >> 2, ic = 3 * (tid & 3);          // and its three entries of W1's
+  float g2[4][4] = {}, g1[3] = {0.f, 0.f, 0.f};
+  float gb = 0.f;  // threads 0..63: b1; 64..127: b2; 128..191: w3; 192: b3; 193: L
+  const int tiles = (B + TB - 1) / TB;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int base = tile * TB, nb = min(TB, B - base);
+    __syncthreads();  // the weights are in, the last tile's activations are free
+    for (int k = tid; k < TB * MLP_NF; k += GT) {
+      const int r = k / MLP_NF, f = k % MLP_NF;
+      float v = 0.f;
+      if (r < nb) {
+        const int sidx = use_all ? base + r : sample_index(seed, step, base + r, n_total);
+        v = X[static_cast<size_t>(sidx) * MLP_NF + f];
+        if (f == 0) S.ts[r] = t[sidx];
+      }
+      reinterpret_cast<float*>(S.xs[r])[f] = v;
+    }
+    __syncthreads();
+    // layer 1
+    float z[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z[k] = S.b1[u0 + k];
+#pragma unroll
+    for (int q = 0; q < MLP_NF / 4; ++q) {
+      const float4 x = S.xs[lane][q];
+      fma8(z, &S.w1t[4 * q][u0 / 4], x.x);
+      fma8(z, &S.w1t[4 * q + 1][u0 / 4], x.y);
+      fma8(z, &S.w1t[4 * q + 2][u0 / 4], x.z);
+      fma8(z, &S.w1t[4 * q + 3][u0 / 4], x.w);
+    }
+    S.h1[lane][u0 / 4] = make_float4(fmaxf(z[0], 0.f), fmaxf(z[1], 0.f), fmaxf(z[2], 0.f), fmaxf(z[3], 0.f));
+    S.h1[lane][u0 / 4 + 1] = make_float4(fmaxf(z[4], 0.f), fmaxf(z[5], 0.f), fmaxf(z[6], 0.f), fmaxf(z[7], 0.f));
+    __syncthreads();
+    // layer 2
+#pragma unroll
+    for (int k = 0; k < 8; ++k) z[k] = S.b2[u0 + k];
+#pragma unroll 4
+    for (int q = 0; q < MLP_NH / 4; ++q) {
+      const float4 h = S.h1[lane][q];
+      fma8(z, &S.w2t[4 * q][u0 / 4], h.x);
+      fma8(z, &S.w2t[4 * q + 1][u0 / 4], h.y);
+      fma8(z, &S.w2t[4 * q + 2][u0 / 4], h.z);
+      fma8(z, &S.w2t[4 * q + 3][u0 / 4], h.w);
+    }
+    // output, residual
+    float yp = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) yp = fmaf(S.w3[u0 + k], fmaxf(z[k], 0.f), yp);
+    S.ypart[wp][lane] = yp;
+    __syncthreads();
+    float res = 0.f;  // every warp adds the shares in the same order
+    if (lane < nb) {
+      float y = S.b3;
+#pragma unroll
+      for (int q = 0; q < GT / 32; ++q) y += S.ypart[q][lane];
+      res = y - S.ts[lane];
+    }
+    const float dy = res * invB;
+    if (wp == 0) {
+      float l = 0.5f * res * res * invB, d = dy;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        l += __shfl_xor_sync(0xffffffffu, l, o);
+        d += __shfl_xor_sync(0xffffffffu, d, o);
+      }
+      if (lane == 0) S.dy[0] = d, S.dy[1] = l;
+    }
+    // w3's gradient and dz2 = dy w3 [z2 > 0]
+    float dz[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float g = dy * fmaxf(z[k], 0.f);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+      if (lane == 0) S.gw3[u0 + k] = g;
+      dz[k] = z[k] > 0.f ? dy * S.w3[u0 + k] : 0.f;
+    }
+    S.dz2[lane][u0 / 4] = make_float4(dz[0], dz[1], dz[2], dz[3]);
+    S.dz2[lane][u0 / 4 + 1] = make_float4(dz[4], dz[5], dz[6], dz[7]);
+    __syncthreads();
+    // dz1[r][i] = (sum_j dz2[r][j] W2[j][i]) [h1 > 0]
+    float e[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int q = 0; q < MLP_NH / 4; ++q) {
+      const float4 d = S.dz2[lane][q];
+      fma8(e, &S.w2[4 * q][u0 / 4], d.x);
+      fma8(e, &S.w2[4 * q + 1][u0 / 4], d.y);
+      fma8(e, &S.w2[4 * q + 2][u0 / 4], d.z);
+      fma8(e, &S.w2[4 * q + 3][u0 / 4], d.w);
+    }
+    const float4 ha = S.h1[lane][u0 / 4], hb = S.h1[lane][u0 / 4 + 1];
+    S.d1[lane][u0 / 4] = make_float4(ha.x > 0.f ? e[0] : 0.f, ha.y > 0.f ? e[1] : 0.f, ha.z > 0.f ? e[2] : 0.f,
+                                     ha.w > 0.f ? e[3] : 0.f);
+    S.d1[lane][u0 / 4 + 1] = make_float4(hb.x > 0.f ? e[4] : 0.f, hb.y > 0.f ? e[5] : 0.f, hb.z > 0.f ? e[6] : 0.f,
+                                         hb.w > 0.f ? e[7] : 0.f);
+    // W2's gradient: sum_r dz2[r][j] h1[r][i]
+#pragma unroll 4
+    for (int r = 0; r < TB; ++r) {
+      const float4 d = S.dz2[r][ja / 4], h = S.h1[r][ib / 4];
+      const float dd[4] = {d.x, d.y, d.z, d.w}, hh[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) g2[p][q] = fmaf(dd[p], hh[q], g2[p][q]);
+    }
+    __syncthreads();
+    // W1's gradient: sum_r dz1[r][j] x[r][i]; the biases' and w3's
+#pragma unroll 4
+    for (int r = 0; r < TB; ++r) {
+      const float d = reinterpret_cast<const float*>(S.d1[r])[jc];
+      const float* x = reinterpret_cast<const float*>(S.xs[r]) + ic;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) g1[q] = fmaf(d, x[q], g1[q]);
+    }
+    if (tid < 2 * MLP_NH) {
+      const float* col = reinterpret_cast<const float*>(tid < MLP_NH ? S.d1[0] : S.dz2[0]) + (tid & (MLP_NH - 1));
+      float g = 0.f;
+#pragma unroll 8
+      for (int r = 0; r < TB; ++r) g += col[r * RS];
+      gb += g;
+    } else if (tid < 3 * MLP_NH) {
+      gb += S.gw3[tid - 2 * MLP_NH];
+    } else if (tid < 3 * MLP_NH + 2) {
+      gb += S.dy[tid - 3 * MLP_NH];
+    }
   }
-  __syncthreads();
-  // layer 2
-  for (int k = tid; k < TB * MLP_NH; k += blockDim.x) {
-    const int r = k / MLP_NH, j = k % MLP_NH;
-    float z = b2[j];
-    for (int i = 0; i < MLP_NH; ++i) z = fmaf(W2[j * MLP_NH + i], h1[r][i], z);
-    z2[r][j] = z;
-  }
-  __syncthreads();
-  // output, residual, loss
-  if (tid < TB) {
-    float y = b3;
-    for (int j = 0; j < MLP_NH; ++j) y = fmaf(w3[j], fmaxf(z2[tid][j], 0.f), y);
-    const float res = tid < nb ? y - ts[tid] : 0.f;
-    dy[tid] = res * invB;
-    atomicAdd(loss, 0.5f * res * res * invB);
-  }
-  __syncthreads();
-  // output layer gradients
-  float* gW1 = grad;
-  float* gb1 = gW1 + MLP_NH * MLP_NF;
-  float* gW2 = gb1 + MLP_NH;
-  float* gb2 = gW2 + MLP_NH * MLP_NH;
-  float* gw3 = gb2 + MLP_NH;
-  if (tid < MLP_NH) {
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g = fmaf(dy[r], fmaxf(z2[r][tid], 0.f), g);
-    atomicAdd(gw3 + tid, g);
-  }
-  if (tid == MLP_NH) {
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g += dy[r];
-    atomicAdd(gw3 + MLP_NH, g);
-  }
-  __syncthreads();
-  // dz2 = dy w3 [z2 > 0]
-  for (int k = tid; k < TB * MLP_NH; k += blockDim.x) {
-    const int r = k / MLP_NH, j = k % MLP_NH;
-    z2[r][j] = z2[r][j] > 0.f ? dy[r] * w3[j] : 0.f;
-  }
-  __syncthreads();
-  // gW2[j][i] = sum_r dz2[r][j] h1[r][i]; gb2[j] = sum_r dz2[r][j]
-  for (int k = tid; k < MLP_NH * MLP_NH; k += blockDim.x) {
-    const int j = k / MLP_NH, i = k % MLP_NH;
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g = fmaf(z2[r][j], h1[r][i], g);
-    atomicAdd(gW2 + k, g);
-  }
-  if (tid < MLP_NH) {
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g += z2[r][tid];
-    atomicAdd(gb2 + tid, g);
-  }
-  // dz1[r][i] = (sum_j dz2[r][j] W2[j][i]) [h1 > 0]
-  for (int k = tid; k < TB * MLP_NH; k += blockDim.x) {
-    const int r = k / MLP_NH, i = k % MLP_NH;
-    float g = 0.f;
-    for (int j = 0; j < MLP_NH; ++j) g = fmaf(z2[r][j], W2[j * MLP_NH + i], g);
-    d1[r][i] = h1[r][i] > 0.f ? g : 0.f;
-  }
-  __syncthreads();
-  for (int k = tid; k < MLP_NH * MLP_NF; k += blockDim.x) {
-    const int j = k / MLP_NF, i = k % MLP_NF;
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g = fmaf(d1[r][j], xs[r][i], g);
-    atomicAdd(gW1 + k, g);
-  }
-  if (tid < MLP_NH) {
-    float g = 0.f;
-    for (int r = 0; r < TB; ++r) g += d1[r][tid];
-    atomicAdd(gb1 + tid, g);
-  }
+  float* out = part + static_cast<size_t>(blockIdx.x) * MLP_PART;
+  float* o2 = out + MLP_NH * MLP_NF + MLP_NH;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) out[jc * MLP_NF + ic + q] = g1[q];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o2[(ja + p) * MLP_NH + ib + q] = g2[p][q];
+  if (tid < MLP_NH) out[MLP_NH * MLP_NF + tid] = gb;
+  else if (tid < 3 * MLP_NH + 2) o2[MLP_NH * MLP_NH + tid - MLP_NH] = gb;  // b2, w3, b3, L follow each other
 }
 
-__global__ void adam_kernel(float* w, float* m, float* v, const float* g, float lr, float c1, float c2) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= MLP_NPARAM) return;
-  const float gk = g[k];
-  const float mk = 0.9f * m[k] + 0.1f * gk;
-  const float vk = 0.999f * v[k] + 0.001f * gk * gk;
+// Sum of the blocks' shares per parameter (and of L), then the Adam update
+// (w != NULL) or the gradient and L themselves. A block takes 32 parameters:
+// warp s adds the shares s, s + 8, ..., the warps' sums are added in order.
+__global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ part, int blocks, float* __restrict__ w,
+                                                      float* __restrict__ m, float* __restrict__ v, float lr, float c1,
+                                                      float c2, float* __restrict__ grad, float* __restrict__ loss) {
+  __shared__ float sum[8][32];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k = 32 * blockIdx.x + lane;
+  float s = 0.f;
+  if (k <= MLP_NPARAM) {
+#pragma unroll 8
+    for (int b = wp; b < blocks; b += 8) s += part[static_cast<size_t>(b) * MLP_PART + k];
+  }
+  sum[wp][lane] = s;
+  __syncthreads();
+  if (wp || k > MLP_NPARAM) return;
+  float g = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) g += sum[q][lane];
+  if (k == MLP_NPARAM) {
+    *loss = g;
+    return;
+  }
+  if (!w) {
+    grad[k] = g;
+    return;
+  }
+  const float mk = 0.9f * m[k] + 0.1f * g;
+  const float vk = 0.999f * v[k] + 0.001f * g * g;
   m[k] = mk;
   v[k] = vk;
   w[k] -= lr * (mk * c1) / (sqrtf(vk * c2) + 1e-8f);
@@ -244,16 +359,31 @@ cudaError_t mlp_sample_labels(const MlpSampleArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Blocks of a gradient over B samples: one per tile of 32, at most two per SM.
+int mlp_blocks(int B) {
+  const int tiles = B / TB + (B % TB != 0);
+  return tiles < 2 * 152 ? tiles : 2 * 152;
+}
+
 cudaError_t mlp_grad(const float* w, const float* X, const float* t, int n_total, int B, int step, uint64_t seed,
-                     bool use_all, float* grad, float* loss, cudaStream_t st) {
-  grad_kernel<<<(B + TB - 1) / TB, 256, 0, st>>>(w, X, t, n_total, B, step, seed, use_all ? 1 : 0, grad, loss);
+                     bool use_all, float* part, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem));
+  if (e != cudaSuccess) return e;
+  grad_kernel<<<mlp_blocks(B), GT, sizeof(GradSmem), st>>>(w, X, t, n_total, B, step, seed, use_all ? 1 : 0, part);
   return cudaGetLastError();
 }
 
-cudaError_t mlp_adam(float* w, float* m, float* v, const float* g, float lr, int step, cudaStream_t st) {
+cudaError_t mlp_gradient(const float* part, int B, float* grad, float* loss, cudaStream_t st) {
+  reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(part, mlp_blocks(B), nullptr, nullptr, nullptr, 0.f, 0.f, 0.f,
+                                                            grad, loss);
+  return cudaGetLastError();
+}
+
+cudaError_t mlp_adam(const float* part, int B, float* w, float* m, float* v, float lr, int step, float* loss,
+                     cudaStream_t st) {
   const float c1 = 1.f / (1.f - powf(0.9f, static_cast<float>(step)));
   const float c2 = 1.f / (1.f - powf(0.999f, static_cast<float>(step)));
-  adam_kernel<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(w, m, v, g, lr, c1, c2);
+  reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(part, mlp_blocks(B), w, m, v, lr, c1, c2, nullptr, loss);
   return cudaGetLastError();
 }
 

@@ -12,6 +12,9 @@ constexpr int MLP_NF = 12;  // inputs
 constexpr int MLP_NH = 64;  // hidden units per layer
 // Parameter vector: W1[64][12], b1[64], W2[64][64], b2[64], w3[64], b3.
 constexpr int MLP_NPARAM = MLP_NH * MLP_NF + MLP_NH + MLP_NH * MLP_NH + MLP_NH + MLP_NH + 1;  // 5057
+// One block's share of a gradient: the parameters, the loss, padding.
+constexpr int MLP_PART = 5088;
+static_assert(MLP_PART > MLP_NPARAM && MLP_PART % 32 == 0, "shares hold every parameter and the loss");
 // Criterion record (floats): mu[12], sigma[12], xmin[12], xmax[12], params[5057].
 constexpr int MLP_RECORD = 4 * MLP_NF + MLP_NPARAM;  // 5105
 
