@@ -260,26 +260,6 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   if (!features || !labels || !record || n < 2 || n > (1 << 30) || steps < 1 || batch < 1 || !(lr > 0))
     return fail(OCTGRAV_ERR_ARG, "bad argument");
   const int F = og::MLP_NF;
-  // targets: log10 of the error label; inputs standardised per feature
-  std::vector<float> y(n), X(static_cast<size_t>(n) * F);
-  double mu[og::MLP_NF] = {0}, sd[og::MLP_NF] = {0};
-  for (int64_t k = 0; k < n; ++k)
-    for (int i = 0; i < F; ++i) mu[i] += features[k * F + i];
-  for (int i = 0; i < F; ++i) mu[i] /= static_cast<double>(n);
-  for (int64_t k = 0; k < n; ++k)
-    for (int i = 0; i < F; ++i) sd[i] += (features[k * F + i] - mu[i]) * (features[k * F + i] - mu[i]);
-  for (int i = 0; i < F; ++i) sd[i] = std::max(std::sqrt(sd[i] / static_cast<double>(n)), 1e-6);
-  float xmin[og::MLP_NF], xmax[og::MLP_NF];
-  for (int i = 0; i < F; ++i) { xmin[i] = INFINITY; xmax[i] = -INFINITY; }
-  for (int64_t k = 0; k < n; ++k) {
-    y[k] = static_cast<float>(std::log10(std::max(static_cast<double>(labels[k]), 1e-12)));
-    for (int i = 0; i < F; ++i) {
-      const float v = static_cast<float>((features[k * F + i] - mu[i]) / sd[i]);
-      X[k * F + i] = v;
-      xmin[i] = std::min(xmin[i], v);
-      xmax[i] = std::max(xmax[i], v);
-    }
-  }
   // He-uniform initialisation from a counter-based generator
   std::vector<float> w(og::MLP_NPARAM, 0.f);
   uint64_t rs = seed;
@@ -292,22 +272,29 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int B = static_cast<int>(std::min<int64_t>(batch, n));
   const size_t np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
+  const size_t nx = static_cast<size_t>(F) * n;
   Scratch S;
-  int rc = S.buf.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(X.size()) + Scratch::room(n) +
-                         Scratch::room(np) + Scratch::room(1));
+  int rc = S.buf.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + 2 * Scratch::room(n) +
+                         Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) + Scratch::room(1));
   if (rc) return rc;
-  float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(X.size()),
-        *dy = S.take(n), *part = S.take(np), *dl = S.take(1);
-  CUDA_TRY(cudaMemcpyAsync(dx, X.data(), 4 * X.size(), cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(dy, y.data(), 4 * n, cudaMemcpyHostToDevice, st));
+  float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(nx),
+        *dlab = S.take(n), *dy = S.take(n), *part = S.take(np), *dstd = S.take(og::MLP_STD_FLOATS), *drec = S.take(4 * F),
+        *dl = S.take(1);
+  CUDA_TRY(cudaMemcpyAsync(dx, features, 4 * nx, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dlab, labels, 4 * n, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dw, w.data(), 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemsetAsync(dm, 0, 2 * Scratch::room(og::MLP_NPARAM), st));  // dm and dv follow each other
+  {  // targets: log10 of the error label; inputs standardised per feature
+    const cudaError_t e = og::mlp_standardise(dx, dlab, n, dstd, dy, drec, st);
+    if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "standardisation failed: %s", cudaGetErrorString(e));
+  }
   for (int k = 1; k <= steps; ++k) {
     cudaError_t e = og::mlp_grad(dw, dx, dy, static_cast<int>(n), B, k, seed, false, part, st);
     if (e == cudaSuccess) e = og::mlp_adam(part, B, dw, dm, dv, static_cast<float>(lr), k, dl, st);
     if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "training kernels failed: %s", cudaGetErrorString(e));
   }
-  float l = 0;
+  float l = 0, stats[4 * og::MLP_NF];
+  CUDA_TRY(cudaMemcpyAsync(stats, drec, sizeof stats, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(w.data(), dw, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(&l, dl, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
@@ -318,10 +305,10 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   // differ in the last bits).
   constexpr float kRangeMargin = 1e-3f;
   for (int i = 0; i < F; ++i) {
-    record[i] = static_cast<float>(mu[i]);
-    record[12 + i] = static_cast<float>(sd[i]);
-    record[24 + i] = xmin[i] - kRangeMargin;
-    record[36 + i] = xmax[i] + kRangeMargin;
+    record[i] = stats[i];
+    record[12 + i] = stats[12 + i];
+    record[24 + i] = stats[24 + i] - kRangeMargin;
+    record[36 + i] = stats[36 + i] + kRangeMargin;
   }
   std::memcpy(record + 48, w.data(), 4 * og::MLP_NPARAM);
   if (final_loss) *final_loss = l;

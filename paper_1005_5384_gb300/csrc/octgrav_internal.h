@@ -157,6 +157,12 @@ struct MlpSampleArgs {
 };
 cudaError_t mlp_sample_features(const MlpSampleArgs& a, cudaStream_t st);
 cudaError_t mlp_sample_labels(const MlpSampleArgs& a, cudaStream_t st);
+// Standardise the n samples' features in place (12 floats each), write the
+// targets y = log10(max(label, 1e-12)) and record[0..48): mean, deviation and
+// range of the standardised values per feature. scratch: MLP_STD_FLOATS
+// floats, 8-byte aligned.
+cudaError_t mlp_standardise(float* feat, const float* label, int64_t n, float* scratch, float* y, float* record,
+                            cudaStream_t st);
 // A training step's gradient in two launches. mlp_grad writes the shares of
 // mlp_blocks(B) blocks to part (MLP_PART floats each); use_all: the B samples
 // are X[0..B) instead of B counter-based draws. mlp_gradient adds them into

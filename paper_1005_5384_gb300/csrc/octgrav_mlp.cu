@@ -91,6 +91,102 @@ __global__ void label_kernel(MlpSampleArgs a) {
 
 // ---------------------------------------------------------------- training
 
+// Standardisation of the inputs: mean and deviation per feature in FP64, then
+// x = (f - mean) / deviation, the range of x, and the targets log10(label).
+// Blocks of 16 rows x 12 features take rows in strides of the grid and leave
+// partial results that every block of the next pass adds in the same order.
+// Three passes over the features (3 MB for 65,536 samples, from L2) and a few
+// FP64 operations per value, where the host's loops took 2.4 ms of a call:
+// 100 training steps on 65,536 samples 4.13 ms with them, 2.28 ms with these.
+constexpr int SR = 16;             // rows of a block
+constexpr int ST = SR * MLP_NF;    // its threads
+constexpr int SB = 152;            // blocks
+
+struct StdPart {  // one block's partial results
+  double sum[MLP_NF], sq[MLP_NF];
+  float lo[MLP_NF], hi[MLP_NF];
+};
+static_assert(SB * sizeof(StdPart) <= 4 * MLP_STD_FLOATS, "partial results fit their place");
+
+// Sums of the features (SQ: of their squared distances from the mean).
+template <bool SQ>
+__global__ void __launch_bounds__(ST) std_sum_kernel(const float* __restrict__ feat, int64_t n, StdPart* part) {
+  __shared__ double red[SR][MLP_NF];
+  const int f = threadIdx.x % MLP_NF, r = threadIdx.x / MLP_NF;
+  double mean = 0;
+  if (SQ) {
+#pragma unroll 8
+    for (int b = 0; b < static_cast<int>(gridDim.x); ++b) mean += part[b].sum[f];
+    mean /= static_cast<double>(n);
+  }
+  double s = 0;
+  for (int64_t k = static_cast<int64_t>(blockIdx.x) * SR + r; k < n; k += static_cast<int64_t>(gridDim.x) * SR) {
+    const double d = static_cast<double>(feat[k * MLP_NF + f]) - mean;
+    s += SQ ? d * d : d;
+  }
+  red[r][f] = s;
+  __syncthreads();
+  if (r == 0) {
+    for (int q = 1; q < SR; ++q) s += red[q][f];
+    (SQ ? part[blockIdx.x].sq : part[blockIdx.x].sum)[f] = s;
+  }
+}
+
+// feat becomes x in place; record[0..24) = mean, deviation (block 0).
+__global__ void __launch_bounds__(ST) std_apply_kernel(float* feat, const float* __restrict__ label, int64_t n,
+                                                        StdPart* part, float* __restrict__ y, float* __restrict__ record) {
+  __shared__ float lo[SR][MLP_NF], hi[SR][MLP_NF];
+  const int f = threadIdx.x % MLP_NF, r = threadIdx.x / MLP_NF;
+  double mean = 0, sq = 0;
+#pragma unroll 8
+  for (int b = 0; b < static_cast<int>(gridDim.x); ++b) {
+    mean += part[b].sum[f];
+    sq += part[b].sq[f];
+  }
+  mean /= static_cast<double>(n);
+  const double dev = fmax(sqrt(sq / static_cast<double>(n)), 1e-6);
+  if (blockIdx.x == 0 && r == 0) {
+    record[f] = static_cast<float>(mean);
+    record[MLP_NF + f] = static_cast<float>(dev);
+  }
+  float l = INFINITY, h = -INFINITY;
+  for (int64_t k = static_cast<int64_t>(blockIdx.x) * SR + r; k < n; k += static_cast<int64_t>(gridDim.x) * SR) {
+    const float x = static_cast<float>((static_cast<double>(feat[k * MLP_NF + f]) - mean) / dev);
+    feat[k * MLP_NF + f] = x;
+    l = x < l ? x : l;
+    h = h < x ? x : h;
+    if (f == 0) {
+      const double v = label[k];
+      y[k] = static_cast<float>(log10(v < 1e-12 ? 1e-12 : v));
+    }
+  }
+  lo[r][f] = l;
+  hi[r][f] = h;
+  __syncthreads();
+  if (r == 0) {
+    for (int q = 1; q < SR; ++q) {
+      l = lo[q][f] < l ? lo[q][f] : l;
+      h = h < hi[q][f] ? hi[q][f] : h;
+    }
+    part[blockIdx.x].lo[f] = l;
+    part[blockIdx.x].hi[f] = h;
+  }
+}
+
+// record[24..48) = range of x per feature.
+__global__ void std_range_kernel(const StdPart* __restrict__ part, int blocks, float* __restrict__ record) {
+  const int f = threadIdx.x;
+  if (f >= MLP_NF) return;
+  float l = INFINITY, h = -INFINITY;
+#pragma unroll 8
+  for (int b = 0; b < blocks; ++b) {
+    l = part[b].lo[f] < l ? part[b].lo[f] : l;
+    h = h < part[b].hi[f] ? part[b].hi[f] : h;
+  }
+  record[2 * MLP_NF + f] = l;
+  record[3 * MLP_NF + f] = h;
+}
+
 // Counter-based uniform index in [0, n): splitmix64 of (seed, step, b).
 __device__ __forceinline__ int sample_index(uint64_t seed, int step, int b, int n) {
   uint64_t z = seed + 0x9E3779B97F4A7C15ull * (static_cast<uint64_t>(step) * 1000003ull + b + 1);
@@ -356,6 +452,18 @@ cudaError_t mlp_sample_labels(const MlpSampleArgs& a, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
   const long long warps = static_cast<long long>(a.n) * a.chunks;
   label_kernel<<<static_cast<unsigned>((warps * 32 + 255) / 256), 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t mlp_standardise(float* feat, const float* label, int64_t n, float* scratch, float* y, float* record,
+                            cudaStream_t st) {
+  const int64_t rows = (n + SR - 1) / SR;
+  const int blocks = rows < SB ? static_cast<int>(rows) : SB;
+  StdPart* part = reinterpret_cast<StdPart*>(scratch);
+  std_sum_kernel<false><<<blocks, ST, 0, st>>>(feat, n, part);
+  std_sum_kernel<true><<<blocks, ST, 0, st>>>(feat, n, part);
+  std_apply_kernel<<<blocks, ST, 0, st>>>(feat, label, n, part, y, record);
+  std_range_kernel<<<1, 32, 0, st>>>(part, blocks, record);
   return cudaGetLastError();
 }
 

@@ -15,6 +15,8 @@ constexpr int MLP_NPARAM = MLP_NH * MLP_NF + MLP_NH + MLP_NH * MLP_NH + MLP_NH +
 // One block's share of a gradient: the parameters, the loss, padding.
 constexpr int MLP_PART = 5088;
 static_assert(MLP_PART > MLP_NPARAM && MLP_PART % 32 == 0, "shares hold every parameter and the loss");
+// Floats of the standardisation's partial results (152 blocks).
+constexpr int MLP_STD_FLOATS = 152 * 6 * MLP_NF;
 // Criterion record (floats): mu[12], sigma[12], xmin[12], xmax[12], params[5057].
 constexpr int MLP_RECORD = 4 * MLP_NF + MLP_NPARAM;  // 5105
 
