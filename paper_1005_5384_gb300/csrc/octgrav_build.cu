@@ -25,9 +25,13 @@ constexpr int MAXD = 21;          // depth limit (Morton keys of 3 x 21 bits)
 constexpr int NLEV = MAXD + 1;    // levels 0..21
 constexpr int TB = 256;           // threads per block
 constexpr int IPT = 16;           // elements per thread in the chunked kernels
-constexpr int TILE = TB * IPT;    // particles per chunk (sort, box, keys)
-constexpr int GL = 4096;          // blocks of the level kernels
-constexpr int GLT = 1024;         // threads of the level scan (GL / GLT entries each)
+constexpr int TILE = TB * IPT;    // particles per chunk (sort)
+constexpr int SUB = 8;            // blocks per chunk in the key pass
+constexpr int BSUB = 2;           // blocks per chunk in the box pass
+constexpr int LT = 512;           // threads of the level kernel (16 warps) ...
+constexpr int LBMAX = 1024;       // ... and the most blocks it may have
+constexpr int NT = 128;           // threads of the node kernel
+constexpr long long WAIT_LIMIT = 1ll << 31;  // cycles (~1 s) before a grid barrier gives up
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LBINS = 32;  // leaf size bins of the moment pass (32 = "32 or more")
 constexpr int IBINS = 256; // work-item size bins of the default processing order (item_max <= 256)
@@ -41,10 +45,15 @@ struct Chunk {  // TILE particles (or fewer) of one system
   int nbs, pad0, pad1, pad2;  // chunks of the system
 };
 
+// misc[] slots (int), zeroed before a build: counts, status bits, arrivals at
+// the grid barriers of the level and the node kernel, nodes per level
+enum { M_NGROUPS = 0, M_NITEMS, M_NLEAVES, M_MAXGROUP, M_STATUS, M_BAR_LEVELS, M_BAR_NODES, M_NODES };
+constexpr int MISC = M_NODES + NLEV;
+
 // Scratch layout (byte offsets into one allocation).
 struct Layout {
   size_t keyA, keyB, valA, valB, cnt, dtot, part, sg, xs, ms, chunks, offs, chunk0;
-  size_t ckey, cpar, cpf, cpc, csys, cfc, cnc, spl, lpre, bsum, lvl, misc;
+  size_t ckey, cpar, cpf, cpc, csys, cfc, cnc, spl, lpre, nlist, bsum, lvl, misc;
   size_t sstart, send, lofs, ni, lorder, lhist, ihist, gmark, gidx, gcell, nitem, ioff, sblk;
   size_t total;
 };
@@ -65,7 +74,7 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   L.valB = take(4 * n);
   L.cnt = take(4 * 256 * n_chunks);
   L.dtot = take(4 * 256 * static_cast<size_t>(n_sys));
-  L.part = take(8 * 6 * n_chunks);
+  L.part = take(8 * 6 * BSUB * n_chunks);
   L.sg = take(sizeof(SysGeo) * n_sys);
   L.xs = take(24 * n);
   L.ms = take(8 * n);
@@ -81,9 +90,10 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   L.cnc = take(4 * cap);
   L.spl = take(4 * 9 * std::min<int64_t>(n, cap));
   L.lpre = take(4 * std::min<int64_t>(n, cap));
-  L.bsum = take(4 * GL);
+  L.nlist = take(4 * cap);
+  L.bsum = take(4 * LBMAX);
   L.lvl = take(4 * (NLEV + 2));
-  L.misc = take(4 * 16);
+  L.misc = take(4 * MISC);
   L.sstart = take(4 * static_cast<size_t>(n_sys) * NLEV);
   L.send = take(4 * static_cast<size_t>(n_sys) * NLEV);
   L.lofs = take(4 * static_cast<size_t>(n_sys) * NLEV);
@@ -101,8 +111,6 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   return L;
 }
 
-// misc[] slots (int)
-enum { M_NGROUPS = 0, M_NITEMS = 1, M_NLEAVES = 2, M_MAXGROUP = 3, M_STATUS = 4 };
 
 template <class T>
 T* at(void* base, size_t off) {
@@ -163,17 +171,46 @@ __device__ int block_scan_excl(int v, int* total) {
   return before + x - v;
 }
 
+// Barrier over all blocks of a cooperative launch: every block adds one to
+// *bar and waits until it reaches `target` (a multiple of the grid size that
+// grows from barrier to barrier). Writes before it are visible to every block
+// after it. False when the wait ran out (all blocks of a cooperative launch
+// are resident, so that would be a lost block); the kernels then stop and
+// leave GPU_BUILD_STUCK in the status word.
+__device__ bool grid_barrier(int* bar, int target, int* status) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int good = 1, v;
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(bar) : "memory");
+    const long long t0 = clock64();
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target) break;
+      if (clock64() - t0 > WAIT_LIMIT) {
+        atomicOr(status, GPU_BUILD_STUCK);
+        good = 0;
+        break;
+      }
+    }
+    ok = good;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
 // ---------------------------------------------------------------- keys and sort
 
-// Bounding box per chunk; flags non-finite coordinates or masses and
+// Bounding box per half of a chunk; flags non-finite coordinates or masses and
 // negative masses.
 __global__ void __launch_bounds__(TB) k_bbox(const double* __restrict__ pos, const double* __restrict__ mass,
                                              const Chunk* __restrict__ ch, double* __restrict__ part,
                                              int* __restrict__ misc) {
-  const Chunk c = ch[blockIdx.x];
+  const Chunk c = ch[blockIdx.x / BSUB];
   double mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
   bool bad = false;
-  for (int k = threadIdx.x; k < c.count; k += TB) {
+  const int k0 = static_cast<int>(blockIdx.x % BSUB) * (TILE / BSUB), k1 = min(c.count, k0 + TILE / BSUB);
+  for (int k = k0 + threadIdx.x; k < k1; k += TB) {
     const int64_t i = c.first + k;
     for (int d = 0; d < 3; ++d) {
       const double v = pos[3 * i + d];
@@ -210,7 +247,7 @@ __global__ void __launch_bounds__(TB) k_root(const double* __restrict__ part, co
                                              SysGeo* __restrict__ sg) {
   const int s = blockIdx.x;
   double mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (int b = chunk0[s] + threadIdx.x; b < chunk0[s + 1]; b += TB)
+  for (int b = BSUB * chunk0[s] + threadIdx.x; b < BSUB * chunk0[s + 1]; b += TB)
     for (int d = 0; d < 3; ++d) {
       mn[d] = lesser(mn[d], part[6 * b + d]);
       mx[d] = greater(mx[d], part[6 * b + 3 + d]);
@@ -251,26 +288,34 @@ __global__ void __launch_bounds__(TB) k_root(const double* __restrict__ part, co
 __global__ void __launch_bounds__(TB) k_morton(const double* __restrict__ pos, const Chunk* __restrict__ ch,
                                                const SysGeo* __restrict__ sg, uint64_t* __restrict__ key,
                                                uint32_t* __restrict__ val) {
-  const Chunk c = ch[blockIdx.x];
+  const Chunk c = ch[blockIdx.x / SUB];
   const SysGeo g = sg[c.sys];
   const double* lo = g.lo;
   const double side = g.side;
   const double scale = 2097152.0;  // 2^21
   const uint64_t qmax = (1ull << MAXD) - 1;
-  for (int k = threadIdx.x; k < c.count; k += TB) {
+  const int k0 = static_cast<int>(blockIdx.x % SUB) * (TILE / SUB), k1 = min(c.count, k0 + TILE / SUB);
+  for (int k = k0 + threadIdx.x; k < k1; k += TB) {
     const int64_t i = c.first + k;
     uint64_t q[3];
     for (int d = 0; d < 3; ++d) {
       // The quantised coordinate is floor(fl(fl(x - lo) / side) * 2^21) =
       // floor(fl(fl(x - lo) * 2^21 / side)). a = fl(x - lo) * g.rscale is
-      // within 4 ulp (< 2^-29 for a <= 2^21) of fl(fl(x - lo) * 2^21 / side),
-      // so whenever no integer lies within 2^-28 of a the floors agree; the
-      // rare remaining cases take the division.
+      // within 4 ulp (< 2^-29 for a <= 2^21) of fl(fl(x - lo) * 2^21 / side).
+      // Adding 1.5 * 2^22 rounds a to a multiple of 2^-30 (half a unit more)
+      // and leaves it in the low mantissa bits, so whenever its fraction is 4
+      // units or more from an integer the floors agree; the rare remaining
+      // cases take the division. Three FP64 operations per coordinate, the
+      // rest on the integer pipe: FP64 issue bounds this pass (72 us at 1M
+      // particles with floor() of both ends of the interval, 22 us now).
       const double dx = pos[3 * i + d] - lo[d];
       const double a = dx * g.rscale;
-      double v = floor(a - 0x1p-28);
-      if (v != floor(a + 0x1p-28)) v = floor((dx / side) * scale);
-      q[d] = v <= 0 ? 0 : (v >= static_cast<double>(qmax) ? qmax : static_cast<uint64_t>(v));
+      const double magic = 6291456.0;
+      const long long u = __double_as_longlong(a + magic) - __double_as_longlong(magic);
+      const int frac = static_cast<int>(u) & ((1 << 30) - 1);
+      long long v = u >> 30;
+      if (frac < 4 || frac > (1 << 30) - 5) v = static_cast<long long>(floor((dx / side) * scale));
+      q[d] = v <= 0 ? 0 : (v >= static_cast<long long>(qmax) ? qmax : static_cast<uint64_t>(v));
     }
     key[i] = spread21(q[0]) | (spread21(q[1]) << 1) | (spread21(q[2]) << 2);
     val[i] = static_cast<uint32_t>(i);
@@ -453,186 +498,227 @@ __global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, in
   if (s <= NLEV + 1) lvl[s] = s == 0 ? 0 : n_sys;
 }
 
-// Block b of GL takes a contiguous range of the level's cells.
-__device__ __forceinline__ void level_range(const int* lvl, int L, int& lb, int& le, int& c0, int& c1) {
-  lb = lvl[L];
-  le = lvl[L + 1];
-  const int nl = le - lb;
-  const int chunk = (nl + GL - 1) / GL;
-  c0 = min(le, lb + static_cast<int>(blockIdx.x) * chunk);
-  c1 = min(le, c0 + chunk);
-}
-
-// First position p in [a, b) whose child octant at depth D is >= o (b if
-// none); octants ascend inside a cell. The warp probes 32 evenly spaced
-// positions per round (all lanes get the same answer).
-__device__ int warp_partition(const uint64_t* __restrict__ code, int a, int b, int D, int o, int lane) {
-  // invariant: the answer lies in [a, b], and b is the end or a known hit
-  while (b - a > 32) {
-    const int64_t span = b - a;
-    const int p = a + static_cast<int>((lane + 1) * span / 33);
-    const unsigned m = __ballot_sync(FULL, octant_at(code[p], D) >= o);
-    const int k = m ? __ffs(m) - 1 : 32;
-    const int lo = k == 0 ? a : a + static_cast<int>(k * span / 33) + 1;
-    const int hi = k == 32 ? b : a + static_cast<int>((k + 1) * span / 33);
-    a = lo;
-    b = hi;
-  }
-  const int p = a + lane;
-  const unsigned m = __ballot_sync(FULL, p < b && octant_at(code[p], D) >= o);
-  return m ? a + __ffs(m) - 1 : b;
-}
-
 // Split points of a cell holding particles [f, f + cnt): sp[o] = the first
-// position whose child octant at depth D is >= o, sp[0] = f, sp[8] = f + cnt.
-// One warp; a cell of at most 32 particles takes a single round of loads.
-// Every lane returns the same sp.
+// position whose child octant at depth D is >= o, sp[0] = f, sp[8] = f + cnt
+// (octants ascend inside a cell). One warp; every lane returns the same sp.
+// The seven boundaries are searched together: a round probes 32 evenly spaced
+// positions of each one's interval with seven independent loads per lane, so a
+// cell of a million particles takes four rounds of load latency and one of at
+// most 32 particles a single load (one boundary after the other took seven
+// times as many rounds).
 __device__ void warp_split(const uint64_t* __restrict__ code, int f, int cnt, int D, int lane, int* sp) {
   sp[0] = f;
   sp[8] = f + cnt;
   if (cnt <= 32) {  // one probe per particle
     const int oc = lane < cnt ? octant_at(code[f + lane], D) : 8;
+#pragma unroll
     for (int o = 1; o < 8; ++o) {
       const unsigned m = __ballot_sync(FULL, oc >= o);
       sp[o] = m ? f + __ffs(m) - 1 : f + cnt;
     }
     return;
   }
-  for (int o = 1; o < 8; ++o) sp[o] = warp_partition(code, sp[o - 1], f + cnt, D, o, lane);
+  // invariant: boundary o lies in [a[o], b[o]], and b[o] is the end or a known hit
+  int a[8], b[8], span = cnt;
+#pragma unroll
+  for (int o = 1; o < 8; ++o) {
+    a[o] = f;
+    b[o] = f + cnt;
+  }
+  while (span > 32) {
+    int oc[8];
+#pragma unroll
+    for (int o = 1; o < 8; ++o) {
+      const int64_t w = b[o] - a[o];
+      const int p = a[o] + static_cast<int>((lane + 1) * w / 33);
+      oc[o] = p < b[o] ? octant_at(code[p], D) : 8;
+    }
+    span = 0;
+#pragma unroll
+    for (int o = 1; o < 8; ++o) {
+      const int64_t w = b[o] - a[o];
+      const unsigned m = __ballot_sync(FULL, oc[o] >= o);
+      const int k = m ? __ffs(m) - 1 : 32;
+      const int lo = k == 0 ? a[o] : min(b[o], a[o] + static_cast<int>(k * w / 33) + 1);
+      const int hi = k == 32 ? b[o] : min(b[o], a[o] + static_cast<int>((k + 1) * w / 33));
+      a[o] = lo;
+      b[o] = hi;
+      span = max(span, hi - lo);
+    }
+  }
+  int oc[8];
+#pragma unroll
+  for (int o = 1; o < 8; ++o) oc[o] = a[o] + lane < b[o] ? octant_at(code[a[o] + lane], D) : 8;
+#pragma unroll
+  for (int o = 1; o < 8; ++o) {
+    const unsigned m = __ballot_sync(FULL, oc[o] >= o && a[o] + lane < b[o]);
+    sp[o] = m ? a[o] + __ffs(m) - 1 : b[o];
+  }
 }
 
-// Split points of every cell of level L (the host's partition points; one
-// warp per cell), and the block-local exclusive prefix of the children counts.
-__global__ void __launch_bounds__(TB) k_split(int L, const uint64_t* __restrict__ code, Cells C, int n_leaf,
-                                              const int* __restrict__ lvl, int* __restrict__ spl,
-                                              int* __restrict__ lpre, int* __restrict__ bsum) {
-  constexpr int W = TB / 32;
-  __shared__ int sn[W];
-  __shared__ int carry;
-  int lb, le, c0, c1;
-  level_range(lvl, L, lb, le, c0, c1);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x == 0) carry = 0;
-  for (int base = c0; base < c1; base += W) {
-    const int c = base + w;
-    int nch = 0;
-    if (c < c1) {  // warp-uniform
-      const int f = C.pf[c], cnt = C.pc[c];
-      int sp[9];
-      if (cnt <= n_leaf || L >= MAXD) {
-        for (int o = 0; o < 9; ++o) sp[o] = f;
-      } else {
-        warp_split(code, f, cnt, L + 1, lane, sp);
-        for (int o = 0; o < 8; ++o) nch += sp[o + 1] > sp[o];
+// After a barrier that ran out: a tree without cells, which the rest of the
+// build passes through without touching anything (the host reports the status).
+__device__ void no_cells(int* lvl) {
+  if (threadIdx.x <= NLEV + 1) lvl[threadIdx.x] = 0;
+}
+
+// All levels of the tree in one cooperative launch. Per level: every block
+// takes a contiguous range of the level's cells and finds the split points of
+// those that hold more than n_leaf particles (a warp per cell); after a
+// barrier every block adds the blocks' children counts up to its own, which
+// places its children in the host's breadth-first order, and writes them;
+// after a second barrier they are the next level. The loop ends with the first
+// level without children. The cells that were split are also listed per level
+// (nlist, M_NODES) for the moment pass.
+//
+// Latency bounds it: a level is a few dependent rounds of loads and two
+// barriers (5 us; the levels with tens of thousands of cells up to 20 us, where
+// a warp's cells are all split). As three launches per level for 21 levels (4096
+// blocks each, most of them empty) the levels took 425 us at 1M particles and
+// 270 us at 5000 (sum of the launches); 327 us and 84 us now.
+__global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ code, Cells C, int n_leaf, int* lvl,
+                                                  int* spl, int* lpre, int* nlist, int* bsum, int cap, int* misc) {
+  constexpr int W = LT / 32;
+  __shared__ int wsum[W];
+  __shared__ int sh_before, sh_total;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grid = gridDim.x;
+  const unsigned lt = (1u << lane) - 1u;
+  int lb = lvl[0], le = lvl[1], bars = 0;
+  for (int L = 0; L < MAXD; ++L) {
+    const int nl = le - lb;
+    // cells per warp; block b's warps take consecutive ranges of its range
+    const int per = (nl + grid * W - 1) / (grid * W);
+    const int b0 = lb + static_cast<int>(min(static_cast<int64_t>(blockIdx.x) * per * W, static_cast<int64_t>(nl)));
+    const int c0 = min(le, b0 + w * per), c1 = min(le, c0 + per);
+    int mine = 0;  // children of this warp's cells
+    for (int base = c0; base < c1; base += 32) {
+      const int c = base + lane;
+      const int cnt = c < c1 ? C.pc[c] : 0;
+      const int f = c < c1 ? C.pf[c] : 0;
+      unsigned todo = __ballot_sync(FULL, cnt > n_leaf);
+      const unsigned nodes = todo;
+      int nch = 0;
+      while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        int sp[9];
+        warp_split(code, __shfl_sync(FULL, f, k), __shfl_sync(FULL, cnt, k), L + 1, lane, sp);
+        int n = 0, own = sp[0];
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+          n += sp[o + 1] > sp[o];
+          own = lane == o + 1 ? sp[o + 1] : own;
+        }
+        if (lane < 9) spl[9 * static_cast<int64_t>(base + k - lb) + lane] = own;
+        if (lane == k) nch = n;
       }
+      int x = nch;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, d);
+        if (lane >= d) x += y;
+      }
+      int at = 0;
+      if (lane == 0 && nodes) at = atomicAdd(&misc[M_NODES + L], __popc(nodes));
+      at = __shfl_sync(FULL, at, 0);
+      if (nch) {
+        C.nc[c] = nch;
+        lpre[c - lb] = mine + x - nch;
+        nlist[lb + at + __popc(nodes & lt)] = c;
+      }
+      mine += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) wsum[w] = mine;
+    __syncthreads();
+    if (w == 0) {  // children before each warp, and the block's
+      const int v = lane < W ? wsum[lane] : 0;
+      int x = v;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, d);
+        if (lane >= d) x += y;
+      }
+      if (lane < W) wsum[lane] = x - v;
+      if (lane == 31) bsum[blockIdx.x] = x;
+    }
+    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS])) {
+      no_cells(lvl);
+      return;
+    }
+    {  // children of the blocks before this one, and of all
+      int before = 0, all = 0;
+      for (int b = threadIdx.x; b < grid; b += LT) {
+        const int v = __ldcg(&bsum[b]);
+        all += v;
+        before += b < static_cast<int>(blockIdx.x) ? v : 0;
+      }
+#pragma unroll
+      for (int d = 16; d; d >>= 1) {
+        before += __shfl_xor_sync(FULL, before, d);
+        all += __shfl_xor_sync(FULL, all, d);
+      }
+      if (threadIdx.x == 0) sh_before = sh_total = 0;
+      __syncthreads();
       if (lane == 0) {
-        int* d = &spl[9 * static_cast<int64_t>(c - lb)];
-        for (int o = 0; o < 9; ++o) d[o] = sp[o];
+        atomicAdd(&sh_before, before);
+        atomicAdd(&sh_total, all);
+      }
+      __syncthreads();
+    }
+    const int total = sh_total;
+    const int64_t next = static_cast<int64_t>(le) + total;
+    if (total == 0 || next > cap) {  // the same in every block
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        for (int k = L + 2; k <= NLEV; ++k) lvl[k] = le;
+        if (next > cap) {
+          atomicOr(&misc[M_STATUS], GPU_BUILD_OVERFLOW);
+          misc[M_NODES + L] = 0;
+        }
+      }
+      if (next > cap)  // the unsplit cells are no nodes
+        for (int c = c0 + lane; c < c1; c += 32) C.nc[c] = 0;
+      return;
+    }
+    // emit: of the cells that were split four at a time, lane (k, o) writing
+    // child o of the k-th
+    const int first = le + sh_before + wsum[w];
+    const int o = lane & 7, sub = lane >> 3;
+    for (int base = c0; base < c1; base += 32) {
+      unsigned nodes = __ballot_sync(FULL, base + lane < c1 && C.nc[base + lane] > 0);
+      while (nodes) {
+        int c = -1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (nodes && sub == k) c = base + __ffs(nodes) - 1;
+          nodes &= nodes - 1;
+        }
+        int f = 0, e = 0;
+        if (c >= 0) {
+          f = spl[9 * static_cast<int64_t>(c - lb) + o];
+          e = spl[9 * static_cast<int64_t>(c - lb) + o + 1];
+        }
+        const unsigned m = __ballot_sync(FULL, e > f) >> (8 * sub) & 255u;
+        if (e > f) {
+          const int k0 = first + lpre[c - lb], k = k0 + __popc(m & ((1u << o) - 1u));
+          if ((m & ((1u << o) - 1u)) == 0) C.fc[c] = k0;
+          C.key[k] = (C.key[c] << 3) | static_cast<uint64_t>(o);
+          C.par[k] = c;
+          C.pf[k] = f;
+          C.pc[k] = e - f;
+          C.sys[k] = C.sys[c];
+          C.fc[k] = -1;
+          C.nc[k] = 0;
+        }
       }
     }
-    if (lane == 0) sn[w] = nch;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int run = carry;
-      for (int k = 0; k < W && base + k < c1; ++k) {
-        lpre[base + k - lb] = run;
-        run += sn[k];
-      }
-      carry = run;
+    if (blockIdx.x == 0 && threadIdx.x == 0) lvl[L + 2] = static_cast<int>(next);
+    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS])) {
+      no_cells(lvl);
+      return;
     }
-    __syncthreads();
+    lb = le;
+    le = static_cast<int>(next);
   }
-  if (threadIdx.x == 0) bsum[blockIdx.x] = carry;
-}
-
-// Offsets of the blocks' children and the end of level L + 1; a level that
-// does not fit the cell capacity stops the build (status overflow).
-__global__ void __launch_bounds__(GLT) k_scan_level(int L, int* __restrict__ bsum, int* __restrict__ lvl, int cap,
-                                                    int* __restrict__ misc) {
-  constexpr int PER = GL / GLT;
-  __shared__ int ws[32];
-  int e[PER], v = 0;
-#pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    e[k] = bsum[PER * threadIdx.x + k];
-    v += e[k];
-  }
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = v;
-  for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(FULL, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int t = ws[lane];
-    for (int d = 1; d < 32; d <<= 1) {
-      const int y = __shfl_up_sync(FULL, t, d);
-      if (lane >= d) t += y;
-    }
-    ws[lane] = t;
-  }
-  __syncthreads();
-  int run = (w ? ws[w - 1] : 0) + x - v;
-#pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    bsum[PER * threadIdx.x + k] = run;
-    run += e[k];
-  }
-  if (threadIdx.x == 0) {
-    const int le = lvl[L + 1];
-    const int64_t next = static_cast<int64_t>(le) + ws[31];
-    if (next > cap) {
-      atomicOr(&misc[M_STATUS], GPU_BUILD_OVERFLOW);
-      lvl[L + 2] = le;
-    } else {
-      lvl[L + 2] = static_cast<int>(next);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(TB) k_emit(int L, Cells C, const int* __restrict__ lvl, const int* __restrict__ spl,
-                                             const int* __restrict__ lpre, const int* __restrict__ boff,
-                                             const int* __restrict__ misc) {
-  if (misc[M_STATUS] & GPU_BUILD_OVERFLOW) return;
-  int lb, le, c0, c1;
-  level_range(lvl, L, lb, le, c0, c1);
-  for (int c = c0 + threadIdx.x; c < c1; c += TB) {
-    const int* sp = &spl[9 * static_cast<int64_t>(c - lb)];
-    int nch = 0;
-    for (int o = 0; o < 8; ++o) nch += sp[o + 1] > sp[o];
-    if (!nch) continue;
-    int w = le + boff[blockIdx.x] + lpre[c - lb];
-    C.fc[c] = w;
-    C.nc[c] = nch;
-    const uint64_t k = C.key[c];
-    const int s = C.sys[c];
-    for (int o = 0; o < 8; ++o) {
-      if (sp[o + 1] <= sp[o]) continue;
-      C.key[w] = (k << 3) | static_cast<uint64_t>(o);
-      C.par[w] = c;
-      C.pf[w] = sp[o];
-      C.pc[w] = sp[o + 1] - sp[o];
-      C.sys[w] = s;
-      C.fc[w] = -1;
-      C.nc[w] = 0;
-      ++w;
-    }
-  }
-}
-
-// After a level loop capped at max_level < MAXD: flag a cell of level
-// max_level that still needs splitting (the caller rebuilds without the cap),
-// and close the level table so that lvl[NLEV] is the cell count.
-__global__ void k_depth_check(int max_level, Cells C, int* __restrict__ lvl, int n_leaf, int* __restrict__ misc) {
-  const int lb = lvl[max_level], le = lvl[max_level + 1];
-  bool deeper = false;
-  for (int c = lb + blockIdx.x * blockDim.x + threadIdx.x; c < le; c += gridDim.x * blockDim.x)
-    deeper |= C.pc[c] > n_leaf;
-  if (__syncthreads_or(deeper) && threadIdx.x == 0) atomicOr(&misc[M_STATUS], GPU_BUILD_DEEPER);
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    for (int L = max_level + 2; L <= NLEV; ++L) lvl[L] = le;
 }
 
 // Level of cell c: the last L with lvl[L] <= c.
@@ -720,61 +806,45 @@ struct Props {  // final-order FP64 arrays and records
 
 __device__ __forceinline__ int final_index(const int* ni, int c) { return ni ? ni[c] : c; }
 
-// Tight box, boundary cube, mass, centre of mass and second moments of cell
-// c (a leaf from its particles, a node from its children with the
-// parallel-axis shift, in the host build's operation order), then its records.
-template <bool LEAF>
-__device__ __forceinline__ void cell_props(int c, Cells C, const int* __restrict__ ni, const double* __restrict__ xs,
-                                           const double* __restrict__ ms, const Props& P) {
-  const int j = final_index(ni, c);
-  double bn[3] = {INFINITY, INFINITY, INFINITY}, bx[3] = {-INFINITY, -INFINITY, -INFINITY};
-  double Mc = 0, sx = 0, sy = 0, sz = 0;
-  const int f = C.pf[c], cnt = C.pc[c], nch = LEAF ? 0 : C.nc[c];
-  const int jc = LEAF ? 0 : final_index(ni, C.fc[c]);  // children are contiguous in both orders
-  if (LEAF) {
-    for (int t = f; t < f + cnt; ++t) {
-      const double* xp = &xs[3 * static_cast<int64_t>(t)];
-      const double x0 = xp[0], x1 = xp[1], x2 = xp[2], m = ms[t];
-      bn[0] = lesser(bn[0], x0);
-      bn[1] = lesser(bn[1], x1);
-      bn[2] = lesser(bn[2], x2);
-      bx[0] = greater(bx[0], x0);
-      bx[1] = greater(bx[1], x1);
-      bx[2] = greater(bx[2], x2);
-      Mc += m;
-      sx = fma(m, x0, sx);
-      sy = fma(m, x1, sy);
-      sz = fma(m, x2, sz);
+// Tight box, boundary cube, mass, centre of mass and second moments of a
+// cell: sums over its members in the host build's operation order.
+struct Moments {
+  double bn[3], bx[3];  // tight box
+  double M, sx, sy, sz; // mass, mass-weighted positions
+  double cu[4], cm[3];  // boundary cube (centre, half side), centre of mass
+  double s6[6];         // second moments about cm
+
+  __device__ __forceinline__ void clear() {
+    for (int d = 0; d < 3; ++d) {
+      bn[d] = INFINITY;
+      bx[d] = -INFINITY;
     }
-  } else {
-    for (int q = jc; q < jc + nch; ++q) {
-      for (int d = 0; d < 3; ++d) {
-        bn[d] = lesser(bn[d], P.bmin[3 * q + d]);
-        bx[d] = greater(bx[d], P.bmax[3 * q + d]);
-      }
-      const double m = P.M[q];
-      Mc += m;
-      sx = fma(m, P.com[3 * q], sx);
-      sy = fma(m, P.com[3 * q + 1], sy);
-      sz = fma(m, P.com[3 * q + 2], sz);
+    M = sx = sy = sz = 0;
+    for (int k = 0; k < 6; ++k) s6[k] = 0;
+  }
+  __device__ __forceinline__ void add_mass(double m, double x, double y, double z) {
+    M += m;
+    sx = fma(m, x, sx);
+    sy = fma(m, y, sy);
+    sz = fma(m, z, sz);
+  }
+  __device__ __forceinline__ void centre() {
+    for (int d = 0; d < 3; ++d) cu[d] = (bn[d] + bx[d]) * 0.5;
+    double e = bx[0] - bn[0];
+    if (bx[1] - bn[1] > e) e = bx[1] - bn[1];
+    if (bx[2] - bn[2] > e) e = bx[2] - bn[2];
+    cu[3] = 0.5 * e;
+    if (M > 0) {
+      cm[0] = sx / M;
+      cm[1] = sy / M;
+      cm[2] = sz / M;
+    } else {
+      cm[0] = cu[0];
+      cm[1] = cu[1];
+      cm[2] = cu[2];
     }
   }
-  double cu[4], cm[3], s6[6] = {0, 0, 0, 0, 0, 0};
-  for (int d = 0; d < 3; ++d) cu[d] = (bn[d] + bx[d]) * 0.5;
-  double e = bx[0] - bn[0];
-  if (bx[1] - bn[1] > e) e = bx[1] - bn[1];
-  if (bx[2] - bn[2] > e) e = bx[2] - bn[2];
-  cu[3] = 0.5 * e;
-  if (Mc > 0) {
-    cm[0] = sx / Mc;
-    cm[1] = sy / Mc;
-    cm[2] = sz / Mc;
-  } else {
-    cm[0] = cu[0];
-    cm[1] = cu[1];
-    cm[2] = cu[2];
-  }
-  auto add_outer = [&](double wt, double y0, double y1, double y2) {
+  __device__ __forceinline__ void add_outer(double wt, double y0, double y1, double y2) {
     const double w0 = wt * y0, w1 = wt * y1, w2 = wt * y2;
     s6[0] = fma(w0, y0, s6[0]);
     s6[1] = fma(w1, y1, s6[1]);
@@ -782,45 +852,121 @@ __device__ __forceinline__ void cell_props(int c, Cells C, const int* __restrict
     s6[3] = fma(w0, y1, s6[3]);
     s6[4] = fma(w0, y2, s6[4]);
     s6[5] = fma(w1, y2, s6[5]);
-  };
-  if (LEAF) {
-    for (int t = f; t < f + cnt; ++t) {
-      const double* xp = &xs[3 * static_cast<int64_t>(t)];
-      add_outer(ms[t], xp[0] - cm[0], xp[1] - cm[1], xp[2] - cm[2]);
+  }
+  // FP64 arrays and the walk kernel's records of cell j (final order).
+  __device__ __forceinline__ void store(int j, uint64_t key, int f, int cnt, int2 link, const Props& P) const {
+    for (int d = 0; d < 3; ++d) {
+      P.bmin[3 * j + d] = bn[d];
+      P.bmax[3 * j + d] = bx[d];
+      P.com[3 * j + d] = cm[d];
     }
-  } else {
-    for (int q = jc; q < jc + nch; ++q) {
-      for (int k = 0; k < 6; ++k) s6[k] += P.S[6 * q + k];
-      add_outer(P.M[q], P.com[3 * q] - cm[0], P.com[3 * q + 1] - cm[1], P.com[3 * q + 2] - cm[2]);
+    for (int d = 0; d < 4; ++d) P.cube[4 * j + d] = cu[d];
+    for (int k = 0; k < 6; ++k) P.S[6 * j + k] = s6[k];
+    P.M[j] = M;
+    P.key[j] = key;
+    P.geo[j] = make_float4(static_cast<float>(cu[0]), static_cast<float>(cu[1]), static_cast<float>(cu[2]),
+                           static_cast<float>(cu[3]));
+    P.link[j] = link;
+    float chi[3], clo[3];
+    for (int d = 0; d < 3; ++d) {
+      chi[d] = static_cast<float>(cm[d]);
+      clo[d] = static_cast<float>(cm[d] - static_cast<double>(chi[d]));
     }
+    const double tr = s6[0] + s6[1] + s6[2];
+    P.mp[4 * j] = make_float4(chi[0], chi[1], chi[2], static_cast<float>(M));
+    P.mp[4 * j + 1] = make_float4(clo[0], clo[1], clo[2], static_cast<float>(cnt));
+    P.mp[4 * j + 2] = make_float4(static_cast<float>(3.0 * s6[0]), static_cast<float>(3.0 * s6[1]),
+                                  static_cast<float>(3.0 * s6[2]), static_cast<float>(3.0 * s6[3]));
+    P.mp[4 * j + 3] = make_float4(static_cast<float>(3.0 * s6[4]), static_cast<float>(3.0 * s6[5]),
+                                  static_cast<float>(1.5 * tr), static_cast<float>(0.5 * tr));
+    P.pcount[j] = cnt;
+    P.cfirst[j] = f;
   }
-  for (int d = 0; d < 3; ++d) {
-    P.bmin[3 * j + d] = bn[d];
-    P.bmax[3 * j + d] = bx[d];
-    P.com[3 * j + d] = cm[d];
+};
+
+// A leaf, from its particles.
+__device__ __forceinline__ void leaf_props(int c, Cells C, const int* __restrict__ ni, const double* __restrict__ xs,
+                                           const double* __restrict__ ms, const Props& P) {
+  Moments A;
+  A.clear();
+  const int f = C.pf[c], cnt = C.pc[c];
+  for (int t = f; t < f + cnt; ++t) {
+    const double* xp = &xs[3 * static_cast<int64_t>(t)];
+    for (int d = 0; d < 3; ++d) {
+      A.bn[d] = lesser(A.bn[d], xp[d]);
+      A.bx[d] = greater(A.bx[d], xp[d]);
+    }
+    A.add_mass(ms[t], xp[0], xp[1], xp[2]);
   }
-  for (int d = 0; d < 4; ++d) P.cube[4 * j + d] = cu[d];
-  for (int k = 0; k < 6; ++k) P.S[6 * j + k] = s6[k];
-  P.M[j] = Mc;
-  // records read by the walk kernel
-  P.key[j] = C.key[c];
-  P.geo[j] = make_float4(static_cast<float>(cu[0]), static_cast<float>(cu[1]), static_cast<float>(cu[2]),
-                         static_cast<float>(cu[3]));
-  P.link[j] = LEAF ? make_int2(f, -cnt) : make_int2(jc, nch);
-  float chi[3], clo[3];
-  for (int d = 0; d < 3; ++d) {
-    chi[d] = static_cast<float>(cm[d]);
-    clo[d] = static_cast<float>(cm[d] - static_cast<double>(chi[d]));
+  A.centre();
+  for (int t = f; t < f + cnt; ++t) {
+    const double* xp = &xs[3 * static_cast<int64_t>(t)];
+    A.add_outer(ms[t], xp[0] - A.cm[0], xp[1] - A.cm[1], xp[2] - A.cm[2]);
   }
-  const double tr = s6[0] + s6[1] + s6[2];
-  P.mp[4 * j] = make_float4(chi[0], chi[1], chi[2], static_cast<float>(Mc));
-  P.mp[4 * j + 1] = make_float4(clo[0], clo[1], clo[2], static_cast<float>(cnt));
-  P.mp[4 * j + 2] = make_float4(static_cast<float>(3.0 * s6[0]), static_cast<float>(3.0 * s6[1]),
-                                static_cast<float>(3.0 * s6[2]), static_cast<float>(3.0 * s6[3]));
-  P.mp[4 * j + 3] = make_float4(static_cast<float>(3.0 * s6[4]), static_cast<float>(3.0 * s6[5]),
-                                static_cast<float>(1.5 * tr), static_cast<float>(0.5 * tr));
-  P.pcount[j] = cnt;
-  P.cfirst[j] = f;
+  A.store(final_index(ni, c), C.key[c], f, cnt, make_int2(f, -cnt), P);
+}
+
+// A node, from its children (contiguous in both orders) with the
+// parallel-axis shift. The children's records are loaded ahead of the sums,
+// four at a time, so that a node waits for a few rounds of loads and not for
+// one per child and pass.
+__device__ __forceinline__ void node_props(int c, Cells C, const int* __restrict__ ni, const Props& P) {
+  Moments A;
+  A.clear();
+  const int nch = C.nc[c], jc = final_index(ni, C.fc[c]);
+  double m[8], x[8], y[8], z[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int j = jc + min(q, nch - 1);
+    m[q] = P.M[j];
+    x[q] = P.com[3 * j];
+    y[q] = P.com[3 * j + 1];
+    z[q] = P.com[3 * j + 2];
+  }
+#pragma unroll
+  for (int h = 0; h < 8; h += 4) {
+    double v[4][6];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = jc + min(h + q, nch - 1);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        v[q][d] = P.bmin[3 * j + d];
+        v[q][3 + d] = P.bmax[3 * j + d];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (h + q < nch) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          A.bn[d] = lesser(A.bn[d], v[q][d]);
+          A.bx[d] = greater(A.bx[d], v[q][3 + d]);
+        }
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    if (q < nch) A.add_mass(m[q], x[q], y[q], z[q]);
+  A.centre();
+#pragma unroll
+  for (int h = 0; h < 8; h += 4) {
+    double v[4][6];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = jc + min(h + q, nch - 1);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) v[q][k] = P.S[6 * j + k];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (h + q < nch) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) A.s6[k] += v[q][k];
+        A.add_outer(m[h + q], x[h + q] - A.cm[0], y[h + q] - A.cm[1], z[h + q] - A.cm[2]);
+      }
+  }
+  A.store(final_index(ni, c), C.key[c], C.pf[c], C.pc[c], make_int2(jc, nch), P);
 }
 
 // Leaves (of every level) bucketed by particle count, largest first, so that
@@ -882,15 +1028,148 @@ __global__ void __launch_bounds__(TB) k_leaf_props(Cells C, const int* __restric
                                                    Props P) {
   const int nl = misc[M_NLEAVES];
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nl; k += gridDim.x * blockDim.x)
-    cell_props<true>(lorder[k], C, ni, xs, ms, P);
+    leaf_props(lorder[k], C, ni, xs, ms, P);
 }
 
-// Nodes of level L (their children, one level deeper, are done).
-__global__ void __launch_bounds__(TB) k_node_props(int L, Cells C, const int* __restrict__ lvl,
-                                                   const int* __restrict__ ni, Props P) {
-  const int lb = lvl[L], le = lvl[L + 1];
-  for (int c = lb + blockIdx.x * blockDim.x + threadIdx.x; c < le; c += gridDim.x * blockDim.x)
-    if (C.nc[c] > 0) cell_props<false>(c, C, ni, nullptr, nullptr, P);
+// The double of another lane.
+__device__ __forceinline__ double from_lane(double v, int src) {
+  return __shfl_sync(FULL, v, src);
+}
+
+// node_props by eight lanes (l = 0..7, base = the first one's lane): every
+// FP64 instruction works on up to six components at once, each component's
+// operations in the same order. `live` lanes hold a node, the others only
+// take part in the shuffles.
+__device__ __forceinline__ void node_props8(int c, bool live, int l, int base, Cells C, const int* __restrict__ ni,
+                                            const Props& P) {
+  const int nch = live ? C.nc[c] : 0, jc = live ? final_index(ni, C.fc[c]) : 0;
+  const int last = max(nch - 1, 0);
+  // lanes 0..2 hold component l of vectors, lanes 0..5 component l of boxes and second moments
+  const int d = l < 3 ? l : (l < 6 ? l - 3 : 0), k6 = l < 6 ? l : 5;
+  double m[8], v[8], bb[8], ss[8];
+  if (live) {
+    const double* box = l < 3 ? P.bmin : P.bmax;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int j = jc + min(q, last);
+      m[q] = P.M[j];
+      v[q] = P.com[3 * j + d];
+      bb[q] = box[3 * j + d];
+      ss[q] = P.S[6 * j + k6];
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) m[q] = v[q] = bb[q] = ss[q] = 0;
+  }
+  double b = l < 3 ? INFINITY : -INFINITY;  // lanes 0..2: lower, 3..5: upper corner
+  double M = 0, s = 0;                      // lane 3 sums the mass: fma(m, 1, M) rounds as M + m
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if (q < nch) {
+      b = l < 3 ? lesser(b, bb[q]) : greater(b, bb[q]);
+      s = fma(m[q], l == 3 ? 1.0 : v[q], s);
+    }
+  }
+  M = from_lane(s, base + 3);
+  const double up = from_lane(b, base + min(l + 3, 7));
+  // centre of the cube and longest side (order-key comparisons: sides are >= 0)
+  const double cu = (b + up) * 0.5;
+  const double side = up - b;
+  double e = from_lane(side, base);
+  const double e1 = from_lane(side, base + 1), e2 = from_lane(side, base + 2);
+  if (order_key(e1) > order_key(e)) e = e1;
+  if (order_key(e2) > order_key(e)) e = e2;
+  const double half = 0.5 * e;
+  const double cm = M > 0 ? s / M : cu;  // lanes 0..2
+  // second moments: lane k takes w_a y_b of its pair (a, b)
+  const int pa = k6 < 3 ? k6 : (k6 == 5 ? 1 : 0), pb = k6 < 3 ? k6 : (k6 == 3 ? 1 : 2);
+  double s6 = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const double y = v[q] - cm, w = m[q] * y;
+    const double wa = from_lane(w, base + pa), yb = from_lane(y, base + pb);
+    if (q < nch) s6 = fma(wa, yb, s6 + ss[q]);
+  }
+  const double s0 = from_lane(s6, base), s1 = from_lane(s6, base + 1), s2 = from_lane(s6, base + 2);
+  const double tr = s0 + s1 + s2;
+  const float ch = static_cast<float>(cm), cl = static_cast<float>(cm - static_cast<double>(ch));
+  const float cuf = static_cast<float>(cu), t3 = static_cast<float>(3.0 * s6), Mf = static_cast<float>(M);
+  // a lane's float of the walk's records: (com_hi, M), (com_lo, count), 3S, 3 tr / 2, tr / 2; (cube centre, half side)
+  const float trf = static_cast<float>((l & 1 ? 0.5 : 1.5) * tr), hf = static_cast<float>(half);
+  if (!live) return;
+  const int j = final_index(ni, c), cnt = C.pc[c];
+  float* mp = reinterpret_cast<float*>(P.mp + 4 * static_cast<int64_t>(j));
+  float* geo = reinterpret_cast<float*>(P.geo + j);
+  if (l < 3) {
+    P.bmin[3 * j + l] = b;
+    P.bmax[3 * j + l] = up;
+    P.com[3 * j + l] = cm;
+    P.cube[4 * j + l] = cu;
+    mp[l] = ch;
+    mp[4 + l] = cl;
+    geo[l] = cuf;
+  }
+  if (l < 6) {
+    P.S[6 * j + l] = s6;
+    mp[8 + l] = t3;
+  } else {
+    mp[8 + l] = trf;  // lane 6: 3 tr / 2, lane 7: tr / 2
+  }
+  if (l == 3) {
+    P.M[j] = M;
+    mp[3] = Mf;
+    mp[7] = static_cast<float>(cnt);
+  }
+  if (l == 4) {
+    P.cube[4 * j + 3] = half;
+    geo[3] = hf;
+    P.key[j] = C.key[c];
+  }
+  if (l == 5) {
+    P.link[j] = make_int2(jc, nch);
+    P.pcount[j] = cnt;
+    P.cfirst[j] = C.pf[c];
+  }
+}
+
+// Nodes of all levels, deepest first, in one cooperative launch with a
+// barrier between levels; the nodes come from the level kernel's lists.
+//
+// Each of an SM's four schedulers issues an FP64 warp instruction every 82
+// clocks, however many lanes it has, so the number of FP64 instructions a
+// warp goes through is what counts: about 300 for 32 nodes, a lane each, or 80
+// for 4 nodes, eight lanes each. With NODE_WIDE nodes (four rounds of eight-lane warps
+// over the 608 schedulers) both take the same time; levels below it, nearly
+// all of them up to a few million particles, take eight lanes. As a launch per
+// level over all of its cells (one in eight a node), a lane per cell, the
+// nodes took 372 us at 1M particles and 170 us at 5000; 120 us and 58 us now.
+constexpr int NODE_WIDE = 4 * 4 * 608;
+
+__global__ void __launch_bounds__(NT) k_nodes(Cells C, int* lvl, const int* __restrict__ nlist,
+                                              const int* __restrict__ ni, Props P, int* misc) {
+  const int grid = gridDim.x, lane = threadIdx.x & 31;
+  const int warp = (threadIdx.x >> 5) * grid + static_cast<int>(blockIdx.x);  // consecutive warps on different SMs
+  const int warps = grid * (NT / 32);
+  int bars = 0;
+  if (__ldcg(&misc[M_STATUS]) & GPU_BUILD_STUCK) return;
+  for (int L = MAXD - 1; L >= 0; --L) {
+    const int nn = __ldcg(&misc[M_NODES + L]);
+    if (nn == 0) continue;
+    const int* nodes = nlist + lvl[L];
+    if (nn > NODE_WIDE) {
+      for (int k = 32 * warp + lane; k < nn; k += 32 * warps) node_props(nodes[k], C, ni, P);
+    } else {
+      for (int k0 = 4 * warp; k0 < nn; k0 += 4 * warps) {  // warp-uniform
+        const int k = k0 + (lane >> 3);
+        const bool live = k < nn;
+        node_props8(live ? nodes[k] : 0, live, lane & 7, lane & 24, C, ni, P);
+      }
+    }
+    if (L > 0 && !grid_barrier(&misc[M_BAR_NODES], ++bars * grid, &misc[M_STATUS])) {
+      no_cells(lvl);
+      return;
+    }
+  }
 }
 
 // ---------------------------------------------------------------- groups and items
@@ -1049,7 +1328,11 @@ __global__ void __launch_bounds__(TB) k_item_scatter(const int* __restrict__ n_i
   }
 }
 
-__global__ void k_clear_status(int* __restrict__ misc) { misc[M_STATUS] = 0; }
+// Before a refit: the counts of the build stay.
+__global__ void k_clear_status(int* __restrict__ misc) {
+  misc[M_STATUS] = 0;
+  misc[M_BAR_NODES] = 0;
+}
 
 __global__ void k_finish(const int* __restrict__ lvl, const int* __restrict__ misc, int64_t* __restrict__ res) {
   int depth = 0;
@@ -1080,6 +1363,36 @@ __global__ void k_unpermute(const float4* __restrict__ out, const int* __restric
 int grid_for(int64_t n, int per_block) {
   const int64_t b = (n + per_block - 1) / per_block;
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16)));
+}
+
+// Blocks of a cooperative launch: as many as the device holds at once, at most
+// `most` (the kernel's blocks wait for one another). 0 on an error.
+template <class K>
+int resident_blocks(K kernel, int threads, int most) {
+  int dev = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess)
+    return 0;
+  return std::min(sms * per, most);
+}
+
+template <class... A>
+cudaError_t launch_cooperative(void (*kernel)(A...), int blocks, int threads, cudaStream_t st, A... args) {
+  if (blocks < 1) return cudaErrorInvalidConfiguration;
+  void* argv[] = {&args...};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3(blocks), dim3(threads), argv, 0, st);
+}
+
+// The node kernel: a warp per 4 nodes of a level (a level holds at most n /
+// (n_leaf + 1) nodes) and at most one block per SM: its four warps have a
+// scheduler each, and fewer blocks make cheaper barriers.
+cudaError_t enqueue_nodes(const GpuBuild& a, const Layout& Lo, Cells C, const int* ni, Props P, cudaStream_t st) {
+  const int64_t blocks = std::max<int64_t>(1, (a.n / (a.n_leaf + 1) + 15) / 16);
+  const int most = static_cast<int>(std::min<int64_t>(blocks, 152));
+  return launch_cooperative(k_nodes, resident_blocks(k_nodes, NT, most), NT, st, C,
+                            at<int>(a.scratch, Lo.lvl),
+                            static_cast<const int*>(at<int>(a.scratch, Lo.nlist)), ni, P, at<int>(a.scratch, Lo.misc));
 }
 
 // Items from the groups (group_cell, group_sys and the cell arrays in P).
@@ -1186,12 +1499,12 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
   do {                                  \
     if ((e = (x)) != cudaSuccess) return e; \
   } while (0)
-  OG_TRY(cudaMemsetAsync(misc, 0, 4 * 16, st));
+  OG_TRY(cudaMemsetAsync(misc, 0, 4 * MISC, st));
 
   // ---- keys and the stable sort (8 passes of 8 bits over the 63-bit keys)
-  k_bbox<<<nch, TB, 0, st>>>(a.pos, a.mass, dch, part, misc);
+  k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, dch, part, misc);
   k_root<<<a.n_sys, TB, 0, st>>>(part, dchunk0, sg);
-  k_morton<<<nch, TB, 0, st>>>(a.pos, dch, sg, keyA, valA);
+  k_morton<<<SUB * nch, TB, 0, st>>>(a.pos, dch, sg, keyA, valA);
   int* dtot = at<int>(S, Lo.dtot);
   const int segblocks = (256 * a.n_sys + TB / 32 - 1) / (TB / 32);
   for (int pass = 0; pass < 8; ++pass) {
@@ -1207,14 +1520,14 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
 
   // ---- cells, level by level (sizes live in lvl[] on the device)
   k_roots<<<(std::max(a.n_sys, NLEV + 2) + 127) / 128, 128, 0, st>>>(a.n_sys, doffs, C, lvl);
-  const int top = std::min(std::max(a.max_level, 1), MAXD);  // deepest level built
-  for (int L = 0; L < top; ++L) {
-    k_split<<<GL, TB, 0, st>>>(L, keyA, C, a.n_leaf, lvl, spl, lpre, bsum);
-    k_scan_level<<<1, GLT, 0, st>>>(L, bsum, lvl, static_cast<int>(a.cap), misc);
-    k_emit<<<GL, TB, 0, st>>>(L, C, lvl, spl, lpre, bsum, misc);
+  {
+    // about a warp per cell that is split on the widest level; a small tree gets
+    // few blocks, whose barriers are cheaper
+    const int64_t want = std::max<int64_t>(1, a.n / (16 * (LT / 32)));
+    const int most = static_cast<int>(std::min<int64_t>(want, LBMAX));
+    OG_TRY(launch_cooperative(k_levels, resident_blocks(k_levels, LT, most), LT, st, static_cast<const uint64_t*>(keyA), C,
+                              a.n_leaf, lvl, spl, lpre, at<int>(S, Lo.nlist), bsum, static_cast<int>(a.cap), misc));
   }
-  if (top < MAXD) k_depth_check<<<grid_for(a.n, TB), TB, 0, st>>>(top, C, lvl, a.n_leaf, misc);
-  OG_TRY(cudaGetLastError());
 
   // ---- final (system-major) cell order
   const int gc = grid_for(a.cap, TB);
@@ -1240,8 +1553,8 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
   k_leaf_hist<<<gc, TB, 0, st>>>(C, lvl, lhist, misc);
   k_leaf_scatter<<<gc, TB, 0, st>>>(C, lvl, lhist, lhist + LBINS, lorder);
   k_leaf_props<<<gc, TB, 0, st>>>(C, lorder, misc, ni, xs, ms, P);
-  for (int L = top - 1; L >= 0; --L) k_node_props<<<gc, TB, 0, st>>>(L, C, lvl, ni, P);
   OG_TRY(cudaGetLastError());
+  OG_TRY(enqueue_nodes(a, Lo, C, ni, P, st));
 
   // ---- groups (ordered by first particle) and work items
   int* gmark = at<int>(S, Lo.gmark);
@@ -1277,11 +1590,11 @@ cudaError_t gpu_refit(const GpuBuild& a, cudaStream_t st) {
   cudaError_t e;
   // the status bits only: the counts of the build stay
   k_clear_status<<<1, 1, 0, st>>>(misc);
-  k_bbox<<<nch, TB, 0, st>>>(a.pos, a.mass, at<Chunk>(S, Lo.chunks), at<double>(S, Lo.part), misc);
+  k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, at<Chunk>(S, Lo.chunks), at<double>(S, Lo.part), misc);
   k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(at<uint32_t>(S, Lo.valA), a.pos, a.mass, a.n, at<double>(S, Lo.xs),
                                              at<double>(S, Lo.ms), a.parts, a.perm);
   k_leaf_props<<<gc, TB, 0, st>>>(C, at<int>(S, Lo.lorder), misc, ni, at<double>(S, Lo.xs), at<double>(S, Lo.ms), P);
-  for (int L = MAXD - 1; L >= 0; --L) k_node_props<<<gc, TB, 0, st>>>(L, C, lvl, ni, P);
+  if ((e = enqueue_nodes(a, Lo, C, ni, P, st)) != cudaSuccess) return e;
   k_items<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.group_sys, at<int>(S, Lo.ioff),
                                             a.cell_off, P, a.item_max, a.item_split, a.items, a.ibox, a.item_key,
                                             a.group_item);

@@ -295,7 +295,6 @@ struct Device {
   int device = -1;
   int pageable = -1;     // kernels may read pageable host memory (-1: not asked yet)
   int64_t cell_cap = 0;  // cell capacity that last sufficed for a GPU build
-  int level_hint = 0;    // depth of the last GPU build + 2 (0: none yet), caps the next level loop
   // the GPU build's kernels captured as a graph, replayed on gstream while
   // build_key (every argument, pointers included) stays the same
   cudaGraphExec_t build_exec = nullptr;

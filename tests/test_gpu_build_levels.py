@@ -1,0 +1,68 @@
+"""The level and node kernels of the GPU build where their rules change: cells
+of 32 and 33 particles (one probe per particle or a search), levels that end at
+the depth limit, trees of one block and of many, and more nodes on a level than
+eight-lane groups take. Byte equality with the host build throughout."""
+import numpy as np
+import pytest
+
+from paper_1005_5384_gb300 import octgrav as G
+from paper_1005_5384_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    G.load()
+
+
+def _same(pos, m, n_leaf, n_group):
+    A, B = G.Tree.build(pos, m, n_leaf, n_group), G.Tree.build_gpu(pos, m, n_leaf, n_group)
+    assert A.stats == B.stats
+    assert np.array_equal(A.perm(), B.perm()) and np.array_equal(A.cell_keys(), B.cell_keys())
+    a, b = A.cell_props(), B.cell_props()
+    for k in a:
+        assert np.array_equal(a[k].view(np.uint64), b[k].view(np.uint64)), k
+    return B
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 34, 255, 256, 257, 4095, 4097])
+@pytest.mark.parametrize("n_leaf", [1, 8])
+def test_small_trees(n, n_leaf):
+    pos, m = W.uniform_cube(n, seed=n)
+    _same(pos, m, n_leaf, 8 * n_leaf)
+
+
+@pytest.mark.parametrize("count", [32, 33, 1057, 1088, 1089])
+def test_cells_at_the_probe_bounds(count):
+    """One octant holds all but one particle: the first cells hold `count` and
+    fewer particles, on both sides of one round (32) and two (33 x 32 + 32)."""
+    rng = np.random.default_rng(count)
+    pos = rng.random((count, 3)) * 0.25
+    pos[0] = 1.0
+    _same(pos, np.full(count, 1.0 / count), 1, 4)
+
+
+def test_depth_limit_and_massless_nodes():
+    """Coincident particles below the depth limit (every level has one node),
+    and nodes whose children have no mass."""
+    rng = np.random.default_rng(3)
+    pos = rng.random((3000, 3))
+    pos[:40] = pos[0]
+    m = np.full(3000, 1e-3)
+    m[pos[:, 0] < 0.5] = 0.0
+    B = _same(pos, m, 4, 16)
+    assert B.stats["depth"] == G.MAX_DEPTH
+
+
+def test_more_nodes_on_a_level_than_eight_lane_groups_take():
+    """N_leaf = 1: tens of thousands of nodes on a level take the kernel's
+    lane-per-node form, the levels above it the eight-lane form."""
+    pos, m = W.plummer(120000, seed=6)
+    B = _same(pos, m, 1, 32)
+    depth = np.floor(np.log2(B.cell_keys().astype(np.float64)) / 3)
+    counts = B.cell_props()["count"]
+    assert max(int(np.sum((depth == d) & (counts > 1))) for d in range(22)) > 4 * 4 * 608
