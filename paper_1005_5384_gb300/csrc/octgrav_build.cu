@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "octgrav_internal.h"
@@ -1452,15 +1453,12 @@ cudaError_t gpu_build_tables(const GpuBuild& a, cudaStream_t st) {
   const std::vector<Chunk> ch = make_chunks(a.offsets, a.n_sys, chunk0);
   const Layout Lo = layout(a.n, a.n_sys, (a.n + TILE - 1) / TILE + a.n_sys, a.cap);
   if (Lo.total > a.scratch_bytes) return cudaErrorInvalidValue;
-  cudaError_t e;
-  if ((e = cudaMemcpyAsync(at<Chunk>(a.scratch, Lo.chunks), ch.data(), sizeof(Chunk) * ch.size(),
-                           cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(at<int64_t>(a.scratch, Lo.offs), a.offsets, 8 * (a.n_sys + 1), cudaMemcpyHostToDevice,
-                           st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(at<int>(a.scratch, Lo.chunk0), chunk0.data(), 4 * (a.n_sys + 1), cudaMemcpyHostToDevice,
-                           st)) != cudaSuccess)
-    return e;
-  return cudaSuccess;
+  // chunks, offsets and first chunks lie side by side: one copy
+  std::vector<char> host(Lo.chunk0 + 4 * static_cast<size_t>(a.n_sys + 1) - Lo.chunks);
+  std::memcpy(host.data(), ch.data(), sizeof(Chunk) * ch.size());
+  std::memcpy(host.data() + (Lo.offs - Lo.chunks), a.offsets, 8 * static_cast<size_t>(a.n_sys + 1));
+  std::memcpy(host.data() + (Lo.chunk0 - Lo.chunks), chunk0.data(), 4 * static_cast<size_t>(a.n_sys + 1));
+  return cudaMemcpyAsync(at<char>(a.scratch, Lo.chunks), host.data(), host.size(), cudaMemcpyHostToDevice, st);
 }
 
 cudaError_t gpu_build(const GpuBuild& a, cudaStream_t st) {

@@ -7,6 +7,103 @@
 
 namespace ogh {
 
+namespace {
+
+constexpr size_t kIdleSets = 2, kIdleBytes = size_t{1} << 30;
+
+struct IdleSet {
+  unsigned long long context;
+  Device D;
+};
+std::mutex idle_mu;
+// never destroyed: the driver may be gone before static destructors run
+std::vector<IdleSet>& idle_sets() {
+  static std::vector<IdleSet>& v = *new std::vector<IdleSet>();
+  return v;
+}
+
+// Identity of the current context, never used twice (0: unknown). A context
+// made anew after cudaDeviceReset has another one.
+unsigned long long context_id() {
+  using IdFn = CUresult (*)(CUcontext, unsigned long long*);
+  static const IdFn fn = []() -> IdFn {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<IdFn>(f);
+  }();
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;  // NULL: the calling thread's current context
+}
+
+}  // namespace
+
+bool release_idle() {
+  std::vector<IdleSet> sets;
+  {
+    std::lock_guard<std::mutex> g(idle_mu);
+    sets.swap(idle_sets());
+  }
+  const unsigned long long id = sets.empty() ? 0 : context_id();
+  bool any = false;
+  for (IdleSet& s : sets)
+    if (s.context == id) {  // others went with their context
+      s.D.release();
+      any = true;
+    }
+  return any;
+}
+
+void take_idle(int device, Device& D) {
+  const unsigned long long id = context_id();
+  Device got;
+  {
+    std::lock_guard<std::mutex> g(idle_mu);
+    std::vector<IdleSet>& sets = idle_sets();
+    for (size_t k = sets.size(); k-- > 0;)
+      if (sets[k].D.device == device && sets[k].context == id && id) {
+        got = std::move(sets[k].D);
+        sets.erase(sets.begin() + k);
+        break;
+      }
+  }
+  if (got.device < 0) return;
+  std::vector<DevBuf*> mine;  // what D already holds stays (a criterion set before the upload)
+  D.for_each([&](DevBuf& b) { mine.push_back(&b); });
+  size_t k = 0;
+  got.for_each([&](DevBuf& b) {
+    if (!mine[k]->p) std::swap(*mine[k], b);
+    ++k;
+  });
+  got.release();  // the rest
+}
+
+void give_idle(Device& D) {
+  int cur = -1;
+  size_t bytes = 0;
+  D.dbg.release();
+  D.for_each([&](DevBuf& b) { bytes += b.cap; });
+  const bool keep = bytes > 0 && bytes <= kIdleBytes && cudaGetDevice(&cur) == cudaSuccess && cur == D.device &&
+                    cudaDeviceSynchronize() == cudaSuccess;
+  const unsigned long long id = keep ? context_id() : 0;
+  if (id) {
+    std::lock_guard<std::mutex> g(idle_mu);
+    std::vector<IdleSet>& sets = idle_sets();
+    for (size_t k = sets.size(); k-- > 0;)  // sets of a context that is gone
+      if (sets[k].D.device == cur && sets[k].context != id) sets.erase(sets.begin() + k);
+    if (sets.size() < kIdleSets) {
+      D.release_graph();
+      D.cell_cap = 0;
+      sets.push_back({id, std::move(D)});
+      D = Device();
+      return;
+    }
+  }
+  D.release();
+}
+
 // Host memory reused by a thread's one-shot calls: the per-system build
 // arrays and the tree's host images keep their pages from call to call (at
 // N = 1M a call otherwise touches ~200 MB of fresh memory).
@@ -206,6 +303,7 @@ int upload(octgrav_tree* t, cudaStream_t st) {
   if (D.device >= 0 && D.device != dev) {
     D.release();
   }
+  if (D.device < 0 && t->dev == &t->own) take_idle(dev, D);
   D.device = dev;
   int rc;
   if (!t->gpu) {  // a GPU-built tree already lives in these arrays
@@ -385,6 +483,12 @@ int forces_host(octgrav_tree* t, double eps, double theta, double G, double* acc
   if (rc) return rc;
   // unpermute on the device, copy FP64 results straight into the caller's arrays
   Device& D = *t->dev;
+  if (D.device < 0 && t->dev == &t->own) {
+    int dev = 0;
+    CUDA_TRY(cudaGetDevice(&dev));
+    take_idle(dev, D);
+    D.device = dev;
+  }
   if ((rc = D.acc64.reserve(24 * t->n)) || (rc = D.pot64.reserve(8 * t->n))) return rc;
   if ((rc = forces_dev64(t, eps, theta, G, static_cast<double*>(D.acc64.p), static_cast<double*>(D.pot64.p), st,
                          ev)))
@@ -554,7 +658,10 @@ int build_gpu_common(int n_sys, const int64_t* offsets, const double* pos, const
     if (offsets[s + 1] <= offsets[s]) return fail(OCTGRAV_ERR_ARG, "empty or decreasing system %d", s);
   const int64_t n = offsets[n_sys];
   if (n >= (1ll << 31) - 64) return fail(OCTGRAV_ERR_ARG, "too many particles");
-  std::unique_ptr<octgrav_tree> t;
+  struct Free {
+    void operator()(octgrav_tree* p) const { octgrav_free_tree(p); }
+  };
+  std::unique_ptr<octgrav_tree, Free> t;
   try {
     t.reset(new octgrav_tree());
     t->sys_off.assign(offsets, offsets + n_sys + 1);
@@ -572,6 +679,7 @@ int build_gpu_common(int n_sys, const int64_t* offsets, const double* pos, const
   int cur = 0;
   CUDA_TRY(cudaGetDevice(&cur));
   if (D.device >= 0 && D.device != cur) D.release();
+  if (!dev) take_idle(cur, D);
   D.device = cur;
   // every level holds at most n cells (they are disjoint and non-empty)
   const int64_t bound = std::min<int64_t>(22 * n + n_sys, (1ll << 28) - 1);
@@ -605,7 +713,12 @@ int build_gpu_common(int n_sys, const int64_t* offsets, const double* pos, const
   t->max_group = res[og::GB_MAXGROUP];
   t->ordered = true;  // the build wrote the default order (most particles first)
   t->cell_off.resize(n_sys + 1);
-  CUDA_TRY(cudaMemcpy(t->cell_off.data(), D.celloff.p, 8 * (n_sys + 1), cudaMemcpyDeviceToHost));
+  if (n_sys == 1) {
+    t->cell_off[0] = 0;
+    t->cell_off[1] = t->n_cells;
+  } else {
+    CUDA_TRY(cudaMemcpy(t->cell_off.data(), D.celloff.p, 8 * (n_sys + 1), cudaMemcpyDeviceToHost));
+  }
   if ((rc = upload(t.get(), st))) return rc;  // counts, control word, tensor map
   *out = t.release();
   return OCTGRAV_OK;
@@ -1596,7 +1709,8 @@ int octgrav_set_staging(octgrav_tree* t, int mode) {
 void octgrav_free_tree(octgrav_tree* t) {
   if (!t) return;
   if (t->gexec) cudaGraphExecDestroy(t->gexec);
-  t->own.release();
+  if (t->own.device >= 0) give_idle(t->own);
+  else t->own.release();
   delete t;
 }
 
