@@ -509,16 +509,23 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
   uint32_t iss = 0;  // gather4 staging: entries whose copies were issued (multiple of 4)
   int status = 0;
 
+  // The first work indices are dealt out, one to a warp, across the CTAs: the
+  // items come largest first, and taken from the counter alone a CTA's warps
+  // get neighbours in that order, so that a system of about one item per warp
+  // (65k particles at N_group 128) had its largest items on a few SMs.
+  const int dealt = gridDim.x * CtaWarps<MLP>::v;
+  int first = static_cast<int>((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
   for (;;) {
     int item = 0, part = 0;
     if (lane == 0) {
-      item = static_cast<int>(atomicAdd(p.work, 1u));
+      item = first >= 0 ? first : static_cast<int>(atomicAdd(p.work, 1u)) + dealt;
       if (SPLIT) {  // the parts of one item are consecutive work indices
         part = item % p.nparts;
         item /= p.nparts;
       }
       if (p.order && item < p.n_items) item = __ldg(p.order + item);  // longest first
     }
+    first = -1;
     item = __shfl_sync(FULL, item, 0);
     if (SPLIT) part = __shfl_sync(FULL, part, 0);
     if (item >= p.n_items) break;
