@@ -33,6 +33,7 @@
 // FP32 and folded into a compensated (TwoSum) accumulator every ~32 terms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include <mutex>
@@ -75,7 +76,7 @@ struct __align__(128) WarpSmemT {
                                     // rewritten in place into pairs; also the network's input
                                     // tile (32 rows x 16 bf16) during a network step
   int2 leafq[LQ];                   // 512 B: (first particle, count)
-  int lpref[LQ];                    // 256 B: inclusive prefix of counts
+  int lpref[LQ];                    // 256 B: sources of the entries before
   int stack[MLP ? STACK_MLP : STACK];  // packed (first child << 3 | n_child - 1)
   int cidx[GATHER ? NTILE * TILE : 1]; // cell index per ring slot (gather4 staging)
   int mq[MLP ? MQ : 1];             // deferred candidate cells
@@ -279,42 +280,52 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(rsqrt_ftz(a.x), rsqrt_ftz(a.y)); }
 
-struct Acc2 {  // partial sums of the two halves of a pair
-  float2 x, y, z, p;
+// The two scalar FMAs of a packed one (the same results).
+__device__ __forceinline__ float2 fma1(float2 a, float2 b, float2 c) {
+  return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y));
+}
+
+// Partial sums of the two halves of a pair. p + w is -2 phi (a power of two
+// away, so that no rounding changes): p sums the monopoles' share, w the
+// quadrupoles', whose roundings are far smaller; one sum for both would round
+// twice per cell (20 % more error at 1M particles).
+struct Acc2 {
+  float2 x, y, z, p, w;
 };
 
 // Two cell records side by side (each field holds record a in .x, record b
 // in .y): centre of mass relative to the group centre and negated (nc), -M,
-// S3 = 3 S, T3 = 3T and T = tr(S)/2. 96 bytes = six 16-byte loads.
+// the traceless quadrupole S = 3 sum m y y^T - tr I, k = -eps^2 tr and 2M.
+// 96 bytes = six 16-byte loads.
 struct CellPair {
-  float2 ncx, ncy, ncz, nM, sxx, syy, szz, sxy, sxz, syz, t3, t;
+  float2 ncx, ncy, ncz, nM, sxx, syy, szz, sxy, sxz, syz, k, M2;
 };
 
 // Particle-cell interaction: second-order Taylor expansion of the Plummer
 // kernel about the cell's centre of mass (monopole + quadrupole). With
-// d = x_i - com, r^2 = |d|^2 + eps^2, S3 = 3S, q = d.S3.d, T = trS/2:
-//   a   += d (-M + (3T - 2.5 q/r^2)/r^2) / r^3 + S3 d / r^5
-//   phi -= (M + (q/(2 r^2) - T)/r^2) / r
+// d = x_i - com, r^2 = |d|^2 + eps^2 and q = d.S.d - eps^2 tr:
+//   a   += (S d - (M r^2 + 2.5 q/r^2) d) / r^5
+//   phi -= M/r + q/(2 r^5)
+// The trace part of the expansion, (d.3S.d)/(2 r^5) - tr/(2 r^3), differs from
+// the traceless one by the constant in q alone: 32 packed operations for two
+// interactions, one less than with the trace carried through both sums.
 __device__ __forceinline__ void body_cell2(float2 X, float2 Y, float2 Z, float2 eps2, const CellPair& c,
                                            Acc2& a) {
   const float2 dx = add2(X, c.ncx), dy = add2(Y, c.ncy), dz = add2(Z, c.ncz);
   const float2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, eps2)));
   const float2 rinv = rsqrt2(r2);
   const float2 rinv2 = mul2(rinv, rinv);
-  const float2 rinv3 = mul2(rinv, rinv2);
-  const float2 rinv5 = mul2(rinv3, rinv2);
+  const float2 rinv5 = mul2(mul2(rinv, rinv2), rinv2);
   const float2 sx = fma2(c.sxx, dx, fma2(c.sxy, dy, mul2(c.sxz, dz)));
   const float2 sy = fma2(c.sxy, dx, fma2(c.syy, dy, mul2(c.syz, dz)));
   const float2 sz = fma2(c.sxz, dx, fma2(c.syz, dy, mul2(c.szz, dz)));
-  const float2 q = fma2(dx, sx, fma2(dy, sy, mul2(dz, sz)));
-  const float2 t1 = mul2(q, rinv2);
-  const float2 t2 = fma2(f2(-2.5f), t1, c.t3);
-  const float2 cd = mul2(fma2(t2, rinv2, c.nM), rinv3);
-  a.x = fma2(cd, dx, fma2(rinv5, sx, a.x));
-  a.y = fma2(cd, dy, fma2(rinv5, sy, a.y));
-  a.z = fma2(cd, dz, fma2(rinv5, sz, a.z));
-  const float2 np2 = fma2(fma2(f2(-0.5f), t1, c.t), rinv2, c.nM);  // -(M + (q/(2r^2) - T)/r^2)
-  a.p = fma2(np2, rinv, a.p);
+  const float2 q = fma2(dx, sx, fma2(dy, sy, fma2(dz, sz, c.k)));
+  const float2 cb = fma2(f2(-2.5f), mul2(q, rinv2), mul2(c.nM, r2));
+  a.x = fma2(rinv5, fma2(cb, dx, sx), a.x);
+  a.y = fma2(rinv5, fma2(cb, dy, sy), a.y);
+  a.z = fma2(rinv5, fma2(cb, dz, sz), a.z);
+  a.p = fma2(c.M2, rinv, a.p);
+  a.w = fma2(q, rinv5, a.w);
 }
 
 // Two source particles side by side: negated positions (relative to the group
@@ -334,7 +345,7 @@ __device__ __forceinline__ void body_body2(float2 X, float2 Y, float2 Z, float2 
   a.x = fma2(nmr3, dx, a.x);  // += m_j (x_j - x_i) / r^3
   a.y = fma2(nmr3, dy, a.y);
   a.z = fma2(nmr3, dz, a.z);
-  a.p = add2(a.p, nmr);       // -= m_j / r
+  a.p = fma2(f2(-2.f), nmr, a.p);  // += 2 m_j / r
 }
 
 // ---- particle-packed evaluation (two particles per lane): the halves of
@@ -342,37 +353,47 @@ __device__ __forceinline__ void body_body2(float2 X, float2 Y, float2 Z, float2 
 // source quantities enter as one value broadcast to both halves.
 
 // One cell record for the particle-packed layout (48 bytes = three 16-byte
-// loads): centre of mass relative to the group centre, negated, -M, S3 = 3S
-// (xx, yy, zz, xy, xz, yz), 3T and T = tr(S)/2.
+// loads): CellPair's fields of one cell.
 struct CellRec {
-  float ncx, ncy, ncz, nM, sxx, syy, szz, sxy, sxz, syz, t3, t;
+  float ncx, ncy, ncz, nM, sxx, syy, szz, sxy, sxz, syz, k, M2;
 };
 constexpr int CREC = 3;  // float4 per cell record in the evaluated tile
 static_assert(16 * CREC <= 64, "packed cell records must fit the tile's ring slots");
 static_assert(16 * 32 + 4 * 32 <= 32 * 32, "packed sources and indices must fit a chunk");
 
 // Particle-cell interaction of two particles (X, Y, Z halves) with one cell:
-// the same expansion as body_cell2, with the monopole folded into the bracket,
-//   a += (S3 d + (3T - 2.5 q/r^2 - M r^2) d) / r^5
-// (33 packed operations for two interactions).
+// the same 32 operations. With three different 64-bit operands a packed FMA
+// holds the FMA pipe for three cycles instead of two, and operands that
+// neighbouring instructions share are read once: hence the products of S and d
+// column by column, and (SP) the monopole's potential, which nothing waits for,
+// as two scalar FMAs. Of 112 orders of these statements and operands timed at
+// 1M particles (7.62 to 8.0 ms) this was the fastest; in place 7.67 ms, the same with
+// a packed potential 7.77. Other scalar splits were slower, as issue slots run
+// out. The learned kernel keeps the potential packed (1.72 against 1.74 ms).
+template <bool SP>
 __device__ __forceinline__ void body_cellP(float2 X, float2 Y, float2 Z, float2 eps2, const CellRec& c,
                                            Acc2& a) {
   const float2 dx = add2(X, f2(c.ncx)), dy = add2(Y, f2(c.ncy)), dz = add2(Z, f2(c.ncz));
-  const float2 r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, eps2)));
+  const float2 r2 = fma2(dy, dy, fma2(dz, dz, fma2(dx, dx, eps2)));
   const float2 rinv = rsqrt2(r2);
+  const float2 tx0 = mul2(dz, f2(c.sxz));
+  const float2 ty0 = mul2(f2(c.syz), dz);
+  const float2 tz0 = mul2(f2(c.szz), dz);
+  const float2 tx1 = fma2(f2(c.sxx), dx, tx0);
+  const float2 ty1 = fma2(dx, f2(c.sxy), ty0);
+  const float2 tz1 = fma2(dx, f2(c.sxz), tz0);
+  const float2 sx = fma2(f2(c.sxy), dy, tx1);
+  const float2 sy = fma2(f2(c.syy), dy, ty1);
+  const float2 sz = fma2(f2(c.syz), dy, tz1);
   const float2 rinv2 = mul2(rinv, rinv);
-  const float2 rinv5 = mul2(mul2(rinv, rinv2), rinv2);
-  const float2 sx = fma2(f2(c.sxx), dx, fma2(f2(c.sxy), dy, mul2(f2(c.sxz), dz)));
-  const float2 sy = fma2(f2(c.sxy), dx, fma2(f2(c.syy), dy, mul2(f2(c.syz), dz)));
-  const float2 sz = fma2(f2(c.sxz), dx, fma2(f2(c.syz), dy, mul2(f2(c.szz), dz)));
-  const float2 q = fma2(dx, sx, fma2(dy, sy, mul2(dz, sz)));
-  const float2 t1 = mul2(q, rinv2);
-  const float2 cb = fma2(f2(c.nM), r2, fma2(f2(-2.5f), t1, f2(c.t3)));  // 3T - 2.5 q/r^2 - M r^2
-  a.x = fma2(rinv5, fma2(cb, dx, sx), a.x);
-  a.y = fma2(rinv5, fma2(cb, dy, sy), a.y);
-  a.z = fma2(rinv5, fma2(cb, dz, sz), a.z);
-  const float2 np2 = fma2(fma2(f2(-0.5f), t1, f2(c.t)), rinv2, f2(c.nM));
-  a.p = fma2(np2, rinv, a.p);
+  const float2 rinv5 = mul2(rinv2, mul2(rinv2, rinv));
+  const float2 q = fma2(sx, dx, fma2(dz, sz, fma2(dy, sy, f2(c.k))));
+  const float2 cb = fma2(f2(-2.5f), mul2(rinv2, q), mul2(r2, f2(c.nM)));
+  a.z = fma2(fma2(cb, dz, sz), rinv5, a.z);
+  a.x = fma2(fma2(dx, cb, sx), rinv5, a.x);
+  a.y = fma2(fma2(cb, dy, sy), rinv5, a.y);
+  a.p = SP ? fma1(rinv, f2(c.M2), a.p) : fma2(rinv, f2(c.M2), a.p);
+  a.w = fma2(q, rinv5, a.w);
 }
 
 // Particle-particle interaction of two particles with one source (negated
@@ -387,7 +408,7 @@ __device__ __forceinline__ void body_bodyP(float2 X, float2 Y, float2 Z, float2 
   a.x = fma2(nmr3, dx, a.x);
   a.y = fma2(nmr3, dy, a.y);
   a.z = fma2(nmr3, dz, a.z);
-  a.p = add2(a.p, nmr);
+  a.p = fma2(f2(-2.f), nmr, a.p);
 }
 
 // Error-free transformation: hi + t = s + e exactly.
@@ -413,8 +434,8 @@ struct Particles {
       two_sum_into(hi[r].x, lo[r].x, part[r].x.x + part[r].x.y);
       two_sum_into(hi[r].y, lo[r].y, part[r].y.x + part[r].y.y);
       two_sum_into(hi[r].z, lo[r].z, part[r].z.x + part[r].z.y);
-      two_sum_into(hi[r].p, lo[r].p, part[r].p.x + part[r].p.y);
-      part[r].x = part[r].y = part[r].z = part[r].p = f2(0.f);
+      two_sum_into(hi[r].p, lo[r].p, (part[r].p.x + part[r].p.y) + (part[r].w.x + part[r].w.y));
+      part[r].x = part[r].y = part[r].z = part[r].p = part[r].w = f2(0.f);
     }
   }
 };
@@ -431,18 +452,22 @@ __device__ __forceinline__ void two_sum_into2(float2& hi, float2& lo, float2 t) 
 // Two particles per lane in the halves of every register (particle-packed
 // layout): positions, partial sums since the last fold and compensated
 // accumulators (value = hi + lo), each half one particle.
+struct Acc4x2 {
+  float2 x, y, z, p;
+};
+
 struct ParticlesP {
   float2 X, Y, Z;
   int idx[2];  // tree positions, -1 for an empty slot
   Acc2 part;
-  Acc2 hi, lo;
+  Acc4x2 hi, lo;
 
   __device__ __forceinline__ void fold() {
     two_sum_into2(hi.x, lo.x, part.x);
     two_sum_into2(hi.y, lo.y, part.y);
     two_sum_into2(hi.z, lo.z, part.z);
-    two_sum_into2(hi.p, lo.p, part.p);
-    part.x = part.y = part.z = part.p = f2(0.f);
+    two_sum_into2(hi.p, lo.p, add2(part.p, part.w));
+    part.x = part.y = part.z = part.p = part.w = f2(0.f);
   }
 };
 
@@ -506,6 +531,11 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
   // cell entries whose copies were issued, `done` those evaluated. Tile
   // (e / TILE) % NTILE holds entry e; its k-th use completes phase k.
   uint32_t app = 0, done = 0;
+  uint32_t app_slot = 0, done_slot = 0;  // app and done modulo the ring (96 is no power of two)
+  auto advance = [](uint32_t slot, uint32_t by) {  // by <= the ring
+    const uint32_t t = slot + by;
+    return t >= NTILE * TILE ? t - NTILE * TILE : t;
+  };
   uint32_t iss = 0;  // gather4 staging: entries whose copies were issued (multiple of 4)
   int status = 0;
 
@@ -595,16 +625,15 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       P.X = make_float2(px[0], px[1]);
       P.Y = make_float2(py[0], py[1]);
       P.Z = make_float2(pz[0], pz[1]);
-      P.part.x = P.part.y = P.part.z = P.part.p = f2(0.f);
-      P.hi = P.part;
-      P.lo = P.part;
+      P.part.x = P.part.y = P.part.z = P.part.p = P.part.w = f2(0.f);
+      P.hi = P.lo = Acc4x2{f2(0.f), f2(0.f), f2(0.f), f2(0.f)};
     } else {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         P.X[r] = f2(px[r]);
         P.Y[r] = f2(py[r]);
         P.Z[r] = f2(pz[r]);
-        P.part[r].x = P.part[r].y = P.part[r].z = P.part[r].p = f2(0.f);
+        P.part[r].x = P.part[r].y = P.part[r].z = P.part[r].p = P.part[r].w = f2(0.f);
         P.hi[r] = P.lo[r] = Acc4{0.f, 0.f, 0.f, 0.f};
       }
     }
@@ -612,7 +641,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
 
     // ---- evaluation of one ring tile holding n records
     auto eval_tile = [&](int n) -> bool {
-      const uint32_t tile = (done / TILE) % NTILE;
+      const uint32_t tile = done_slot / TILE;
       const uint32_t parity = (done / (TILE * NTILE)) & 1u;
       if (STAGE == STAGE_ASYNC) {
         __syncwarp();  // the lanes' completed copies (waited by the caller) are visible
@@ -623,17 +652,23 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       // Rewrite the tile in place into the pair layout: record e becomes half
       // (e & 1) of pair e >> 1; an odd last record is paired with zeros.
       float v[12];
-#pragma unroll
-      for (int f = 0; f < 12; ++f) v[f] = 0.f;
-      if (lane < n) {
+      auto read = [&]() {
         const float4 q0 = base[lane * REC], q1 = base[lane * REC + 1];
         const float4 q2 = base[lane * REC + 2], q3 = base[lane * REC + 3];
         v[0] = -((q0.x - chi.x) + (q1.x - clo.x));
         v[1] = -((q0.y - chi.y) + (q1.y - clo.y));
         v[2] = -((q0.z - chi.z) + (q1.z - clo.z));
+        const float tr = 2.f * q3.w;
         v[3] = -q0.w;
-        v[4] = q2.x; v[5] = q2.y; v[6] = q2.z; v[7] = q2.w;
-        v[8] = q3.x; v[9] = q3.y; v[10] = q3.z; v[11] = q3.w;
+        v[4] = q2.x - tr; v[5] = q2.y - tr; v[6] = q2.z - tr; v[7] = q2.w;
+        v[8] = q3.x; v[9] = q3.y; v[10] = -tr * E2.x; v[11] = 2.f * q0.w;
+      };
+      if (n == TILE) {  // all but an item's last tile
+        read();
+      } else {
+#pragma unroll
+        for (int f = 0; f < 12; ++f) v[f] = 0.f;
+        if (lane < n) read();
       }
       __syncwarp();
       const int npad = (n + 1) & ~1;
@@ -652,8 +687,8 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
           for (int k = sl; k < npad / 2; k += s) {  // records 2k and 2k+1
             const CellRec c0 = load_cell_rec(pb + CREC * (2 * k));
             const CellRec c1 = load_cell_rec(pb + CREC * (2 * k + 1));
-            body_cellP(P.X, P.Y, P.Z, E2, c0, P.part);
-            body_cellP(P.X, P.Y, P.Z, E2, c1, P.part);
+            body_cellP<!MLP>(P.X, P.Y, P.Z, E2, c0, P.part);
+            body_cellP<!MLP>(P.X, P.Y, P.Z, E2, c1, P.part);
           }
         }
       } else {
@@ -679,36 +714,42 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       if (STAGE != STAGE_ASYNC) fence_proxy_async();
       __syncwarp();
       done += TILE;
+      done_slot = advance(done_slot, TILE);
       return true;
     };
 
     // ---- particle-particle evaluation in chunks of PCH sources (Listing 4).
     // Chunk k+1 is copied asynchronously while chunk k is evaluated. The
     // sources are either the particles of the queued leaves (rank -> particle
-    // through the prefix of leaf counts) or, with `own`, the item's whole
+    // through the sources of the leaves before) or, with `own`, the item's whole
     // group, whose pass excludes the self term.
+    // A chunk's leaves: the lanes' two entries that start in it (first0, first1:
+    // the sources before them) set a bit each, and a source's entry is the
+    // number of starts up to it, counted from the earlier chunks' on.
     int n_pp = 0;
-    auto pp_pass = [&](int total, int nq, bool own) {
+    auto pp_pass = [&](int total, int first0, int first1, bool own) {
       const int nchunk = (total + PCH - 1) / PCH;
+      int before = -1;  // entries that start before the chunk, less one
       auto stage = [&](int k) -> int {
         const int rk = k * PCH + lane;
         int j = -1;
+        unsigned starts = 0;
+        if (!own) {
+          const unsigned d0 = first0 - k * PCH, d1 = first1 - k * PCH;
+          starts = __reduce_or_sync(FULL, (d0 < 32u ? 1u << d0 : 0u) | (d1 < 32u ? 1u << d1 : 0u));
+        }
         if (rk < total) {
           if (own) {
             j = gfirst + rk;
           } else {
-            int lo = 0, hi = nq - 1;  // first entry whose inclusive prefix exceeds rk
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (S.lpref[mid] > rk) hi = mid; else lo = mid + 1;
-            }
-            const int start = lo ? S.lpref[lo - 1] : 0;
-            j = S.leafq[lo].x + (rk - start);
+            const int e = before + __popc(starts & (lt | (1u << lane)));
+            j = S.leafq[e].x + (rk - S.lpref[e]);
           }
           const uint32_t dst = smem_u32(&S.pbuf[k & 1][2 * lane]);
           cp_async16(dst, p.parts + 2 * j);
           cp_async16(dst + 16, p.parts + 2 * j + 1);
         }
+        before += __popc(starts);
         cp_async_commit();
         return j;
       };
@@ -816,11 +857,13 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       }
       const int tot0 = __shfl_sync(FULL, s0, 31);
       const int total = tot0 + __shfl_sync(FULL, s1, 31);
+      s0 -= c0;  // sources before the entry
+      s1 += tot0 - c1;
       S.lpref[lane] = s0;
-      S.lpref[lane + 32] = s1 + tot0;
+      S.lpref[lane + 32] = s1;
       __syncwarp();
       n_pp += total;
-      pp_pass(total, nq, false);
+      pp_pass(total, lane < nq ? s0 : INT_MAX, lane + 32 < nq ? s1 : INT_MAX, false);
     };
 
     // The group's own particles: they sit in the group's own leaves, which are
@@ -828,7 +871,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
     // left out, instead of through the leaf queue.
     if (!SPLIT || part == 0) {
       n_pp += gcount;
-      pp_pass(gcount, 0, true);
+      pp_pass(gcount, 0, 0, true);
     }
 
     // ---- walk (Listing 1): root opened; children of up to 4 nodes per step
@@ -861,18 +904,13 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       const int k = lane >> 3, slot = lane & 7;
       const int packed = k < npop ? S.stack[top - npop + k] : 0;
       const int nch = (packed & 7) + 1;
-      nx_valid = (k < npop) && (slot < nch);
-      nx_c = (packed >> 3) + slot;
-      if (nx_valid && static_cast<unsigned>(nx_c) >= static_cast<unsigned>(p.n_cells)) {
-        status |= ST_INDEX;
-        nx_valid = false;
-      }
-      nx_g = make_float4(0.f, 0.f, 0.f, 0.f);
-      nx_lk = make_int2(0, 0);
-      if (nx_valid) {
-        nx_g = __ldg(p.geo + nx_c);
-        nx_lk = __ldg(p.link + nx_c);
-      }
+      const int child = (packed >> 3) + slot;
+      const bool there = (k < npop) && (slot < nch);
+      nx_valid = there && static_cast<unsigned>(child) < static_cast<unsigned>(p.n_cells);
+      if (there && !nx_valid) status |= ST_INDEX;
+      nx_c = nx_valid ? child : 0;  // lanes without a child load cell 0 and ignore it
+      nx_g = __ldg(p.geo + nx_c);
+      nx_lk = __ldg(p.link + nx_c);
       __syncwarp();  // stack reads precede the next step's pushes
     };
     // Learned criterion: the opening test with theta_hi opens, with theta_lo
@@ -962,7 +1000,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       // leaves of the own group are evaluated by the own pass, not queued
       const bool own_leaf = open && leaf && lk.x >= gfirst && lk.x < gfirst + gcount;
       const unsigned m_acc = __ballot_sync(FULL, valid && !open);
-      const unsigned m_leaf = __ballot_sync(FULL, open && leaf);
+      const unsigned m_leaf = CAPTURE ? __ballot_sync(FULL, open && leaf) : 0u;
       const unsigned m_lq = __ballot_sync(FULL, open && leaf && !own_leaf);
       const unsigned m_node = __ballot_sync(FULL, open && !leaf);
       const int nn = __popc(m_node);
@@ -986,8 +1024,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       unsigned m_stage = m_acc;  // the accepted cells this warp evaluates
       if (SPLIT) m_stage = __ballot_sync(FULL, valid && !open && (n_pc + __popc(m_acc & lt)) % p.nparts == part);
       if ((m_stage >> lane) & 1u) {
-        const uint32_t e = app + __popc(m_stage & lt);
-        const uint32_t se = e % (NTILE * TILE);
+        const uint32_t se = advance(app_slot, __popc(m_stage & lt));
         if (STAGE == STAGE_BULK) {
           const uint32_t bar = bar0 + 8 * (se / TILE);
           mbar_expect_tx(bar, 64);
@@ -1006,6 +1043,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       const int na = __popc(m_stage);
       const uint32_t old = app;
       app += na;
+      app_slot = advance(app_slot, na);
       n_pc += __popc(m_acc);
       if (STAGE == STAGE_ASYNC) cp_async_commit();
       __syncwarp();  // all expect_tx / index writes of this step are done
@@ -1042,7 +1080,10 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       if (STAGE == STAGE_ASYNC) {
         cp_async_wait_all();
         __syncwarp();
-        if (rem) app += TILE - rem;
+        if (rem) {
+          app += TILE - rem;
+          app_slot = advance(app_slot, TILE - rem);
+        }
       } else if (rem) {
         __syncwarp();
         if (lane == 0 && app >= drop_end) {
@@ -1061,6 +1102,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
           mbar_arrive(bar);
         }
         app += TILE - rem;
+        app_slot = advance(app_slot, TILE - rem);
         iss = app;
       }
       while (done < app) {
@@ -1070,6 +1112,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
           const uint32_t tile = (done / TILE) % NTILE;
           if (STAGE != STAGE_ASYNC) mbar_wait_bounded(bar0 + 8 * tile, (done / (TILE * NTILE)) & 1u);
           done += TILE;
+          done_slot = advance(done_slot, TILE);
           continue;
         }
         if (!eval_tile(n)) ok = false;
@@ -1124,7 +1167,7 @@ __global__ void __launch_bounds__(CtaWarps<MLP>::v * 32, MLP ? 1 : 2) walk_eval_
       for (int r = 0; r < R; ++r) {
         if (P.idx[r] >= 0) {
           const float4 v = make_float4(G * (H[r].x + L[r].x), G * (H[r].y + L[r].y),
-                                       G * (H[r].z + L[r].z), G * (H[r].p + L[r].p));
+                                       G * (H[r].z + L[r].z), G * (-0.5f * (H[r].p + L[r].p)));
           if (SPLIT)
             p.part_out[static_cast<size_t>(part) * p.n + P.idx[r]] = v;
           else
