@@ -91,7 +91,7 @@ int octgrav_tree_upload(octgrav_tree *t, void *stream);
  *   order with octgrav_tree_perm.
  *   eps > 0, theta >= 0, G finite. For a batched tree the values apply to every
  *   system unless octgrav_set_system_params was called.
- * Launches exactly one kernel. Device-side failures (stack overflow, timeout)
+ * Launches one kernel (two where the lists are split, see octgrav_set_split). Device-side failures (stack overflow, timeout)
  * are recorded in a status word read by octgrav_status. Errors: ERR_ARG,
  * ERR_CUDA. */
 int octgrav_forces_device(octgrav_tree *t, double eps, double theta, double G, float *acc4_dev,
@@ -482,9 +482,10 @@ int octgrav_set_fault(octgrav_tree *t, int stack_cap, int64_t drop_item);
  * accepted cells and queued leaves whose sequence numbers are j modulo nparts
  * (part 0 also the group's own particles), and the parts' results are summed
  * in part order by a second kernel, so a launch is deterministic but rounds
- * differently from an unsplit one (FP32 sums of nparts partial results).
- * Applies to launches with the plain opening test and staging mode 1 that
- * capture no lists; others run unsplit. Errors: ERR_ARG. */
+ * differently from an unsplit one (a sum of nparts FP32 results). Until this is
+ * called a tree of at most 2550 work items is split over 2, 4 or 8 warps by
+ * their number. Applies to launches with the plain opening test that capture no
+ * lists; others run unsplit. Errors: ERR_ARG. */
 int octgrav_set_split(octgrav_tree *t, int nparts);
 
 void octgrav_free_tree(octgrav_tree *t);
@@ -507,8 +508,9 @@ void octgrav_free_tree(octgrav_tree *t);
  * The tree's settings apply as in octgrav_forces_device -- staging mode,
  * particles per lane, per-system parameters and the learned criterion (whose
  * network stays in the tree's device memory; set it on the current device) --
- * except the list split of octgrav_set_split, which needs a per-part output
- * buffer: these launches run unsplit and round like an unsplit launch.
+ * except a list split asked for with octgrav_set_split: these launches run as
+ * octgrav_forces_device does where that was not called (the parts' outputs of
+ * a small tree are in the arena).
  * The status word, work-queue counter and per-item counts live in a
  * fixed-size array inside the library (2 MiB + 256 B per GPU, kept until the
  * process exits), so the tree may have at most OCTGRAV_NOALLOC_MAX_ITEMS work

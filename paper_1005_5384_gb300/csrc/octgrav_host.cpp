@@ -296,6 +296,33 @@ int build_oneshot(const double* pos, const double* mass, int64_t n, int n_leaf, 
 }
 
 
+// Parts that fill the GPU's 2432 warp slots for a system of few work items:
+// the largest power of two up to 8 that keeps items x parts within 2.1 times
+// the slots (every part repeats the item's walk, so more parts than that cost
+// more than the shorter evaluation gains). Times by parts 1 / 2 / 4 / 8 (us,
+// theta 0.5 to 0.7): 112 items 48 / 37 / 28 / 26, 340 150 / 100 / 74 / 62, 688
+// 195 / 140 / 107 / 127, 1111 448 / 346 / 309 / 411, 2516 504 / 389 / 498 / 727.
+int auto_parts(int64_t n_items) {
+  int parts = 8;
+  while (parts > 1 && n_items * parts > 5100) parts /= 2;
+  return parts;
+}
+
+// Parts of a list-split launch of t (1: no split): launches with the plain
+// criterion that capture no lists split, as octgrav_set_split said or, without
+// it, by auto_parts.
+int split_parts(const octgrav_tree* t, bool capture) {
+  if (capture || t->learned) return 1;
+  return t->nparts > 0 ? t->nparts : auto_parts(t->n_items);
+}
+
+// The parts' outputs, reserved where the work items are made, so that a launch
+// (which may be in a stream capture) allocates nothing.
+int reserve_parts(octgrav_tree* t) {
+  const int parts = split_parts(t, false);
+  return parts > 1 ? t->dev->split.reserve(sizeof(float4) * parts * static_cast<size_t>(t->n)) : OCTGRAV_OK;
+}
+
 int upload(octgrav_tree* t, cudaStream_t st) {
   int dev = 0;
   CUDA_TRY(cudaGetDevice(&dev));
@@ -328,7 +355,7 @@ int upload(octgrav_tree* t, cudaStream_t st) {
     t->perm_on_device = true;
   }
   if ((rc = D.counts.reserve(t->n_items * sizeof(int2)))) return rc;
-  if ((rc = D.ctl.reserve(64))) return rc;
+  if ((rc = D.ctl.reserve(64)) || (rc = reserve_parts(t))) return rc;
   {
     cudaError_t e = og::encode_mp_map(&t->mp_map, D.mp.p, static_cast<int>(t->n_cells));
     if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "tensor map encode failed: %s", cudaGetErrorString(e));
@@ -377,12 +404,6 @@ og::KParams make_params(octgrav_tree* t, float4* out) {
     p.theta_fb2 = static_cast<float>(static_cast<double>(t->theta_fb) * t->theta_fb);
   }
   return p;
-}
-
-// Parts of a list-split launch of t (1: no split): only plain-criterion,
-// cp.async-staged launches that capture no lists split.
-int split_parts(const octgrav_tree* t, bool capture) {
-  return (t->nparts > 1 && !capture && !t->learned && t->stage == og::STAGING_ASYNC) ? t->nparts : 1;
 }
 
 int launch(octgrav_tree* t, double eps, double theta, double G, float4* out, cudaStream_t st,
@@ -800,7 +821,8 @@ int rebuild_items(octgrav_tree* t) {
     t->n_items = res[og::GB_NITEMS];
     t->ordered = true;
     t->host_valid = false;
-    return t->dev->counts.reserve(t->n_items * sizeof(int2));
+    if (int rc = t->dev->counts.reserve(t->n_items * sizeof(int2))) return rc;
+    return reserve_parts(t);
   }
   make_items(t);
   t->uploaded = false;
@@ -1393,12 +1415,14 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   const bool from_device = t->gpu;
   const size_t n = static_cast<size_t>(t->n), nc = static_cast<size_t>(t->n_cells),
                ni = static_cast<size_t>(t->n_items);
+  // a few work items run split, as a launch does until octgrav_set_split is called
+  const int nparts = t->learned ? 1 : auto_parts(t->n_items);
   // arena layout: the device arrays, each starting on a 256-byte boundary
-  const size_t sizes[7] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
+  const size_t sizes[8] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
                            4 * nc * sizeof(float4), ni * sizeof(int4),      4 * ni * sizeof(float4),
-                           t->sysp.size() * sizeof(float4)};
-  size_t offs[7], total = 0;
-  for (int k = 0; k < 7; ++k) {
+                           t->sysp.size() * sizeof(float4), nparts > 1 ? nparts * n * sizeof(float4) : 0};
+  size_t offs[8], total = 0;
+  for (int k = 0; k < 8; ++k) {
     offs[k] = total;
     total += (sizes[k] + 255) & ~static_cast<size_t>(255);
   }
@@ -1449,6 +1473,9 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   p.n_cells = static_cast<int>(nc);
   p.stage = t->stage;
   p.n_group = t->n_group;
+  p.nparts = nparts;
+  p.n = static_cast<int>(n);
+  p.part_out = reinterpret_cast<float4*>(a + offs[7]);
   if (t->learned) {  // the network stays in the tree's own device memory (set_criterion)
     p.mlp = static_cast<const og::MlpDevice*>(t->dev->mlp.p);
     p.theta_lo2 = static_cast<float>(static_cast<double>(t->theta_lo) * t->theta_lo);
@@ -1482,7 +1509,7 @@ int octgrav_graph_capture(octgrav_tree* t, double eps, double theta, double G, f
     if ((rc = t->dev->split.reserve(sizeof(float4) * np * static_cast<size_t>(t->n)))) return rc;
   }
   og::LaunchInfo li;
-  cudaError_t e = og::prepare_walk_eval(t->ppl, t->stage, t->ctas_per_sm, &li);
+  cudaError_t e = og::prepare_walk_eval(t->ppl, t->stage, split_parts(t, false), t->ctas_per_sm, &li);
   if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "kernel preparation failed: %s", cudaGetErrorString(e));
   CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   rc = launch(t, eps, theta, G, reinterpret_cast<float4*>(acc4_dev), st);

@@ -353,7 +353,7 @@ struct octgrav_tree {
   int n_leaf = 0, n_group = 0, n_sys = 0;
   int ppl = 2, ctas_per_sm = 0;
   int fault_stack_cap = 0, fault_drop_item = 0;  // failure injection (octgrav_set_fault; 0 = off)
-  int nparts = 1;  // list split of every work item over this many warps (octgrav_set_split)
+  int nparts = 0;  // list split of every work item over this many warps (octgrav_set_split; 0: auto_parts)
   int stage = og::STAGING_ASYNC;
   bool learned = false;             // learned opening criterion active
   float theta_lo = 0, theta_hi = 0, theta_fb = 0;

@@ -47,8 +47,8 @@ enum : int {
 //   geo   [nc]   float4: boundary cube centre (FP32-rounded) and half side h
 //   link  [nc]   int2:   node -> (first child, number of children 1..8),
 //                        leaf -> (first particle, -count)
-//   mp    [4*nc] float4: q0 = (com_hi.xyz, M), q1 = (com_lo.xyz, T = trS/2),
-//                        q2 = (3Sxx, 3Syy, 3Szz, 3Sxy), q3 = (3Sxz, 3Syz, 3T, 0)
+//   mp    [4*nc] float4: q0 = (com_hi.xyz, M), q1 = (com_lo.xyz, count),
+//                        q2 = (3Sxx, 3Syy, 3Szz, 3Sxy), q3 = (3Sxz, 3Syz, 3T, T = trS/2)
 //   items [ni]   int4:   (root cell of the system, first particle, count, system)
 //   ibox  [4*ni] float4: (gmin.xyz, C_hi.x), (gmax.xyz, C_hi.y), (C_lo.xyz, C_hi.z),
 //                        (first particle, count of the whole group as int bits, 0, 0):
@@ -91,7 +91,7 @@ struct KParams {
   // reports ST_TIMEOUT
   int stack_cap;
   int drop_item;
-  // list split (small systems; 1 = off): work item k is walked by nparts warps,
+  // list split (small systems; <= 1 = off): work item k is walked by nparts warps,
   // part j evaluating the accepted cells and queued leaves whose sequence
   // number is j modulo nparts (part 0 also the group's own particles) into
   // part_out[j * n + particle]; counts are accumulated with atomics
@@ -126,7 +126,7 @@ cudaError_t launch_walk_eval(const KParams& p, int ppl, int ctas_per_sm, bool ca
 
 // Compute (and cache) the launch configuration of a kernel variant without
 // launching it; call before stream capture.
-cudaError_t prepare_walk_eval(int ppl, int stage, int ctas_per_sm, LaunchInfo* info);
+cudaError_t prepare_walk_eval(int ppl, int stage, int nparts, int ctas_per_sm, LaunchInfo* info);
 // out[i] = sum over k of part_out[k * n + i], k = 0 .. nparts - 1 in order
 // (the parts of a list-split launch).
 cudaError_t split_sum(const float4* part_out, int nparts, int n, float4* out, cudaStream_t stream);
@@ -181,7 +181,8 @@ cudaError_t encode_mp_map(CUtensorMap* map, const void* mp, int n_cells);
 
 // Allocation-free launch: like launch_walk_eval, but the status word, the
 // work-queue counter and the per-item counts live in a file-scope device
-// array (no cudaMalloc). p.status, p.work and p.counts are ignored; p.n_items
+// array (no cudaMalloc). p.status, p.work and p.counts are ignored (a list
+// split's part_out is the caller's); p.n_items
 // must not exceed OCTGRAV_NOALLOC_MAX_ITEMS. Waits for the stream and returns
 // the device status bits in *status_bits.
 cudaError_t launch_walk_eval_noalloc(KParams p, int ppl, int ctas_per_sm, cudaStream_t stream,

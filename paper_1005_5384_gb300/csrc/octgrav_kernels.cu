@@ -1276,15 +1276,18 @@ cudaError_t encode_mp_map(CUtensorMap* map, const void* mp, int n_cells) {
 
 size_t walk_eval_smem_bytes() { return sizeof(WarpSmemT<false, false>) * WARPS + 128; }
 
+template <int R, int STAGE>
+cudaError_t launch_s(const KParams& p, int ctas_per_sm, bool capture, cudaStream_t stream, LaunchInfo* info, bool dry) {
+  if (capture) return launch_t<R, STAGE, true>(p, ctas_per_sm, stream, info, dry);
+  return p.nparts > 1 ? launch_t<R, STAGE, false, false, true>(p, ctas_per_sm, stream, info, dry)
+                      : launch_t<R, STAGE, false>(p, ctas_per_sm, stream, info, dry);
+}
+
 template <int STAGE>
-cudaError_t launch_s(const KParams& p, int ppl, int ctas_per_sm, bool capture, cudaStream_t stream,
-                     LaunchInfo* info, bool dry) {
-  if (ppl == 1) {
-    return capture ? launch_t<1, STAGE, true>(p, ctas_per_sm, stream, info, dry)
-                   : launch_t<1, STAGE, false>(p, ctas_per_sm, stream, info, dry);
-  }
-  return capture ? launch_t<2, STAGE, true>(p, ctas_per_sm, stream, info, dry)
-                 : launch_t<2, STAGE, false>(p, ctas_per_sm, stream, info, dry);
+cudaError_t launch_r(const KParams& p, int ppl, int ctas_per_sm, bool capture, cudaStream_t stream, LaunchInfo* info,
+                     bool dry) {
+  return ppl == 1 ? launch_s<1, STAGE>(p, ctas_per_sm, capture, stream, info, dry)
+                  : launch_s<2, STAGE>(p, ctas_per_sm, capture, stream, info, dry);
 }
 
 cudaError_t launch_dispatch(const KParams& p, int ppl, int ctas_per_sm, bool capture, cudaStream_t stream,
@@ -1293,14 +1296,10 @@ cudaError_t launch_dispatch(const KParams& p, int ppl, int ctas_per_sm, bool cap
     return capture ? launch_t<2, STAGE_ASYNC, true, true>(p, ctas_per_sm, stream, info, dry)
                    : launch_t<2, STAGE_ASYNC, false, true>(p, ctas_per_sm, stream, info, dry);
   }
-  if (p.nparts > 1 && !capture && p.stage == STAGE_ASYNC) {  // list split (small systems)
-    return ppl == 1 ? launch_t<1, STAGE_ASYNC, false, false, true>(p, ctas_per_sm, stream, info, dry)
-                    : launch_t<2, STAGE_ASYNC, false, false, true>(p, ctas_per_sm, stream, info, dry);
-  }
   switch (p.stage) {
-    case STAGE_BULK: return launch_s<STAGE_BULK>(p, ppl, ctas_per_sm, capture, stream, info, dry);
-    case STAGE_ASYNC: return launch_s<STAGE_ASYNC>(p, ppl, ctas_per_sm, capture, stream, info, dry);
-    default: return launch_s<STAGE_GATHER4>(p, ppl, ctas_per_sm, capture, stream, info, dry);
+    case STAGE_BULK: return launch_r<STAGE_BULK>(p, ppl, ctas_per_sm, capture, stream, info, dry);
+    case STAGE_ASYNC: return launch_r<STAGE_ASYNC>(p, ppl, ctas_per_sm, capture, stream, info, dry);
+    default: return launch_r<STAGE_GATHER4>(p, ppl, ctas_per_sm, capture, stream, info, dry);
   }
 }
 
@@ -1310,17 +1309,18 @@ cudaError_t launch_walk_eval(const KParams& p, int ppl, int ctas_per_sm, bool ca
 }
 
 namespace {
+// In part order and in FP64 (one rounding): the same sum on every launch.
 __global__ void k_split_sum(const float4* __restrict__ part_out, int nparts, int n, float4* __restrict__ out) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float4 s = part_out[i];
-    for (int k = 1; k < nparts; ++k) {  // in part order: the same sum on every launch
+    double x = 0, y = 0, z = 0, w = 0;
+    for (int k = 0; k < nparts; ++k) {
       const float4 v = part_out[static_cast<size_t>(k) * n + i];
-      s.x += v.x;
-      s.y += v.y;
-      s.z += v.z;
-      s.w += v.w;
+      x += v.x;
+      y += v.y;
+      z += v.z;
+      w += v.w;
     }
-    out[i] = s;
+    out[i] = make_float4(static_cast<float>(x), static_cast<float>(y), static_cast<float>(z), static_cast<float>(w));
   }
 }
 }  // namespace
@@ -1332,9 +1332,10 @@ cudaError_t split_sum(const float4* part_out, int nparts, int n, float4* out, cu
   return cudaGetLastError();
 }
 
-cudaError_t prepare_walk_eval(int ppl, int stage, int ctas_per_sm, LaunchInfo* info) {
+cudaError_t prepare_walk_eval(int ppl, int stage, int nparts, int ctas_per_sm, LaunchInfo* info) {
   KParams p{};
   p.stage = stage;
+  p.nparts = nparts;
   return launch_dispatch(p, ppl, ctas_per_sm, false, nullptr, info, true);
 }
 
@@ -1410,8 +1411,10 @@ cudaError_t launch_walk_eval_noalloc(KParams p, int ppl, int ctas_per_sm, cudaSt
   // the array keeps the previous call's contents: the status word and the
   // work counter must start at zero
   if ((e = cudaMemsetAsync(b, 0, 8, stream)) != cudaSuccess) return e;
+  if (p.nparts > 1 && (e = cudaMemsetAsync(p.counts, 0, sizeof(int2) * p.n_items, stream)) != cudaSuccess) return e;
   if (p.n_items > 0 && (e = launch_walk_eval(p, ppl, ctas_per_sm, false, stream, nullptr)) != cudaSuccess)
     return e;
+  if (p.nparts > 1 && (e = split_sum(p.part_out, p.nparts, p.n, p.out, stream)) != cudaSuccess) return e;
   int h = 0;
   if ((e = cudaMemcpyAsync(&h, b, sizeof(int), cudaMemcpyDeviceToHost, stream)) != cudaSuccess) return e;
   if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return e;
