@@ -17,6 +17,7 @@
 #include <cstring>
 #include <vector>
 
+#include "octgrav_grid.h"
 #include "octgrav_internal.h"
 
 namespace og {
@@ -32,7 +33,6 @@ constexpr int BSUB = 2;           // blocks per chunk in the box pass
 constexpr int LT = 512;           // threads of the level kernel (16 warps) ...
 constexpr int LBMAX = 1024;       // ... and the most blocks it may have
 constexpr int NT = 128;           // threads of the node kernel
-constexpr long long WAIT_LIMIT = 1ll << 31;  // cycles (~1 s) before a grid barrier gives up
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LBINS = 32;  // leaf size bins of the moment pass (32 = "32 or more")
 constexpr int IBINS = 256; // work-item size bins of the default processing order (item_max <= 256)
@@ -170,34 +170,6 @@ __device__ int block_scan_excl(int v, int* total) {
   *total = warp_tot[TB / 32 - 1];
   __syncthreads();  // warp_tot is reused by the next call
   return before + x - v;
-}
-
-// Barrier over all blocks of a cooperative launch: every block adds one to
-// *bar and waits until it reaches `target` (a multiple of the grid size that
-// grows from barrier to barrier). Writes before it are visible to every block
-// after it. False when the wait ran out (all blocks of a cooperative launch
-// are resident, so that would be a lost block); the kernels then stop and
-// leave GPU_BUILD_STUCK in the status word.
-__device__ bool grid_barrier(int* bar, int target, int* status) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int good = 1, v;
-    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(bar) : "memory");
-    const long long t0 = clock64();
-    for (;;) {
-      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if (v >= target) break;
-      if (clock64() - t0 > WAIT_LIMIT) {
-        atomicOr(status, GPU_BUILD_STUCK);
-        good = 0;
-        break;
-      }
-    }
-    ok = good;
-  }
-  __syncthreads();
-  return ok != 0;
 }
 
 // ---------------------------------------------------------------- keys and sort
@@ -642,7 +614,7 @@ __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ c
       if (lane < W) wsum[lane] = x - v;
       if (lane == 31) bsum[blockIdx.x] = x;
     }
-    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS])) {
+    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) {
       no_cells(lvl);
       return;
     }
@@ -713,7 +685,7 @@ __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ c
       }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) lvl[L + 2] = static_cast<int>(next);
-    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS])) {
+    if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) {
       no_cells(lvl);
       return;
     }
@@ -1166,7 +1138,7 @@ __global__ void __launch_bounds__(NT) k_nodes(Cells C, int* lvl, const int* __re
         node_props8(live ? nodes[k] : 0, live, lane & 7, lane & 24, C, ni, P);
       }
     }
-    if (L > 0 && !grid_barrier(&misc[M_BAR_NODES], ++bars * grid, &misc[M_STATUS])) {
+    if (L > 0 && !grid_barrier(&misc[M_BAR_NODES], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) {
       no_cells(lvl);
       return;
     }
@@ -1366,32 +1338,13 @@ int grid_for(int64_t n, int per_block) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16)));
 }
 
-// Blocks of a cooperative launch: as many as the device holds at once, at most
-// `most` (the kernel's blocks wait for one another). 0 on an error.
-template <class K>
-int resident_blocks(K kernel, int threads, int most) {
-  int dev = 0, sms = 0, per = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess)
-    return 0;
-  return std::min(sms * per, most);
-}
-
-template <class... A>
-cudaError_t launch_cooperative(void (*kernel)(A...), int blocks, int threads, cudaStream_t st, A... args) {
-  if (blocks < 1) return cudaErrorInvalidConfiguration;
-  void* argv[] = {&args...};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3(blocks), dim3(threads), argv, 0, st);
-}
-
 // The node kernel: a warp per 4 nodes of a level (a level holds at most n /
 // (n_leaf + 1) nodes) and at most one block per SM: its four warps have a
 // scheduler each, and fewer blocks make cheaper barriers.
 cudaError_t enqueue_nodes(const GpuBuild& a, const Layout& Lo, Cells C, const int* ni, Props P, cudaStream_t st) {
   const int64_t blocks = std::max<int64_t>(1, (a.n / (a.n_leaf + 1) + 15) / 16);
   const int most = static_cast<int>(std::min<int64_t>(blocks, 152));
-  return launch_cooperative(k_nodes, resident_blocks(k_nodes, NT, most), NT, st, C,
+  return launch_cooperative(k_nodes, resident_blocks(k_nodes, NT, most), NT, 0, st, C,
                             at<int>(a.scratch, Lo.lvl),
                             static_cast<const int*>(at<int>(a.scratch, Lo.nlist)), ni, P, at<int>(a.scratch, Lo.misc));
 }
@@ -1523,7 +1476,7 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
     // few blocks, whose barriers are cheaper
     const int64_t want = std::max<int64_t>(1, a.n / (16 * (LT / 32)));
     const int most = static_cast<int>(std::min<int64_t>(want, LBMAX));
-    OG_TRY(launch_cooperative(k_levels, resident_blocks(k_levels, LT, most), LT, st, static_cast<const uint64_t*>(keyA), C,
+    OG_TRY(launch_cooperative(k_levels, resident_blocks(k_levels, LT, most), LT, 0, st, static_cast<const uint64_t*>(keyA), C,
                               a.n_leaf, lvl, spl, lpre, at<int>(S, Lo.nlist), bsum, static_cast<int>(a.cap), misc));
   }
 

@@ -212,6 +212,8 @@ static double splitmix_uniform(uint64_t& s) {
 
 namespace {
 
+constexpr int kTrainSteps = 512;  // training steps of one launch
+
 // One allocation for a call's device arrays, given back when the call ends.
 struct Scratch {
   DevBuf buf;
@@ -244,8 +246,7 @@ int octgrav_mlp_grad(const float* params, const float* x, const float* target, i
   CUDA_TRY(cudaMemcpyAsync(w, params, 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dx, x, 4 * nx, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dt, target, 4 * n, cudaMemcpyHostToDevice, st));
-  cudaError_t e = og::mlp_grad(w, dx, dt, B, B, 0, 0, true, part, st);
-  if (e == cudaSuccess) e = og::mlp_gradient(part, B, g, dl, st);
+  cudaError_t e = og::mlp_gradient(w, dx, dt, B, part, g, dl, st);
   if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "gradient kernel failed: %s", cudaGetErrorString(e));
   float l = 0;
   CUDA_TRY(cudaMemcpyAsync(grad, g, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
@@ -275,11 +276,12 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   const size_t nx = static_cast<size_t>(F) * n;
   Scratch S;
   int rc = S.buf.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + 2 * Scratch::room(n) +
-                         Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) + Scratch::room(1));
+                         Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) +
+                         Scratch::room(2 * kTrainSteps) + Scratch::room(2) + Scratch::room(1));
   if (rc) return rc;
   float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(nx),
         *dlab = S.take(n), *dy = S.take(n), *part = S.take(np), *dstd = S.take(og::MLP_STD_FLOATS), *drec = S.take(4 * F),
-        *dl = S.take(1);
+        *dcoef = S.take(2 * kTrainSteps), *dbar = S.take(2), *dl = S.take(1);
   CUDA_TRY(cudaMemcpyAsync(dx, features, 4 * nx, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dlab, labels, 4 * n, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dw, w.data(), 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
@@ -288,10 +290,22 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
     const cudaError_t e = og::mlp_standardise(dx, dlab, n, dstd, dy, drec, st);
     if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "standardisation failed: %s", cudaGetErrorString(e));
   }
-  for (int k = 1; k <= steps; ++k) {
-    cudaError_t e = og::mlp_grad(dw, dx, dy, static_cast<int>(n), B, k, seed, false, part, st);
-    if (e == cudaSuccess) e = og::mlp_adam(part, B, dw, dm, dv, static_cast<float>(lr), k, dl, st);
-    if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "training kernels failed: %s", cudaGetErrorString(e));
+  // a launch for every 512 steps (a few milliseconds)
+  std::vector<float2> coef(kTrainSteps);
+  for (int k0 = 1; k0 <= steps; k0 += kTrainSteps) {
+    const int nk = std::min(kTrainSteps, steps - k0 + 1);
+    for (int k = 0; k < nk; ++k)
+      coef[k] = make_float2(1.f / (1.f - powf(0.9f, static_cast<float>(k0 + k))),
+                            1.f / (1.f - powf(0.999f, static_cast<float>(k0 + k))));
+    CUDA_TRY(cudaMemcpyAsync(dcoef, coef.data(), sizeof(float2) * nk, cudaMemcpyHostToDevice, st));
+    const cudaError_t e = og::mlp_train_steps(dw, dm, dv, dx, dy, static_cast<int>(n), B, k0, nk, seed,
+                                              static_cast<float>(lr), reinterpret_cast<const float2*>(dcoef), part, dl,
+                                              reinterpret_cast<int*>(dbar), st);
+    if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "training kernel failed: %s", cudaGetErrorString(e));
+    int stuck = 0;
+    CUDA_TRY(cudaMemcpyAsync(&stuck, reinterpret_cast<int*>(dbar) + 1, 4, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    if (stuck) return fail(OCTGRAV_ERR_TIMEOUT, "a training step's barrier timed out");
   }
   float l = 0, stats[4 * og::MLP_NF];
   CUDA_TRY(cudaMemcpyAsync(stats, drec, sizeof stats, cudaMemcpyDeviceToHost, st));

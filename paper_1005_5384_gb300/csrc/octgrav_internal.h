@@ -163,17 +163,19 @@ cudaError_t mlp_sample_labels(const MlpSampleArgs& a, cudaStream_t st);
 // floats, 8-byte aligned.
 cudaError_t mlp_standardise(float* feat, const float* label, int64_t n, float* scratch, float* y, float* record,
                             cudaStream_t st);
-// A training step's gradient in two launches. mlp_grad writes the shares of
-// mlp_blocks(B) blocks to part (MLP_PART floats each); use_all: the B samples
-// are X[0..B) instead of B counter-based draws. mlp_gradient adds them into
-// grad and loss; mlp_adam adds them and updates the parameters, and writes the
-// step's loss.
+// Gradient of sum (y - t)^2 / (2 n) at w over the n samples X (grad, loss). part:
+// mlp_blocks(n) shares of MLP_PART floats.
 int mlp_blocks(int B);
-cudaError_t mlp_grad(const float* w, const float* X, const float* t, int n_total, int B, int step, uint64_t seed,
-                     bool use_all, float* part, cudaStream_t st);
-cudaError_t mlp_gradient(const float* part, int B, float* grad, float* loss, cudaStream_t st);
-cudaError_t mlp_adam(const float* part, int B, float* w, float* m, float* v, float lr, int step, float* loss,
-                     cudaStream_t st);
+cudaError_t mlp_gradient(const float* w, const float* X, const float* t, int n, float* part, float* grad, float* loss,
+                         cudaStream_t st);
+// Training steps step0 .. step0 + steps - 1 (counter-based draws of B of the
+// n_total samples each) in one cooperative launch; coef[k] = the Adam bias
+// corrections of step step0 + k. loss gets the last step's loss. part:
+// mlp_blocks(B) shares; bar: two ints, the second one non-zero afterwards if a
+// barrier's bounded wait ran out.
+cudaError_t mlp_train_steps(float* w, float* m, float* v, const float* X, const float* t, int n_total, int B, int step0,
+                            int steps, uint64_t seed, float lr, const float2* coef, float* part, float* loss, int* bar,
+                            cudaStream_t st);
 
 // Encode the 2-D tensor map over a cell-record array (n_cells rows of 64 B)
 // used by the gather4 staging. Returns cudaSuccess or an error.

@@ -12,6 +12,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "octgrav_grid.h"
 #include "octgrav_internal.h"
 #include "octgrav_mlp.h"
 
@@ -241,12 +242,11 @@ __device__ __forceinline__ void fma8(float* z, const float4* w, float x) {
 // samples in registers and over the block's tiles, and written once: no
 // atomics, so a step's result does not depend on scheduling. One output per thread with
 // W2[j][i] read at a stride of 64 floats put all 32 lanes on one bank:
-// 43 us a step at B = 4096, 17 us now (both with the parameter update).
-__global__ void __launch_bounds__(GT) grad_kernel(const float* __restrict__ w, const float* __restrict__ X,
-                                                   const float* __restrict__ t, int n_total, int B, int step,
-                                                   uint64_t seed, int use_all, float* __restrict__ part) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  GradSmem& S = *reinterpret_cast<GradSmem*>(smem);
+// 43 us a step at B = 4096, 17 us so (both with the parameter update as a second
+// launch).
+__device__ __forceinline__ void block_gradient(GradSmem& S, const float* w, const float* __restrict__ X,
+                                               const float* __restrict__ t, int n_total, int B, int step,
+                                               uint64_t seed, int use_all, float* __restrict__ part) {
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const float* b1 = w + MLP_NH * MLP_NF;
   const float* W2 = b1 + MLP_NH;
@@ -255,16 +255,16 @@ __global__ void __launch_bounds__(GT) grad_kernel(const float* __restrict__ w, c
   float* w1t = reinterpret_cast<float*>(S.w1t);
   float* w2t = reinterpret_cast<float*>(S.w2t);
   float* w2s = reinterpret_cast<float*>(S.w2);
-  for (int k = tid; k < MLP_NH * MLP_NF; k += GT) w1t[(k % MLP_NF) * MLP_NH + k / MLP_NF] = w[k];
-  for (int k = tid; k < MLP_NH * MLP_NH; k += GT) w2s[(k / MLP_NH) * RS + k % MLP_NH] = W2[k];
+  for (int k = tid; k < MLP_NH * MLP_NF; k += GT) w1t[(k % MLP_NF) * MLP_NH + k / MLP_NF] = __ldcg(w + k);
+  for (int k = tid; k < MLP_NH * MLP_NH; k += GT) w2s[(k / MLP_NH) * RS + k % MLP_NH] = __ldcg(W2 + k);
   __syncthreads();
   for (int k = tid; k < MLP_NH * MLP_NH; k += GT) w2t[k] = w2s[(k % MLP_NH) * RS + k / MLP_NH];
   if (tid < MLP_NH) {
-    S.b1[tid] = b1[tid];
-    S.b2[tid] = b2[tid];
-    S.w3[tid] = w3[tid];
+    S.b1[tid] = __ldcg(b1 + tid);
+    S.b2[tid] = __ldcg(b2 + tid);
+    S.w3[tid] = __ldcg(w3 + tid);
   }
-  if (tid == 0) S.b3 = w3[MLP_NH];
+  if (tid == 0) S.b3 = __ldcg(w3 + MLP_NH);
   const float invB = 1.f / static_cast<float>(B);
   const int u0 = 8 * wp;                                // this warp's units
   const int ja = 4 * (tid >> 4), ib = 4 * (tid & 15);   // this thread's 4 x 4 tile of W2's gradient
@@ -406,12 +406,17 @@ __global__ void __launch_bounds__(GT) grad_kernel(const float* __restrict__ w, c
   else if (tid < 3 * MLP_NH + 2) o2[MLP_NH * MLP_NH + tid - MLP_NH] = gb;  // b2, w3, b3, L follow each other
 }
 
-// Sum of the blocks' shares per parameter (and of L), then the Adam update
-// (w != NULL) or the gradient and L themselves. A block takes 32 parameters:
-// warp s adds the shares s, s + 8, ..., the warps' sums are added in order.
-__global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ part, int blocks, float* __restrict__ w,
-                                                      float* __restrict__ m, float* __restrict__ v, float lr, float c1,
-                                                      float c2, float* __restrict__ grad, float* __restrict__ loss) {
+__global__ void __launch_bounds__(GT) grad_kernel(const float* w, const float* __restrict__ X,
+                                                   const float* __restrict__ t, int n, float* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  block_gradient(*reinterpret_cast<GradSmem*>(smem), w, X, t, n, n, 0, 0, 1, part);
+}
+
+// Sum of the blocks' shares per parameter, and of L. A block takes 32
+// parameters: warp s adds the shares s, s + 8, ..., the warps' sums are added in
+// order.
+__global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ part, int blocks,
+                                                      float* __restrict__ grad, float* __restrict__ loss) {
   __shared__ float sum[8][32];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, k = 32 * blockIdx.x + lane;
   float s = 0.f;
@@ -425,19 +430,60 @@ __global__ void __launch_bounds__(256) reduce_kernel(const float* __restrict__ p
   float g = 0.f;
 #pragma unroll
   for (int q = 0; q < 8; ++q) g += sum[q][lane];
-  if (k == MLP_NPARAM) {
-    *loss = g;
-    return;
+  if (k == MLP_NPARAM) *loss = g;
+  else grad[k] = g;
+}
+
+// `steps` training steps in one cooperative launch. Per step: every block's
+// share of the gradient, a grid barrier, then the blocks add the shares of
+// their range of parameters (a thread per parameter and slice of the shares,
+// the slices in order) and apply the Adam update, and a second barrier. coef
+// holds the steps' bias corrections 1 / (1 - 0.9^k) and 1 / (1 - 0.999^k).
+//
+// A step is a chain of short dependent phases, so what it waits for between
+// them counts: as two launches it took 17 us at B = 4096, 14 us so.
+__global__ void __launch_bounds__(GT) train_kernel(float* w, float* m, float* v, const float* __restrict__ X,
+                                                    const float* __restrict__ t, int n_total, int B, int step0,
+                                                    int steps, uint64_t seed, float lr,
+                                                    const float2* __restrict__ coef, float* part,
+                                                    float* loss, int* bar) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  GradSmem& S = *reinterpret_cast<GradSmem*>(smem);
+  float* sum = reinterpret_cast<float*>(S.h1);  // free between the gradients
+  const int grid = gridDim.x, tid = threadIdx.x;
+  const int per = (MLP_NPARAM + 1 + grid - 1) / grid;      // parameters of a block (the last is L)
+  const int k0 = min(MLP_NPARAM + 1, static_cast<int>(blockIdx.x) * per), nk = min(MLP_NPARAM + 1 - k0, per);
+  const int slices = max(1, GT / per);
+  int bars = 0;
+  for (int k = 0; k < steps; ++k) {
+    block_gradient(S, w, X, t, n_total, B, step0 + k, seed, 0, part);
+    if (!grid_barrier(bar, ++bars * grid, bar + 1, 1)) return;
+    const float2 c = coef[k];
+    for (int e0 = 0; e0 < nk; e0 += GT) {  // one round unless the grid is tiny
+      const int e = e0 + (slices > 1 ? tid % per : tid), q = slices > 1 ? tid / per : 0;
+      float s = 0.f;
+      if (e < nk && q < slices) {
+#pragma unroll 8
+        for (int b = q; b < grid; b += slices) s += __ldcg(part + static_cast<size_t>(b) * MLP_PART + k0 + e);
+        if (slices > 1) sum[q * per + e] = s;
+      }
+      if (slices > 1) __syncthreads();
+      if (e < nk && q == 0) {
+        for (int r = 1; r < slices; ++r) s += sum[r * per + e];
+        const int p = k0 + e;
+        if (p == MLP_NPARAM) {
+          *loss = s;
+        } else {
+          const float mk = 0.9f * m[p] + 0.1f * s;
+          const float vk = 0.999f * v[p] + 0.001f * s * s;
+          m[p] = mk;
+          v[p] = vk;
+          w[p] -= lr * (mk * c.x) / (sqrtf(vk * c.y) + 1e-8f);
+        }
+      }
+    }
+    if (!grid_barrier(bar, ++bars * grid, bar + 1, 1)) return;
   }
-  if (!w) {
-    grad[k] = g;
-    return;
-  }
-  const float mk = 0.9f * m[k] + 0.1f * g;
-  const float vk = 0.999f * v[k] + 0.001f * g * g;
-  m[k] = mk;
-  v[k] = vk;
-  w[k] -= lr * (mk * c1) / (sqrtf(vk * c2) + 1e-8f);
 }
 
 }  // namespace
@@ -473,26 +519,23 @@ int mlp_blocks(int B) {
   return tiles < 2 * 152 ? tiles : 2 * 152;
 }
 
-cudaError_t mlp_grad(const float* w, const float* X, const float* t, int n_total, int B, int step, uint64_t seed,
-                     bool use_all, float* part, cudaStream_t st) {
+cudaError_t mlp_gradient(const float* w, const float* X, const float* t, int n, float* part, float* grad, float* loss,
+                         cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem));
   if (e != cudaSuccess) return e;
-  grad_kernel<<<mlp_blocks(B), GT, sizeof(GradSmem), st>>>(w, X, t, n_total, B, step, seed, use_all ? 1 : 0, part);
+  grad_kernel<<<mlp_blocks(n), GT, sizeof(GradSmem), st>>>(w, X, t, n, part);
+  reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(part, mlp_blocks(n), grad, loss);
   return cudaGetLastError();
 }
 
-cudaError_t mlp_gradient(const float* part, int B, float* grad, float* loss, cudaStream_t st) {
-  reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(part, mlp_blocks(B), nullptr, nullptr, nullptr, 0.f, 0.f, 0.f,
-                                                            grad, loss);
-  return cudaGetLastError();
-}
-
-cudaError_t mlp_adam(const float* part, int B, float* w, float* m, float* v, float lr, int step, float* loss,
-                     cudaStream_t st) {
-  const float c1 = 1.f / (1.f - powf(0.9f, static_cast<float>(step)));
-  const float c2 = 1.f / (1.f - powf(0.999f, static_cast<float>(step)));
-  reduce_kernel<<<(MLP_NPARAM + 1 + 31) / 32, 256, 0, st>>>(part, mlp_blocks(B), w, m, v, lr, c1, c2, nullptr, loss);
-  return cudaGetLastError();
+cudaError_t mlp_train_steps(float* w, float* m, float* v, const float* X, const float* t, int n_total, int B, int step0,
+                            int steps, uint64_t seed, float lr, const float2* coef, float* part, float* loss, int* bar,
+                            cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(GradSmem));
+  if (e != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(bar, 0, 8, st)) != cudaSuccess) return e;
+  return launch_cooperative(train_kernel, resident_blocks(train_kernel, GT, mlp_blocks(B), sizeof(GradSmem)), GT,
+                            sizeof(GradSmem), st, w, m, v, X, t, n_total, B, step0, steps, seed, lr, coef, part, loss, bar);
 }
 
 }  // namespace og

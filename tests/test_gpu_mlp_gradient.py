@@ -32,3 +32,17 @@ def test_gradient_at_tile_and_grid_edges(n):
     assert abs(loss - loss64) <= 2e-5 * abs(loss64)
     g2, loss2 = G.mlp_grad(w, x, t)
     assert np.array_equal(g.view(np.uint32), g2.view(np.uint32)) and loss == loss2
+
+
+@pytest.mark.parametrize("batch,steps", [(40, 3), (1000, 513), (20000, 20)])
+def test_training_is_reproducible_and_lowers_the_loss(batch, steps):
+    """Few blocks with many parameters each, a launch boundary (512 steps), and
+    several tiles per block: the same record twice, a loss below the first's."""
+    rng = np.random.default_rng(5)
+    f = rng.standard_normal((30000, 12)).astype(np.float32)
+    label = (10.0 ** (-3.0 + 0.3 * f[:, 0] - 0.2 * f[:, 3])).astype(np.float32)
+    first = G.mlp_train(f, label, steps=1, batch=batch, seed=7)
+    a = G.mlp_train(f, label, steps=steps, batch=batch, seed=7)
+    b = G.mlp_train(f, label, steps=steps, batch=batch, seed=7)
+    assert np.array_equal(a[0].view(np.uint32), b[0].view(np.uint32)) and a[1] == b[1]
+    assert np.all(np.isfinite(a[0])) and a[1] < first[1]
