@@ -47,8 +47,8 @@ struct Chunk {  // TILE particles (or fewer) of one system
 };
 
 // misc[] slots (int), zeroed before a build: counts, status bits, arrivals at
-// the grid barriers of the level and the node kernel, nodes per level
-enum { M_NGROUPS = 0, M_NITEMS, M_NLEAVES, M_MAXGROUP, M_STATUS, M_BAR_LEVELS, M_BAR_NODES, M_NODES };
+// the grid barriers of the sort, the level and the node kernel, nodes per level
+enum { M_NGROUPS = 0, M_NITEMS, M_NLEAVES, M_MAXGROUP, M_STATUS, M_BAR_SORT, M_BAR_LEVELS, M_BAR_NODES, M_NODES };
 constexpr int MISC = M_NODES + NLEV;
 
 // Scratch layout (byte offsets into one allocation).
@@ -138,10 +138,6 @@ __device__ __forceinline__ long long order_key(double x) {
 // wins ties, so signed zeros come out as on the host)
 __device__ __forceinline__ double lesser(double a, double b) { return order_key(b) < order_key(a) ? b : a; }
 __device__ __forceinline__ double greater(double a, double b) { return order_key(a) < order_key(b) ? b : a; }
-
-__device__ __forceinline__ int octant_at(uint64_t code, int child_depth) {
-  return static_cast<int>((code >> (3 * (MAXD - child_depth))) & 7);
-}
 
 // Exclusive block-wide scan of one int per thread (TB threads); returns the
 // exclusive prefix and writes the block total to *total.
@@ -369,9 +365,46 @@ __global__ void __launch_bounds__(TB) k_scan_digits(int* __restrict__ cnt, const
   if (lane == 0) dtot[seg] = run;
 }
 
-// Stable scatter of one chunk by the digit at `shift`: warp w ranks its 512
-// elements round by round (32 at a time, in order), the warps' counts are
-// combined in warp order, and the chunk's offsets come from the scan.
+// Stable ranks of one chunk's keys by the digit at `shift`: warp w ranks its
+// 512 elements round by round (32 at a time, in order); afterwards wc[w][d] is
+// the number of elements of digit d in the warps before, and an element's place
+// among its chunk's digit is wc[w][d] + rk. Returns the chunk's count of digit
+// threadIdx.x.
+__device__ __forceinline__ int chunk_ranks(const uint64_t* kin, const uint32_t* vin, const Chunk& c, int shift,
+                                           int (*wc)[257], uint64_t* kk, uint32_t* vv, int* rk) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int r = 0; r < IPT; ++r) {
+    const int e = w * (32 * IPT) + r * 32 + lane;
+    const bool ok = e < c.count;
+    kk[r] = ok ? __ldcg(kin + c.first + e) : 0ull;
+    vv[r] = ok ? __ldcg(vin + c.first + e) : 0u;
+  }
+#pragma unroll
+  for (int r = 0; r < IPT; ++r) {
+    const int e = w * (32 * IPT) + r * 32 + lane;
+    const int d = e < c.count ? static_cast<int>((kk[r] >> shift) & 255) : 256;
+    const unsigned peers = __match_any_sync(FULL, d);
+    const int before = wc[w][d];
+    rk[r] = before + __popc(peers & lt);
+    __syncwarp();
+    if (lane == __ffs(peers) - 1) wc[w][d] = before + __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  int run = 0;  // warp offsets per digit
+  for (int q = 0; q < TB / 32; ++q) {
+    const int t = wc[q][threadIdx.x];
+    wc[q][threadIdx.x] = run;
+    run += t;
+  }
+  __syncthreads();
+  return run;
+}
+
+// Stable scatter of one chunk by the digit at `shift`; the chunk's offsets come
+// from the scan.
 __global__ void __launch_bounds__(TB) k_downsweep(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                   uint64_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                   const Chunk* __restrict__ ch, int shift,
@@ -379,7 +412,6 @@ __global__ void __launch_bounds__(TB) k_downsweep(const uint64_t* __restrict__ k
   __shared__ int wc[TB / 32][257];  // per-warp digit counters (+ one for empty slots)
   __shared__ int goff[256];
   const Chunk c = ch[blockIdx.x];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int k = threadIdx.x; k < (TB / 32) * 257; k += TB) (&wc[0][0])[k] = 0;
   {  // destination of this chunk's first element of each digit
     int unused;
@@ -390,41 +422,70 @@ __global__ void __launch_bounds__(TB) k_downsweep(const uint64_t* __restrict__ k
   uint64_t kk[IPT];
   uint32_t vv[IPT];
   int rk[IPT];
-  const unsigned lt = (1u << lane) - 1u;
+  chunk_ranks(kin, vin, c, shift, wc, kk, vv, rk);
 #pragma unroll
   for (int r = 0; r < IPT; ++r) {
-    const int e = w * (32 * IPT) + r * 32 + lane;
-    const bool ok = e < c.count;
-    kk[r] = ok ? kin[c.first + e] : 0ull;
-    vv[r] = ok ? vin[c.first + e] : 0u;
-    const int d = ok ? static_cast<int>((kk[r] >> shift) & 255) : 256;
-    const unsigned peers = __match_any_sync(FULL, d);
-    const int before = wc[w][d];
-    rk[r] = before + __popc(peers & lt);
-    __syncwarp();
-    if (lane == __ffs(peers) - 1) wc[w][d] = before + __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  {  // warp offsets per digit
-    const int d = threadIdx.x;
-    int run = 0;
-    for (int q = 0; q < TB / 32; ++q) {
-      const int t = wc[q][d];
-      wc[q][d] = run;
-      run += t;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < IPT; ++r) {
-    const int e = w * (32 * IPT) + r * 32 + lane;
+    const int e = (threadIdx.x >> 5) * (32 * IPT) + r * 32 + (threadIdx.x & 31);
     if (e < c.count) {
       const int d = static_cast<int>((kk[r] >> shift) & 255);
-      const int dst = goff[d] + wc[w][d] + rk[r];
+      const int dst = goff[d] + wc[threadIdx.x >> 5][d] + rk[r];
       kout[dst] = kk[r];
       vout[dst] = vv[r];
     }
+  }
+}
+
+// All eight passes in one cooperative launch, a block per chunk: ranks, the
+// chunk's digit counts, a grid barrier, offsets (every block adds the counts of
+// its system's chunks itself, a thread per digit), scatter, a second barrier.
+// The same order as the passes by three launches each, whose gaps and short
+// grids made up most of the time of a small sort: from the keys to the gather
+// 157 us at 5000 particles, 83 us so. The sums over the chunks grow with their
+// number: 163 and 93 us at 65,536 particles, 159 and 103 us at 64 chunks
+// (262,144), which is where the rule ends.
+constexpr int SORT_CHUNKS = 64;
+
+__global__ void __launch_bounds__(TB) k_sort(uint64_t* keyA, uint32_t* valA, uint64_t* keyB, uint32_t* valB,
+                                             const Chunk* __restrict__ ch, int* cnt, int* misc) {
+  __shared__ int wc[TB / 32][257];
+  __shared__ int goff[256];
+  const Chunk c = ch[blockIdx.x];
+  const int first = ch[c.cs].first, grid = gridDim.x, mine = blockIdx.x;
+  int bars = 0;
+  for (int pass = 0; pass < 8; ++pass) {
+    const int shift = 8 * pass;
+    const bool even = (pass & 1) == 0;
+    for (int k = threadIdx.x; k < (TB / 32) * 257; k += TB) (&wc[0][0])[k] = 0;
+    __syncthreads();
+    uint64_t kk[IPT];
+    uint32_t vv[IPT];
+    int rk[IPT];
+    cnt[256 * mine + threadIdx.x] =
+        chunk_ranks(even ? keyA : keyB, even ? valA : valB, c, shift, wc, kk, vv, rk);
+    if (!grid_barrier(&misc[M_BAR_SORT], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) return;
+    int before = 0, total = 0;
+#pragma unroll 8
+    for (int j = c.cs; j < c.cs + c.nbs; ++j) {
+      const int v = __ldcg(&cnt[256 * j + threadIdx.x]);
+      total += v;
+      before += j < mine ? v : 0;
+    }
+    int unused;
+    goff[threadIdx.x] = first + block_scan_excl(total, &unused) + before;
+    __syncthreads();
+    uint64_t* kout = even ? keyB : keyA;
+    uint32_t* vout = even ? valB : valA;
+#pragma unroll
+    for (int r = 0; r < IPT; ++r) {
+      const int e = (threadIdx.x >> 5) * (32 * IPT) + r * 32 + (threadIdx.x & 31);
+      if (e < c.count) {
+        const int d = static_cast<int>((kk[r] >> shift) & 255);
+        const int dst = goff[d] + wc[threadIdx.x >> 5][d] + rk[r];
+        kout[dst] = kk[r];
+        vout[dst] = vv[r];
+      }
+    }
+    if (pass < 7 && !grid_barrier(&misc[M_BAR_SORT], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) return;
   }
 }
 
@@ -474,16 +535,18 @@ __global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, in
 // Split points of a cell holding particles [f, f + cnt): sp[o] = the first
 // position whose child octant at depth D is >= o, sp[0] = f, sp[8] = f + cnt
 // (octants ascend inside a cell). One warp; every lane returns the same sp.
-// The seven boundaries are searched together: a round probes 32 evenly spaced
-// positions of each one's interval with seven independent loads per lane, so a
-// cell of a million particles takes four rounds of load latency and one of at
-// most 32 particles a single load (one boundary after the other took seven
-// times as many rounds).
+// The seven boundaries are searched together: a round probes 32 positions a
+// power of two apart of each one's interval, seven independent loads per lane,
+// so a cell of a million particles takes four rounds of load latency, one of at
+// most 1024 two and one of at most 32 a single load. (One boundary after the
+// other took seven times as many rounds; probes at 33rds of the intervals
+// spent 10 us of a level on their 64-bit divisions.)
 __device__ void warp_split(const uint64_t* __restrict__ code, int f, int cnt, int D, int lane, int* sp) {
+  const int bit = 3 * (MAXD - D);
   sp[0] = f;
   sp[8] = f + cnt;
   if (cnt <= 32) {  // one probe per particle
-    const int oc = lane < cnt ? octant_at(code[f + lane], D) : 8;
+    const int oc = lane < cnt ? static_cast<int>(code[f + lane] >> bit) & 7 : 8;
 #pragma unroll
     for (int o = 1; o < 8; ++o) {
       const unsigned m = __ballot_sync(FULL, oc >= o);
@@ -492,41 +555,32 @@ __device__ void warp_split(const uint64_t* __restrict__ code, int f, int cnt, in
     return;
   }
   // invariant: boundary o lies in [a[o], b[o]], and b[o] is the end or a known hit
-  int a[8], b[8], span = cnt;
+  int a[8], b[8];
 #pragma unroll
   for (int o = 1; o < 8; ++o) {
     a[o] = f;
     b[o] = f + cnt;
   }
-  while (span > 32) {
+  int sh = max(0, 32 - __clz(cnt - 1) - 5);  // 32 probes 2^sh apart cover the interval
+  for (;;) {
+    const int off = lane << sh;
     int oc[8];
 #pragma unroll
-    for (int o = 1; o < 8; ++o) {
-      const int64_t w = b[o] - a[o];
-      const int p = a[o] + static_cast<int>((lane + 1) * w / 33);
-      oc[o] = p < b[o] ? octant_at(code[p], D) : 8;
-    }
-    span = 0;
+    for (int o = 1; o < 8; ++o)
+      oc[o] = off < b[o] - a[o] ? static_cast<int>(code[a[o] + off] >> bit) & 7 : 8;
 #pragma unroll
     for (int o = 1; o < 8; ++o) {
-      const int64_t w = b[o] - a[o];
-      const unsigned m = __ballot_sync(FULL, oc[o] >= o);
+      const unsigned m = __ballot_sync(FULL, oc[o] >= o);  // a probe beyond the end is a hit
       const int k = m ? __ffs(m) - 1 : 32;
-      const int lo = k == 0 ? a[o] : min(b[o], a[o] + static_cast<int>(k * w / 33) + 1);
-      const int hi = k == 32 ? b[o] : min(b[o], a[o] + static_cast<int>((k + 1) * w / 33));
-      a[o] = lo;
+      const int hi = k == 32 ? b[o] : min(b[o], a[o] + (k << sh));
+      a[o] = k == 0 ? a[o] : min(b[o], a[o] + ((k - 1) << sh) + 1);
       b[o] = hi;
-      span = max(span, hi - lo);
     }
+    if (sh == 0) break;
+    sh = max(0, sh - 5);
   }
-  int oc[8];
 #pragma unroll
-  for (int o = 1; o < 8; ++o) oc[o] = a[o] + lane < b[o] ? octant_at(code[a[o] + lane], D) : 8;
-#pragma unroll
-  for (int o = 1; o < 8; ++o) {
-    const unsigned m = __ballot_sync(FULL, oc[o] >= o && a[o] + lane < b[o]);
-    sp[o] = m ? a[o] + __ffs(m) - 1 : b[o];
-  }
+  for (int o = 1; o < 8; ++o) sp[o] = b[o];
 }
 
 // After a barrier that ran out: a tree without cells, which the rest of the
@@ -557,6 +611,10 @@ __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ c
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grid = gridDim.x;
   const unsigned lt = (1u << lane) - 1u;
   int lb = lvl[0], le = lvl[1], bars = 0;
+  if (__ldcg(&misc[M_STATUS]) & GPU_BUILD_STUCK) {  // the sort did not finish
+    no_cells(lvl);
+    return;
+  }
   for (int L = 0; L < MAXD; ++L) {
     const int nl = le - lb;
     // cells per warp; block b's warps take consecutive ranges of its range
@@ -1456,15 +1514,20 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
   k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, dch, part, misc);
   k_root<<<a.n_sys, TB, 0, st>>>(part, dchunk0, sg);
   k_morton<<<SUB * nch, TB, 0, st>>>(a.pos, dch, sg, keyA, valA);
-  int* dtot = at<int>(S, Lo.dtot);
-  const int segblocks = (256 * a.n_sys + TB / 32 - 1) / (TB / 32);
-  for (int pass = 0; pass < 8; ++pass) {
-    const int sh = 8 * pass;
-    const bool even = (pass & 1) == 0;
-    k_upsweep<<<nch, TB, 0, st>>>(even ? keyA : keyB, dch, sh, cnt);
-    k_scan_digits<<<segblocks, TB, 0, st>>>(cnt, dchunk0, a.n_sys, dtot);
-    k_downsweep<<<nch, TB, 0, st>>>(even ? keyA : keyB, even ? valA : valB, even ? keyB : keyA,
-                                    even ? valB : valA, dch, sh, cnt, dtot);
+  if (nch <= SORT_CHUNKS && resident_blocks(k_sort, TB, nch) == nch) {
+    const Chunk* chunks = dch;
+    OG_TRY(launch_cooperative(k_sort, nch, TB, 0, st, keyA, valA, keyB, valB, chunks, cnt, misc));
+  } else {
+    int* dtot = at<int>(S, Lo.dtot);
+    const int segblocks = (256 * a.n_sys + TB / 32 - 1) / (TB / 32);
+    for (int pass = 0; pass < 8; ++pass) {
+      const int sh = 8 * pass;
+      const bool even = (pass & 1) == 0;
+      k_upsweep<<<nch, TB, 0, st>>>(even ? keyA : keyB, dch, sh, cnt);
+      k_scan_digits<<<segblocks, TB, 0, st>>>(cnt, dchunk0, a.n_sys, dtot);
+      k_downsweep<<<nch, TB, 0, st>>>(even ? keyA : keyB, even ? valA : valB, even ? keyB : keyA,
+                                      even ? valB : valA, dch, sh, cnt, dtot);
+    }
   }
   OG_TRY(cudaGetLastError());
   k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(valA, a.pos, a.mass, a.n, xs, ms, a.parts, a.perm);

@@ -1,7 +1,7 @@
 """The level and node kernels of the GPU build where their rules change: cells
 of 32 and 33 particles (one probe per particle or a search), levels that end at
-the depth limit, trees of one block and of many, and more nodes on a level than
-eight-lane groups take. Byte equality with the host build throughout."""
+the depth limit, trees of one block and of many, more nodes on a level than
+eight-lane groups take, and the most chunks that are sorted in one launch. Byte equality with the host build throughout."""
 import numpy as np
 import pytest
 
@@ -66,3 +66,24 @@ def test_more_nodes_on_a_level_than_eight_lane_groups_take():
     depth = np.floor(np.log2(B.cell_keys().astype(np.float64)) / 3)
     counts = B.cell_props()["count"]
     assert max(int(np.sum((depth == d) & (counts > 1))) for d in range(22)) > 4 * 4 * 608
+
+
+@pytest.mark.parametrize("n", [64 * 4096, 64 * 4096 + 1])
+def test_sort_in_one_launch_and_in_passes(n):
+    """The last size that one launch sorts and the first that it does not."""
+    rng = np.random.default_rng(n)
+    _same(rng.random((n, 3)) ** 3, rng.random(n), 16, 64)
+
+
+@pytest.mark.parametrize("sizes", [[1, 4096, 4097, 2, 9000], [64] * 64, [64] * 65])
+def test_sort_of_several_systems(sizes):
+    """Every system is sorted by itself, whatever its number of chunks; 64 chunks
+    take the one launch and 65 do not."""
+    rng = np.random.default_rng(len(sizes))
+    systems = [(rng.random((k, 3)), rng.random(k)) for k in sizes]
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    A = G.Tree.build_batch(systems, 8, 32)
+    B = G.Tree.build_gpu(np.concatenate([p for p, _ in systems]), np.concatenate([m for _, m in systems]), 8, 32,
+                         offsets=offs)
+    assert A.stats == B.stats
+    assert np.array_equal(A.perm(), B.perm()) and np.array_equal(A.cell_keys(), B.cell_keys())
