@@ -483,8 +483,8 @@ int octgrav_set_fault(octgrav_tree *t, int stack_cap, int64_t drop_item);
  * (part 0 also the group's own particles), and the parts' results are summed
  * in part order by a second kernel, so a launch is deterministic but rounds
  * differently from an unsplit one (a sum of nparts FP32 results). Until this is
- * called a tree of at most 2550 work items is split over 2, 4 or 8 warps by
- * their number. Applies to launches with the plain opening test that capture no
+ * called a tree of at most 3200 work items is split over 2, 4 or 8 warps by
+ * their number and the particles in each. Applies to launches with the plain opening test that capture no
  * lists; others run unsplit. Errors: ERR_ARG. */
 int octgrav_set_split(octgrav_tree *t, int nparts);
 

@@ -296,16 +296,26 @@ int build_oneshot(const double* pos, const double* mass, int64_t n, int n_leaf, 
 }
 
 
-// Parts that fill the GPU's 2432 warp slots for a system of few work items:
-// the largest power of two up to 8 that keeps items x parts within 2.1 times
-// the slots (every part repeats the item's walk, so more parts than that cost
-// more than the shorter evaluation gains). Times by parts 1 / 2 / 4 / 8 (us,
-// theta 0.5 to 0.7): 112 items 48 / 37 / 28 / 26, 340 150 / 100 / 74 / 62, 688
-// 195 / 140 / 107 / 127, 1111 448 / 346 / 309 / 411, 2516 504 / 389 / 498 / 727.
-int auto_parts(int64_t n_items) {
-  int parts = 8;
-  while (parts > 1 && n_items * parts > 5100) parts /= 2;
-  return parts;
+// Parts that fill the GPU's 2432 warp slots for a tree of few work items. Every
+// part repeats the item's walk, so a split pays where the evaluation outweighs
+// it: with many particles per item and long lists. Times of 1 / 2 / 4 / 8 parts
+// (us, theta 0.6):
+//   26 particles an item   92 items  69 / 51 / 39 / 34    652 222 / 162 / 148 / 161
+//                        1253 315 / 281 / 239 / 332      2770 521 / 432 / 558 / 824
+//   15                    318 142 / 96 / 74 / 62         2317 283 / 257 / 344 / 517
+//   8.5                   190  41 / 36 / 31 / 34         1254 124 / 122 / 121 / 184
+//                        2475 170 / 181 / 254 / 407
+//   5                     305  33 / 34 / 33 / 37         1235  69 / 75 / 93 / 144
+// The limits on items x parts are those of 19 and more particles an item (at
+// 3236 items two parts gain 1.10x, at 3550 they lose 3 %); with fewer they fall
+// in proportion, and below 6 particles an item or 1000 a system there is no
+// split (550 particles in 79 items: 23 us alone, 28 in eight parts).
+int auto_parts(const octgrav_tree* t) {
+  const int64_t items = t->n_items;
+  if (t->n < 6 * items || t->n < 1000 * static_cast<int64_t>(t->n_sys)) return 1;
+  const double fill = std::min(1.0, static_cast<double>(t->n) / (19.0 * static_cast<double>(items)));
+  const auto fits = [&](int parts, int most) { return static_cast<double>(items * parts) <= fill * most; };
+  return fits(8, 4640) ? 8 : fits(4, 5200) ? 4 : fits(2, 6400) ? 2 : 1;
 }
 
 // Parts of a list-split launch of t (1: no split): launches with the plain
@@ -313,7 +323,7 @@ int auto_parts(int64_t n_items) {
 // it, by auto_parts.
 int split_parts(const octgrav_tree* t, bool capture) {
   if (capture || t->learned) return 1;
-  return t->nparts > 0 ? t->nparts : auto_parts(t->n_items);
+  return t->nparts > 0 ? t->nparts : auto_parts(t);
 }
 
 // The parts' outputs, reserved where the work items are made, so that a launch
@@ -1416,7 +1426,7 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   const size_t n = static_cast<size_t>(t->n), nc = static_cast<size_t>(t->n_cells),
                ni = static_cast<size_t>(t->n_items);
   // a few work items run split, as a launch does until octgrav_set_split is called
-  const int nparts = t->learned ? 1 : auto_parts(t->n_items);
+  const int nparts = t->learned ? 1 : auto_parts(t);
   // arena layout: the device arrays, each starting on a 256-byte boundary
   const size_t sizes[8] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
                            4 * nc * sizeof(float4), ni * sizeof(int4),      4 * ni * sizeof(float4),
@@ -1653,8 +1663,8 @@ static int autotune_common(int n_sys, const int64_t* offsets, const double* pos,
     }
     octgrav_free_tree(t);
   }
-  // the staging of the accepted cell records, for the winner (a split runs
-  // with per-lane cp.async staging only)
+  // the staging of the accepted cell records, for the winner (a split winner
+  // keeps per-lane cp.async staging)
   if (rc == OCTGRAV_OK && tune_staging && bng >= 0 && bsplit == 1) {
     octgrav_tree* t = nullptr;
     if (!(rc = build_common(n_sys, offsets, pos, mass, n_leaf, bng, &t)) && !(rc = octgrav_set_launch(t, bppl, 0))) {

@@ -1,5 +1,5 @@
 """The list split that launches of small trees choose themselves: the number of
-parts on both sides of the rule's bounds, every staging mode, the
+parts on both sides of the rule's bounds in items and particles, every staging mode, the
 allocation-free call and a user's own stream capture; and source chunks whose
 leaves are shorter and longer than a chunk."""
 import numpy as np
@@ -31,13 +31,22 @@ def _dev(torch, T, eps=0.01, theta=0.6):
     return out.cpu().numpy()
 
 
-@pytest.mark.parametrize("items,parts", [(1, 8), (637, 8), (638, 4), (1275, 4), (1276, 2), (2550, 2), (2551, 1)])
-def test_parts_by_number_of_items(torch, items, parts):
-    """One particle per leaf and group on a line: one work item per particle."""
-    pos = np.zeros((items, 3))
-    pos[:, 0] = np.arange(items) + 0.25 * np.sin(np.arange(items))
-    m = np.full(items, 1.0 / items)
-    T = G.Tree.build_gpu(pos, m, 1, 1)
+def _clumps(items, per_item, seed):
+    """`items` clumps of `per_item` particles: one work item each."""
+    rng = np.random.default_rng(seed)
+    c = rng.random((items, 3)) * 100
+    return (np.repeat(c, per_item, 0) + 1e-4 * rng.random((items * per_item, 3))), rng.random(items * per_item)
+
+
+@pytest.mark.parametrize("items,per_item,parts", [
+    (49, 20, 1), (50, 20, 8), (580, 20, 8), (581, 20, 4), (1300, 20, 4), (1301, 20, 2), (3200, 20, 2), (3201, 20, 1),
+    (111, 9, 1), (112, 9, 8), (170, 6, 8), (200, 6, 4), (500, 6, 2), (1010, 6, 2), (1011, 6, 1), (500, 5, 1)])
+def test_parts_by_number_and_size_of_items(torch, items, per_item, parts):
+    """Both sides of the rule's bounds: the launch equals that of the number of
+    parts that the rule states, and the unsplit one within FP32 rounding."""
+    pos, m = _clumps(items, per_item, 2 * items + per_item)
+    n_leaf = per_item
+    T = G.Tree.build_gpu(pos, m, n_leaf, n_leaf)
     assert T.stats["n_items"] == items
     auto = _dev(torch, T)
     c = T.interaction_counts()
@@ -46,13 +55,21 @@ def test_parts_by_number_of_items(torch, items, parts):
     T.set_split(1)
     one = _dev(torch, T)
     assert T.interaction_counts() == c
-    ref = O.Tree(pos, m, 1, 1).forces(0.01, 0.6)
+    ref = O.Tree(pos, m, n_leaf, n_leaf).forces(0.01, 0.6)
     for a in (auto, one):
-        acc, pot = np.empty((items, 3)), np.empty(items)
+        acc, pot = np.empty((len(m), 3)), np.empty(len(m))
         acc[T.perm()], pot[T.perm()] = a[:, :3], a[:, 3]
-        if items > 1:
-            assert O.rel_rms(acc, ref[0]) <= TOL_RMS
-            assert np.linalg.norm(pot - ref[1]) <= TOL_RMS * np.linalg.norm(ref[1])
+        assert O.rel_rms(acc, ref[0]) <= TOL_RMS
+        assert np.linalg.norm(pot - ref[1]) <= TOL_RMS * np.linalg.norm(ref[1])
+
+
+def test_small_systems_of_a_batch_are_not_split(torch):
+    systems = [_clumps(40, 20, k) for k in range(3)]
+    T = G.Tree.build_batch(systems, 20, 20)
+    assert T.stats["n_items"] == 120
+    auto = _dev(torch, T)
+    T.set_split(1)
+    assert np.array_equal(_dev(torch, T).view(np.uint32), auto.view(np.uint32))
 
 
 def test_staging_modes_and_noalloc_agree(torch):
