@@ -35,6 +35,7 @@ constexpr int LBMAX = 1024;       // ... and the most blocks it may have
 constexpr int NT = 128;           // threads of the node kernel
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LBINS = 32;  // leaf size bins of the moment pass (32 = "32 or more")
+constexpr int IBMAX = 608;  // blocks of the group and item kernel
 constexpr int IBINS = 256; // work-item size bins of the default processing order (item_max <= 256)
 
 struct SysGeo {  // root cube of a system: lower corner, side, 2^21 * fl(1 / side)
@@ -48,14 +49,14 @@ struct Chunk {  // TILE particles (or fewer) of one system
 
 // misc[] slots (int), zeroed before a build: counts, status bits, arrivals at
 // the grid barriers of the sort, the level and the node kernel, nodes per level
-enum { M_NGROUPS = 0, M_NITEMS, M_NLEAVES, M_MAXGROUP, M_STATUS, M_BAR_SORT, M_BAR_LEVELS, M_BAR_NODES, M_NODES };
+enum { M_NGROUPS = 0, M_NITEMS, M_NLEAVES, M_MAXGROUP, M_STATUS, M_BAR_SORT, M_BAR_LEVELS, M_BAR_NODES, M_BAR_ITEMS, M_NODES };
 constexpr int MISC = M_NODES + NLEV;
 
 // Scratch layout (byte offsets into one allocation).
 struct Layout {
   size_t keyA, keyB, valA, valB, cnt, dtot, part, sg, xs, ms, chunks, offs, chunk0;
   size_t ckey, cpar, cpf, cpc, csys, cfc, cnc, spl, lpre, nlist, bsum, lvl, misc;
-  size_t sstart, send, lofs, ni, lorder, lhist, ihist, gmark, gidx, gcell, nitem, ioff, sblk;
+  size_t sstart, send, lofs, ni, lorder, lhist, ihist, gmark, gcell, ioff, isum;
   size_t total;
 };
 
@@ -103,11 +104,9 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   L.lhist = take(4 * 2 * LBINS);
   L.ihist = take(4 * 2 * IBINS);
   L.gmark = take(4 * n);
-  L.gidx = take(4 * n);
   L.gcell = take(4 * n);
-  L.nitem = take(4 * n);
   L.ioff = take(4 * n);
-  L.sblk = take(4 * ((n + TILE - 1) / TILE + 1));
+  L.isum = take(4 * 2 * IBMAX);
   L.total = o;
   return L;
 }
@@ -305,41 +304,6 @@ __global__ void __launch_bounds__(TB) k_upsweep(const uint64_t* __restrict__ key
   cnt[256 * c.cs + threadIdx.x * c.nbs + (blockIdx.x - c.cs)] = h[threadIdx.x];
 }
 
-// Exclusive scan of a[0..m) in place, one block of 1024 threads.
-__global__ void __launch_bounds__(1024) k_scan_single(int* __restrict__ a, const int* __restrict__ m_dev, int m_max,
-                                                      int* __restrict__ total) {
-  const int m = m_dev ? min(*m_dev, m_max) : m_max;
-  __shared__ int ws[32];
-  const int per = (m + 1023) / 1024;
-  const int lo = min(m, threadIdx.x * per), hi = min(m, lo + per);
-  int s = 0;
-  for (int i = lo; i < hi; ++i) s += a[i];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int x = s;
-  for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(FULL, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int t = ws[lane];
-    for (int d = 1; d < 32; d <<= 1) {
-      const int y = __shfl_up_sync(FULL, t, d);
-      if (lane >= d) t += y;
-    }
-    ws[lane] = t;
-  }
-  __syncthreads();
-  int run = (w ? ws[w - 1] : 0) + x - s;
-  for (int i = lo; i < hi; ++i) {
-    const int v = a[i];
-    a[i] = run;
-    run += v;
-  }
-  if (threadIdx.x == 1023 && total) *total = ws[31];
-}
-
 // Per (system, digit): exclusive scan over the system's chunks in place, and
 // the digit's total. One warp per (system, digit).
 __global__ void __launch_bounds__(TB) k_scan_digits(int* __restrict__ cnt, const int* __restrict__ chunk0, int n_sys,
@@ -490,12 +454,15 @@ __global__ void __launch_bounds__(TB) k_sort(uint64_t* keyA, uint32_t* valA, uin
 }
 
 // Particles in tree order: FP64 copies for the moments, hi/lo FP32 records
-// for the walk kernel, and the permutation.
+// for the walk kernel, and the permutation; a build's group marks are cleared
+// on the way.
 __global__ void k_gather(const uint32_t* __restrict__ val, const double* __restrict__ pos,
                          const double* __restrict__ mass, int64_t n, double* __restrict__ xs,
-                         double* __restrict__ ms, float4* __restrict__ parts, int* __restrict__ perm) {
+                         double* __restrict__ ms, float4* __restrict__ parts, int* __restrict__ perm,
+                         int* __restrict__ gmark) {
   for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < n;
        t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    if (gmark) gmark[t] = 0;
     const int64_t i = val[t];
     const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2], m = mass[i];
     xs[3 * t] = x;
@@ -518,7 +485,8 @@ struct Cells {
   int *par, *pf, *pc, *sys, *fc, *nc;
 };
 
-__global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, int* __restrict__ lvl) {
+__global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, int* __restrict__ lvl,
+                        int* __restrict__ lhist) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < n_sys) {
     C.key[s] = 1;
@@ -530,6 +498,7 @@ __global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, in
     C.nc[s] = 0;
   }
   if (s <= NLEV + 1) lvl[s] = s == 0 ? 0 : n_sys;
+  if (s < 2 * LBINS) lhist[s] = 0;
 }
 
 // Split points of a cell holding particles [f, f + cnt): sp[o] = the first
@@ -819,11 +788,6 @@ __global__ void k_new_index(const int* __restrict__ lvl, const int* __restrict__
   }
 }
 
-__global__ void k_one_system_offsets(const int* __restrict__ lvl, int64_t* __restrict__ cell_off) {
-  cell_off[0] = 0;
-  cell_off[1] = lvl[NLEV];
-}
-
 // ---------------------------------------------------------------- cell properties
 
 struct Props {  // final-order FP64 arrays and records
@@ -1006,11 +970,12 @@ __device__ __forceinline__ void node_props(int c, Cells C, const int* __restrict
 __device__ __forceinline__ int leaf_bin(int cnt) { return LBINS - min(cnt, LBINS); }  // 32+ -> bin 0
 
 __global__ void __launch_bounds__(TB) k_leaf_hist(Cells C, const int* __restrict__ lvl, int* __restrict__ lhist,
-                                                  int* __restrict__ misc) {
+                                                  int* __restrict__ misc, int64_t* __restrict__ cell_off) {
   __shared__ int h[LBINS];
   if (threadIdx.x < LBINS) h[threadIdx.x] = 0;
   __syncthreads();
   const int nc = lvl[NLEV];
+  if (cell_off && blockIdx.x == 0 && threadIdx.x < 2) cell_off[threadIdx.x] = threadIdx.x ? nc : 0;
   int leaves = 0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x)
     if (C.nc[c] == 0) {
@@ -1205,157 +1170,215 @@ __global__ void __launch_bounds__(NT) k_nodes(Cells C, int* lvl, const int* __re
 
 // ---------------------------------------------------------------- groups and items
 
-// A group is a cell that is a leaf or holds <= n_group particles while its
-// parent does not (the property is inherited by descendants, so "the first
-// such cell from the root" is exactly this). Marked at its first particle.
-__global__ void k_group_mark(Cells C, const int* __restrict__ lvl, int n_group, int* __restrict__ gmark,
-                             int* __restrict__ gcell) {
-  const int nc = lvl[NLEV];
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-    const bool elig = C.nc[c] == 0 || C.pc[c] <= n_group;
-    const int p = C.par[c];
-    const bool pelig = p >= 0 && C.pc[p] <= n_group;  // a parent is never a leaf
-    if (elig && !pelig) {
-      gmark[C.pf[c]] = 1;
-      gcell[C.pf[c]] = c;
-    }
+struct Items {
+  const int64_t* cell_off;
+  int item_max, split;
+  int4* items;
+  float4* ibox;
+  uint64_t* item_key;
+  int* group_item;
+};
+
+// Work items of group g in cell c (final order) of system s, from item k on, cut
+// by next_item_size (at most item_max particles each), all with the group's
+// box, centre (hi/lo) and particle range. `item(k, size)` sees each of them.
+template <class F>
+__device__ __forceinline__ void group_items(int g, int c, int s, int k, const Props& P, const Items& I, F item) {
+  const int pf = P.cfirst[c], cnt = P.pcount[c];
+  float chi[3], clo[3];
+  for (int d = 0; d < 3; ++d) {
+    const double C0 = P.cube[4 * c + d];
+    chi[d] = static_cast<float>(C0);
+    clo[d] = static_cast<float>(C0 - static_cast<double>(chi[d]));
+  }
+  const float4 b0 = make_float4(static_cast<float>(P.bmin[3 * c]), static_cast<float>(P.bmin[3 * c + 1]),
+                                static_cast<float>(P.bmin[3 * c + 2]), chi[0]);
+  const float4 b1 = make_float4(static_cast<float>(P.bmax[3 * c]), static_cast<float>(P.bmax[3 * c + 1]),
+                                static_cast<float>(P.bmax[3 * c + 2]), chi[1]);
+  const float4 b2 = make_float4(clo[0], clo[1], clo[2], chi[2]);
+  const float4 b3 = make_float4(__int_as_float(pf), __int_as_float(cnt), 0.f, 0.f);
+  const int root = static_cast<int>(I.cell_off[s]);
+  I.group_item[g] = k;
+  for (int off = 0, sz; off < cnt; off += sz, ++k) {
+    sz = next_item_size(cnt - off, I.item_max, I.split != 0);
+    I.items[k] = make_int4(root, pf + off, sz, s);
+    I.ibox[4 * static_cast<int64_t>(k)] = b0;
+    I.ibox[4 * static_cast<int64_t>(k) + 1] = b1;
+    I.ibox[4 * static_cast<int64_t>(k) + 2] = b2;
+    I.ibox[4 * static_cast<int64_t>(k) + 3] = b3;
+    I.item_key[k] = P.key[c];
+    item(sz);
   }
 }
 
-// Block sums of in[0..n) in chunks of TILE.
-__global__ void __launch_bounds__(TB) k_scan_reduce(const int* __restrict__ in, const int* __restrict__ n_dev, int n_max,
-                                                    int* __restrict__ sblk) {
-  const int n = n_dev ? min(*n_dev, n_max) : n_max;
-  const int64_t lo = static_cast<int64_t>(blockIdx.x) * TILE;
-  int s = 0;
-  for (int64_t i = lo + threadIdx.x; i < min(static_cast<int64_t>(n), lo + TILE); i += TB) s += in[i];
-  int tot;
-  block_scan_excl(s, &tot);
-  if (threadIdx.x == 0) sblk[blockIdx.x] = tot;
-}
-
-// out = exclusive prefix of in (chunk offsets from the scanned block sums).
-__global__ void __launch_bounds__(TB) k_scan_down(const int* __restrict__ in, const int* __restrict__ n_dev, int n_max,
-                                                  const int* __restrict__ sblk, int* __restrict__ out) {
-  const int n = n_dev ? min(*n_dev, n_max) : n_max;
-  const int64_t lo = static_cast<int64_t>(blockIdx.x) * TILE + static_cast<int64_t>(threadIdx.x) * IPT;
-  int v[IPT], s = 0;
-#pragma unroll
-  for (int k = 0; k < IPT; ++k) {
-    v[k] = lo + k < n ? in[lo + k] : 0;
-    s += v[k];
-  }
-  int tot;
-  int run = sblk[blockIdx.x] + block_scan_excl(s, &tot);
-#pragma unroll
-  for (int k = 0; k < IPT; ++k) {
-    if (lo + k < n) out[lo + k] = run;
-    run += v[k];
-  }
-}
-
-__global__ void k_group_emit(int64_t n, const int* __restrict__ gmark, const int* __restrict__ gidx,
-                             const int* __restrict__ gcell, Cells C, const int* __restrict__ ni,
-                             int* __restrict__ group_cell, int* __restrict__ group_sys, int* __restrict__ misc) {
-  int mg = 0;
-  for (int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; t < n;
-       t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    if (!gmark[t]) continue;
-    const int g = gidx[t], c = gcell[t];
-    group_cell[g] = final_index(ni, c);
-    group_sys[g] = C.sys[c];
-    mg = max(mg, C.pc[c]);
-  }
-  for (int s = 16; s; s >>= 1) mg = max(mg, __shfl_xor_sync(FULL, mg, s));
-  if ((threadIdx.x & 31) == 0 && mg) atomicMax(&misc[M_MAXGROUP], mg);
-}
-
-__global__ void k_item_count(const int* __restrict__ n_groups, const int* __restrict__ group_cell,
-                             const int* __restrict__ pcount, int item_max, int split, int* __restrict__ nitem) {
+// The items again from the same groups (a refit: boxes and centres change).
+__global__ void k_items(const int* __restrict__ n_groups, const int* __restrict__ group_cell,
+                        const int* __restrict__ group_sys, const int* __restrict__ ioff, Props P, Items I) {
   const int ng = *n_groups;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x)
-    nitem[g] = item_count(pcount[group_cell[g]], item_max, split != 0);
+    group_items(g, group_cell[g], group_sys[g], ioff[g], P, I, [](int) {});
 }
 
-// Work items of every group, cut by next_item_size (at most item_max
-// particles each), all with the group's box, centre (hi/lo) and particle range.
-__global__ void k_items(const int* __restrict__ n_groups, const int* __restrict__ group_cell,
-                        const int* __restrict__ group_sys, const int* __restrict__ ioff, const int64_t* __restrict__ cell_off,
-                        Props P, int item_max, int split, int4* __restrict__ items, float4* __restrict__ ibox,
-                        uint64_t* __restrict__ item_key, int* __restrict__ group_item) {
-  const int ng = *n_groups;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
-    const int c = group_cell[g], s = group_sys[g];
-    const int pf = P.cfirst[c], cnt = P.pcount[c];
-    float chi[3], clo[3];
-    for (int d = 0; d < 3; ++d) {
-      const double C0 = P.cube[4 * c + d];
-      chi[d] = static_cast<float>(C0);
-      clo[d] = static_cast<float>(C0 - static_cast<double>(chi[d]));
-    }
-    const float4 b0 = make_float4(static_cast<float>(P.bmin[3 * c]), static_cast<float>(P.bmin[3 * c + 1]),
-                                  static_cast<float>(P.bmin[3 * c + 2]), chi[0]);
-    const float4 b1 = make_float4(static_cast<float>(P.bmax[3 * c]), static_cast<float>(P.bmax[3 * c + 1]),
-                                  static_cast<float>(P.bmax[3 * c + 2]), chi[1]);
-    const float4 b2 = make_float4(clo[0], clo[1], clo[2], chi[2]);
-    const float4 b3 = make_float4(__int_as_float(pf), __int_as_float(cnt), 0.f, 0.f);
-    const int root = static_cast<int>(cell_off[s]);
-    int k = ioff[g];
-    group_item[g] = k;
-    for (int off = 0, sz; off < cnt; off += sz, ++k) {
-      sz = next_item_size(cnt - off, item_max, split != 0);
-      items[k] = make_int4(root, pf + off, sz, s);
-      ibox[4 * static_cast<int64_t>(k)] = b0;
-      ibox[4 * static_cast<int64_t>(k) + 1] = b1;
-      ibox[4 * static_cast<int64_t>(k) + 2] = b2;
-      ibox[4 * static_cast<int64_t>(k) + 3] = b3;
-      item_key[k] = P.key[c];
+__device__ void finish(const int* lvl, const int* misc, int64_t* res) {
+  int depth = 0;
+  for (int L = 0; L < NLEV; ++L)
+    if (__ldcg(&lvl[L + 1]) > __ldcg(&lvl[L])) depth = L;
+  res[GB_NCELLS] = __ldcg(&lvl[NLEV]);
+  res[GB_NGROUPS] = __ldcg(&misc[M_NGROUPS]);
+  res[GB_NITEMS] = __ldcg(&misc[M_NITEMS]);
+  res[GB_DEPTH] = depth;
+  res[GB_NLEAVES] = __ldcg(&misc[M_NLEAVES]);
+  res[GB_MAXGROUP] = __ldcg(&misc[M_MAXGROUP]);
+  res[GB_STATUS] = __ldcg(&misc[M_STATUS]);
+}
+
+__global__ void k_finish(const int* __restrict__ lvl, const int* __restrict__ misc, int64_t* __restrict__ res) {
+  finish(lvl, misc, res);
+}
+
+// Groups (ordered by first particle), their work items, the items' default
+// processing order and the build's result, in one cooperative launch:
+//   marks: a group is a cell that is a leaf or holds <= n_group particles while
+//     its parent does not (the property is inherited by descendants, so "the
+//     first such cell from the root" is exactly this), marked at its first
+//     particle;
+//   sums: every block counts the groups and items of its range of particles;
+//   group numbers and first items from the sums of the blocks before;
+//   items, a thread per group;
+//   order: most particles first, a counting sort on the item size (the order
+//     inside a size is arbitrary and does not affect any result).
+// Latency-bound: each phase is a few dependent loads. 17 us at 5000 particles
+// and 45 us at 1M, with four barriers of about 2 us; as twelve launches, with
+// two scans of three launches each, the build's end took 56 and 97 us more.
+struct Groups {
+  int n, n_group;
+  int mark;  // 0: the marks of the build are there
+  const int* ni;
+  int *gmark, *gcell;
+  int *group_cell, *group_sys;
+  int *ioff, *isum, *ihist;
+  int* order;
+  int64_t* result;
+};
+
+__global__ void __launch_bounds__(TB) k_groups(Cells C, Props P, Items I, Groups G, int* lvl, int* misc) {
+  static_assert(IBINS == TB, "a thread per size bin");
+  __shared__ int hist[IBINS], base[IBINS];
+  const int grid = gridDim.x, first = blockIdx.x * TB + threadIdx.x, stride = grid * TB;
+  int bars = 0;
+  // all blocks see the same bit of an earlier kernel; a barrier that runs out stops this one
+  const auto sync = [&]() {
+    if (grid_barrier(&misc[M_BAR_ITEMS], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) return true;
+    no_cells(lvl);
+    if (threadIdx.x == 0) finish(lvl, misc, G.result);
+    return false;
+  };
+  if (__ldcg(&misc[M_STATUS]) & GPU_BUILD_STUCK) {
+    if (threadIdx.x == 0) finish(lvl, misc, G.result);
+    return;
+  }
+  if (blockIdx.x == 0)
+    for (int k = threadIdx.x; k < 2 * IBINS; k += TB) G.ihist[k] = 0;
+  if (G.mark) {
+    const int nc = lvl[NLEV];
+    for (int c = first; c < nc; c += stride) {
+      const bool elig = C.nc[c] == 0 || C.pc[c] <= G.n_group;
+      const int p = C.par[c];
+      const bool pelig = p >= 0 && C.pc[p] <= G.n_group;  // a parent is never a leaf
+      if (elig && !pelig) {
+        G.gmark[C.pf[c]] = 1;
+        G.gcell[C.pf[c]] = c;
+      }
     }
   }
-}
+  if (!sync()) return;
 
-// Default processing order of the work items: most particles first (a
-// counting sort on the item size; the order inside a size is arbitrary and
-// does not affect any result).
-__global__ void __launch_bounds__(TB) k_item_hist(const int* __restrict__ n_items, const int4* __restrict__ items,
-                                                  int* __restrict__ ihist) {
-  __shared__ int h[IBINS];
-  for (int k = threadIdx.x; k < IBINS; k += TB) h[k] = 0;
-  __syncthreads();
-  const int ni = *n_items;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ni; k += gridDim.x * blockDim.x)
-    atomicAdd(&h[IBINS - min(items[k].z, IBINS)], 1);
-  __syncthreads();
-  for (int k = threadIdx.x; k < IBINS; k += TB)
-    if (h[k]) atomicAdd(&ihist[k], h[k]);
-}
+  const int64_t per = (static_cast<int64_t>(G.n) + stride - 1) / stride * TB;
+  const int64_t lo = blockIdx.x * per, hi = min(static_cast<int64_t>(G.n), lo + per);
+  const auto marked = [&](int64_t t, int* c) {
+    if (t >= hi || !__ldcg(&G.gmark[t])) return false;
+    *c = __ldcg(&G.gcell[t]);
+    return true;
+  };
+  {
+    int ng = 0, nk = 0, mg = 0, c, tot;
+    for (int64_t t = lo + threadIdx.x; t < hi; t += TB)
+      if (marked(t, &c)) {
+        const int pc = C.pc[c];
+        ++ng;
+        nk += item_count(pc, I.item_max, I.split != 0);
+        mg = max(mg, pc);
+      }
+    block_scan_excl(ng, &tot);
+    if (threadIdx.x == 0) G.isum[2 * blockIdx.x] = tot;
+    block_scan_excl(nk, &tot);
+    if (threadIdx.x == 0) G.isum[2 * blockIdx.x + 1] = tot;
+    for (int s = 16; s; s >>= 1) mg = max(mg, __shfl_xor_sync(FULL, mg, s));
+    if ((threadIdx.x & 31) == 0 && mg) atomicMax(&misc[M_MAXGROUP], mg);
+  }
+  if (!sync()) return;
 
-__global__ void __launch_bounds__(TB) k_item_scatter(const int* __restrict__ n_items, const int4* __restrict__ items,
-                                                     const int* __restrict__ ihist, int* __restrict__ ifill,
-                                                     int* __restrict__ order) {
-  __shared__ int base[IBINS], h[IBINS];
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int k = 0; k < IBINS; ++k) {
-      base[k] = run;
-      run += ihist[k];
+  int ng = 0, nk = 0;  // of all blocks
+  {
+    int bg = 0, bk = 0;
+    for (int j = threadIdx.x; j < grid; j += TB) {
+      const int2 v = __ldcg(reinterpret_cast<const int2*>(G.isum) + j);
+      ng += v.x;
+      nk += v.y;
+      if (j < static_cast<int>(blockIdx.x)) {
+        bg += v.x;
+        bk += v.y;
+      }
+    }
+    block_scan_excl(ng, &ng);
+    block_scan_excl(nk, &nk);
+    block_scan_excl(bg, &bg);
+    block_scan_excl(bk, &bk);
+    for (int64_t t0 = lo; t0 < hi; t0 += TB) {
+      int c = 0, tot;
+      const bool m = marked(t0 + threadIdx.x, &c);
+      const int g = bg + block_scan_excl(m ? 1 : 0, &tot);
+      bg += tot;
+      const int k = bk + block_scan_excl(m ? item_count(C.pc[c], I.item_max, I.split != 0) : 0, &tot);
+      bk += tot;
+      if (m) {
+        G.group_cell[g] = final_index(G.ni, c);
+        G.group_sys[g] = C.sys[c];
+        G.ioff[g] = k;
+      }
     }
   }
-  const int ni = *n_items;
-  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t k0 = static_cast<int64_t>(blockIdx.x) * blockDim.x; k0 < ni; k0 += stride) {
-    for (int k = threadIdx.x; k < IBINS; k += TB) h[k] = 0;
+  if (!sync()) return;
+
+  hist[threadIdx.x] = 0;
+  __syncthreads();
+  for (int g = first; g < ng; g += stride)
+    group_items(g, __ldcg(&G.group_cell[g]), __ldcg(&G.group_sys[g]), __ldcg(&G.ioff[g]), P, I,
+                [&](int sz) { atomicAdd(&hist[IBINS - min(sz, IBINS)], 1); });
+  __syncthreads();
+  if (hist[threadIdx.x]) atomicAdd(&G.ihist[threadIdx.x], hist[threadIdx.x]);
+  if (!sync()) return;
+
+  int tot;
+  base[threadIdx.x] = block_scan_excl(__ldcg(&G.ihist[threadIdx.x]), &tot);
+  int* fill = G.ihist + IBINS;
+  for (int64_t k0 = static_cast<int64_t>(blockIdx.x) * TB; k0 < nk; k0 += stride) {
+    hist[threadIdx.x] = 0;
     __syncthreads();
     const int k = static_cast<int>(k0) + threadIdx.x;
-    const bool live = k < ni;
-    const int b = live ? IBINS - min(items[k].z, IBINS) : 0;
-    const int r = live ? atomicAdd(&h[b], 1) : 0;
+    const bool live = k < nk;
+    const int b = live ? IBINS - min(__ldcg(&I.items[k].z), IBINS) : 0;
+    const int r = live ? atomicAdd(&hist[b], 1) : 0;
     __syncthreads();
-    for (int q = threadIdx.x; q < IBINS; q += TB)
-      if (h[q]) h[q] = atomicAdd(&ifill[q], h[q]);
+    if (hist[threadIdx.x]) hist[threadIdx.x] = atomicAdd(&fill[threadIdx.x], hist[threadIdx.x]);
     __syncthreads();
-    if (live) order[base[b] + h[b] + r] = k;
+    if (live) G.order[base[b] + hist[b] + r] = k;
     __syncthreads();
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    misc[M_NGROUPS] = ng;
+    misc[M_NITEMS] = nk;
+    finish(lvl, misc, G.result);
   }
 }
 
@@ -1363,19 +1386,6 @@ __global__ void __launch_bounds__(TB) k_item_scatter(const int* __restrict__ n_i
 __global__ void k_clear_status(int* __restrict__ misc) {
   misc[M_STATUS] = 0;
   misc[M_BAR_NODES] = 0;
-}
-
-__global__ void k_finish(const int* __restrict__ lvl, const int* __restrict__ misc, int64_t* __restrict__ res) {
-  int depth = 0;
-  for (int L = 0; L < NLEV; ++L)
-    if (lvl[L + 1] > lvl[L]) depth = L;
-  res[GB_NCELLS] = lvl[NLEV];
-  res[GB_NGROUPS] = misc[M_NGROUPS];
-  res[GB_NITEMS] = misc[M_NITEMS];
-  res[GB_DEPTH] = depth;
-  res[GB_NLEAVES] = misc[M_NLEAVES];
-  res[GB_MAXGROUP] = misc[M_MAXGROUP];
-  res[GB_STATUS] = misc[M_STATUS];
 }
 
 __global__ void k_unpermute(const float4* __restrict__ out, const int* __restrict__ perm, int64_t n,
@@ -1407,28 +1417,22 @@ cudaError_t enqueue_nodes(const GpuBuild& a, const Layout& Lo, Cells C, const in
                             static_cast<const int*>(at<int>(a.scratch, Lo.nlist)), ni, P, at<int>(a.scratch, Lo.misc));
 }
 
-// Items from the groups (group_cell, group_sys and the cell arrays in P).
-cudaError_t enqueue_items(const GpuBuild& a, const Layout& Lo, int item_max, cudaStream_t st) {
-  int* misc = at<int>(a.scratch, Lo.misc);
-  int* nitem = at<int>(a.scratch, Lo.nitem);
-  int* ioff = at<int>(a.scratch, Lo.ioff);
-  int* sblk = at<int>(a.scratch, Lo.sblk);
-  const int nmax = static_cast<int>(a.n);
-  const int nb = static_cast<int>((a.n + TILE - 1) / TILE);
+Items item_args(const GpuBuild& a) {
+  return {a.cell_off, a.item_max, a.item_split, a.items, a.ibox, a.item_key, a.group_item};
+}
+
+// Groups and items; with mark = false of the groups that a build has marked.
+cudaError_t enqueue_groups(const GpuBuild& a, const Layout& Lo, bool mark, cudaStream_t st) {
+  void* S = a.scratch;
+  Cells C{at<uint64_t>(S, Lo.ckey), at<int>(S, Lo.cpar), at<int>(S, Lo.cpf), at<int>(S, Lo.cpc),
+          at<int>(S, Lo.csys),      at<int>(S, Lo.cfc),  at<int>(S, Lo.cnc)};
   Props P{a.bmin, a.bmax, a.cube, a.M, a.com, a.S, a.key, a.geo, a.link, a.mp, a.pcount, a.cfirst};
-  k_item_count<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.pcount, item_max, a.item_split,
-                                                 nitem);
-  k_scan_reduce<<<nb, TB, 0, st>>>(nitem, &misc[M_NGROUPS], nmax, sblk);
-  k_scan_single<<<1, 1024, 0, st>>>(sblk, nullptr, nb, &misc[M_NITEMS]);
-  k_scan_down<<<nb, TB, 0, st>>>(nitem, &misc[M_NGROUPS], nmax, sblk, ioff);
-  k_items<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.group_sys, ioff, a.cell_off, P,
-                                            item_max, a.item_split, a.items, a.ibox, a.item_key, a.group_item);
-  int* ihist = at<int>(a.scratch, Lo.ihist);
-  cudaError_t e = cudaMemsetAsync(ihist, 0, 4 * 2 * IBINS, st);
-  if (e != cudaSuccess) return e;
-  k_item_hist<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NITEMS], a.items, ihist);
-  k_item_scatter<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NITEMS], a.items, ihist, ihist + IBINS, a.order);
-  return cudaGetLastError();
+  const Groups G{static_cast<int>(a.n), a.n_group, mark, a.n_sys > 1 ? at<int>(S, Lo.ni) : nullptr,
+                 at<int>(S, Lo.gmark), at<int>(S, Lo.gcell), a.group_cell, a.group_sys, at<int>(S, Lo.ioff),
+                 at<int>(S, Lo.isum), at<int>(S, Lo.ihist), a.order, a.result};
+  const int most = static_cast<int>(std::min<int64_t>((a.n + TB - 1) / TB, IBMAX));
+  return launch_cooperative(k_groups, resident_blocks(k_groups, TB, most), TB, 0, st, C, P, item_args(a), G,
+                            at<int>(S, Lo.lvl), at<int>(S, Lo.misc));
 }
 
 std::vector<Chunk> make_chunks(const int64_t* offsets, int n_sys, std::vector<int>& chunk0) {
@@ -1530,10 +1534,12 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
     }
   }
   OG_TRY(cudaGetLastError());
-  k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(valA, a.pos, a.mass, a.n, xs, ms, a.parts, a.perm);
+  k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(valA, a.pos, a.mass, a.n, xs, ms, a.parts, a.perm,
+                                             at<int>(S, Lo.gmark));
 
   // ---- cells, level by level (sizes live in lvl[] on the device)
-  k_roots<<<(std::max(a.n_sys, NLEV + 2) + 127) / 128, 128, 0, st>>>(a.n_sys, doffs, C, lvl);
+  k_roots<<<(std::max({a.n_sys, NLEV + 2, 2 * LBINS}) + 127) / 128, 128, 0, st>>>(a.n_sys, doffs, C, lvl,
+                                                                                 at<int>(S, Lo.lhist));
   {
     // about a warp per cell that is split on the widest level; a small tree gets
     // few blocks, whose barriers are cheaper
@@ -1556,34 +1562,19 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
     k_sys_bounds<<<gc, TB, 0, st>>>(lvl, C.sys, sstart, send);
     k_sys_offsets<<<1, 1024, 0, st>>>(a.n_sys, sstart, send, lofs, a.cell_off);
     k_new_index<<<gc, TB, 0, st>>>(lvl, C.sys, sstart, lofs, ni);
-  } else {
-    k_one_system_offsets<<<1, 1, 0, st>>>(lvl, a.cell_off);
   }
 
   // ---- properties: every leaf at once, then the nodes deepest level first
   int* lorder = at<int>(S, Lo.lorder);
   int* lhist = at<int>(S, Lo.lhist);
-  OG_TRY(cudaMemsetAsync(lhist, 0, 4 * 2 * LBINS, st));
-  k_leaf_hist<<<gc, TB, 0, st>>>(C, lvl, lhist, misc);
+  k_leaf_hist<<<gc, TB, 0, st>>>(C, lvl, lhist, misc, a.n_sys > 1 ? nullptr : a.cell_off);
   k_leaf_scatter<<<gc, TB, 0, st>>>(C, lvl, lhist, lhist + LBINS, lorder);
   k_leaf_props<<<gc, TB, 0, st>>>(C, lorder, misc, ni, xs, ms, P);
   OG_TRY(cudaGetLastError());
   OG_TRY(enqueue_nodes(a, Lo, C, ni, P, st));
 
-  // ---- groups (ordered by first particle) and work items
-  int* gmark = at<int>(S, Lo.gmark);
-  int* gidx = at<int>(S, Lo.gidx);
-  int* gcell = at<int>(S, Lo.gcell);
-  int* sblk = at<int>(S, Lo.sblk);
-  const int nb = static_cast<int>((a.n + TILE - 1) / TILE);
-  OG_TRY(cudaMemsetAsync(gmark, 0, 4 * a.n, st));
-  k_group_mark<<<gc, TB, 0, st>>>(C, lvl, a.n_group, gmark, gcell);
-  k_scan_reduce<<<nb, TB, 0, st>>>(gmark, nullptr, static_cast<int>(a.n), sblk);
-  k_scan_single<<<1, 1024, 0, st>>>(sblk, nullptr, nb, &misc[M_NGROUPS]);
-  k_scan_down<<<nb, TB, 0, st>>>(gmark, nullptr, static_cast<int>(a.n), sblk, gidx);
-  k_group_emit<<<grid_for(a.n, TB), TB, 0, st>>>(a.n, gmark, gidx, gcell, C, ni, a.group_cell, a.group_sys, misc);
-  OG_TRY(enqueue_items(a, Lo, a.item_max, st));
-  k_finish<<<1, 1, 0, st>>>(lvl, misc, a.result);
+  // ---- groups (ordered by first particle), work items and the result
+  OG_TRY(enqueue_groups(a, Lo, true, st));
 #undef OG_TRY
   return cudaGetLastError();
 }
@@ -1606,12 +1597,11 @@ cudaError_t gpu_refit(const GpuBuild& a, cudaStream_t st) {
   k_clear_status<<<1, 1, 0, st>>>(misc);
   k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, at<Chunk>(S, Lo.chunks), at<double>(S, Lo.part), misc);
   k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(at<uint32_t>(S, Lo.valA), a.pos, a.mass, a.n, at<double>(S, Lo.xs),
-                                             at<double>(S, Lo.ms), a.parts, a.perm);
+                                             at<double>(S, Lo.ms), a.parts, a.perm, nullptr);
   k_leaf_props<<<gc, TB, 0, st>>>(C, at<int>(S, Lo.lorder), misc, ni, at<double>(S, Lo.xs), at<double>(S, Lo.ms), P);
   if ((e = enqueue_nodes(a, Lo, C, ni, P, st)) != cudaSuccess) return e;
-  k_items<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.group_sys, at<int>(S, Lo.ioff),
-                                            a.cell_off, P, a.item_max, a.item_split, a.items, a.ibox, a.item_key,
-                                            a.group_item);
+  k_items<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.group_sys, at<int>(S, Lo.ioff), P,
+                                            item_args(a));
   k_finish<<<1, 1, 0, st>>>(lvl, misc, a.result);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return cudaSuccess;
@@ -1620,12 +1610,8 @@ cudaError_t gpu_refit(const GpuBuild& a, cudaStream_t st) {
 cudaError_t gpu_build_items(const GpuBuild& a, cudaStream_t st) {
   const Layout Lo = layout(a.n, a.n_sys, (a.n + TILE - 1) / TILE + a.n_sys, a.cap);
   if (Lo.total > a.scratch_bytes) return cudaErrorInvalidValue;
-  cudaError_t e = enqueue_items(a, Lo, a.item_max, st);
-  if (e != cudaSuccess) return e;
-  int* misc = at<int>(a.scratch, Lo.misc);
-  const int* lvl = at<int>(a.scratch, Lo.lvl);
-  k_finish<<<1, 1, 0, st>>>(lvl, misc, a.result);
-  return cudaGetLastError();
+  cudaError_t e = cudaMemsetAsync(at<int>(a.scratch, Lo.misc) + M_BAR_ITEMS, 0, 4, st);
+  return e != cudaSuccess ? e : enqueue_groups(a, Lo, false, st);
 }
 
 __global__ void k_pull(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t n16) {

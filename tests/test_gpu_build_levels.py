@@ -1,7 +1,8 @@
 """The level and node kernels of the GPU build where their rules change: cells
 of 32 and 33 particles (one probe per particle or a search), levels that end at
 the depth limit, trees of one block and of many, more nodes on a level than
-eight-lane groups take, and the most chunks that are sorted in one launch. Byte equality with the host build throughout."""
+eight-lane groups take, the most chunks that are sorted in one launch, and groups
+and items on both sides of a block's range. Byte equality with the host build throughout."""
 import numpy as np
 import pytest
 
@@ -87,3 +88,35 @@ def test_sort_of_several_systems(sizes):
                          offsets=offs)
     assert A.stats == B.stats
     assert np.array_equal(A.perm(), B.perm()) and np.array_equal(A.cell_keys(), B.cell_keys())
+
+
+def _same_items(A, B):
+    a, b = A.item_info(), B.item_info()
+    assert A.stats == B.stats and a.keys() == b.keys()
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 608 * 256, 608 * 256 + 1])
+@pytest.mark.parametrize("n_group", [1, 8, 300])
+def test_groups_and_items(n, n_group):
+    """One particle range per block of the group kernel and two, groups of one
+    particle and of more than an item holds, and items cut anew."""
+    pos, m = W.plummer(n, seed=n)
+    A, B = G.Tree.build(pos, m, min(8, n_group), n_group), G.Tree.build_gpu(pos, m, min(8, n_group), n_group)
+    _same_items(A, B)
+    for ppl in (1, 2):
+        A.set_launch(ppl)
+        B.set_launch(ppl)
+        _same_items(A, B)
+
+
+def test_groups_of_several_systems_and_of_coincident_particles():
+    rng = np.random.default_rng(8)
+    systems = [(rng.random((k, 3)), rng.random(k)) for k in (700, 1, 3000, 257)]
+    systems[2][0][:900] = systems[2][0][0]
+    offs = np.array([0, 700, 701, 3701, 3958], np.int64)
+    A = G.Tree.build_batch(systems, 8, 64)
+    B = G.Tree.build_gpu(np.concatenate([p for p, _ in systems]), np.concatenate([m for _, m in systems]), 8, 64,
+                         offsets=offs)
+    _same_items(A, B)
