@@ -35,6 +35,7 @@ constexpr int LBMAX = 1024;       // ... and the most blocks it may have
 constexpr int NT = 128;           // threads of the node kernel
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LBINS = 32;  // leaf size bins of the moment pass (32 = "32 or more")
+constexpr int SORT_CHUNKS4 = 8, SORT_CHUNKS2 = 64;  // most chunks that k_sort takes with four and two blocks each
 constexpr int IBMAX = 608;  // blocks of the group and item kernel
 constexpr int IBINS = 256; // work-item size bins of the default processing order (item_max <= 256)
 
@@ -74,7 +75,7 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   L.keyB = take(8 * n);
   L.valA = take(4 * n);
   L.valB = take(4 * n);
-  L.cnt = take(4 * 256 * n_chunks);
+  L.cnt = take(4 * 256 * std::max<int64_t>(n_chunks, 2 * SORT_CHUNKS2));
   L.dtot = take(4 * 256 * static_cast<size_t>(n_sys));
   L.part = take(8 * 6 * BSUB * n_chunks);
   L.sg = take(sizeof(SysGeo) * n_sys);
@@ -330,24 +331,25 @@ __global__ void __launch_bounds__(TB) k_scan_digits(int* __restrict__ cnt, const
 }
 
 // Stable ranks of one chunk's keys by the digit at `shift`: warp w ranks its
-// 512 elements round by round (32 at a time, in order); afterwards wc[w][d] is
+// 32 K elements round by round (32 at a time, in order); afterwards wc[w][d] is
 // the number of elements of digit d in the warps before, and an element's place
 // among its chunk's digit is wc[w][d] + rk. Returns the chunk's count of digit
 // threadIdx.x.
+template <int K>
 __device__ __forceinline__ int chunk_ranks(const uint64_t* kin, const uint32_t* vin, const Chunk& c, int shift,
                                            int (*wc)[257], uint64_t* kk, uint32_t* vv, int* rk) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-  for (int r = 0; r < IPT; ++r) {
-    const int e = w * (32 * IPT) + r * 32 + lane;
+  for (int r = 0; r < K; ++r) {
+    const int e = w * (32 * K) + r * 32 + lane;
     const bool ok = e < c.count;
     kk[r] = ok ? __ldcg(kin + c.first + e) : 0ull;
     vv[r] = ok ? __ldcg(vin + c.first + e) : 0u;
   }
 #pragma unroll
-  for (int r = 0; r < IPT; ++r) {
-    const int e = w * (32 * IPT) + r * 32 + lane;
+  for (int r = 0; r < K; ++r) {
+    const int e = w * (32 * K) + r * 32 + lane;
     const int d = e < c.count ? static_cast<int>((kk[r] >> shift) & 255) : 256;
     const unsigned peers = __match_any_sync(FULL, d);
     const int before = wc[w][d];
@@ -386,7 +388,7 @@ __global__ void __launch_bounds__(TB) k_downsweep(const uint64_t* __restrict__ k
   uint64_t kk[IPT];
   uint32_t vv[IPT];
   int rk[IPT];
-  chunk_ranks(kin, vin, c, shift, wc, kk, vv, rk);
+  chunk_ranks<IPT>(kin, vin, c, shift, wc, kk, vv, rk);
 #pragma unroll
   for (int r = 0; r < IPT; ++r) {
     const int e = (threadIdx.x >> 5) * (32 * IPT) + r * 32 + (threadIdx.x & 31);
@@ -399,21 +401,26 @@ __global__ void __launch_bounds__(TB) k_downsweep(const uint64_t* __restrict__ k
   }
 }
 
-// All eight passes in one cooperative launch, a block per chunk: ranks, the
-// chunk's digit counts, a grid barrier, offsets (every block adds the counts of
-// its system's chunks itself, a thread per digit), scatter, a second barrier.
+// All eight passes in one cooperative launch, W blocks per chunk: ranks, the
+// blocks' digit counts, a grid barrier, offsets (every block adds the counts of
+// its system's blocks itself, a thread per digit), scatter, a second barrier.
 // The same order as the passes by three launches each, whose gaps and short
 // grids made up most of the time of a small sort: from the keys to the gather
-// 157 us at 5000 particles, 83 us so. The sums over the chunks grow with their
-// number: 163 and 93 us at 65,536 particles, 159 and 103 us at 64 chunks
-// (262,144), which is where the rule ends.
-constexpr int SORT_CHUNKS = 64;
-
+// 157 us at 5000 particles, 48 us so. The rest is latency: a warp ranks its 16 /
+// W rounds one after the other, and the sums grow with the blocks. Times of W =
+// 1 / 2 / 4 / 8 (us): 5000 particles 83 / 79 / 48 / 54, 16,384 87 / 62 / 50 / 69,
+// 32,768 85 / 67 / 57 / 97, 65,536 87 / 67 / 71 / 146, 262,144 100 / 98 / 176
+// (159 by three launches a pass). Hence four blocks a chunk up to 8 chunks, two
+// up to 64.
+template <int W>
 __global__ void __launch_bounds__(TB) k_sort(uint64_t* keyA, uint32_t* valA, uint64_t* keyB, uint32_t* valB,
                                              const Chunk* __restrict__ ch, int* cnt, int* misc) {
   __shared__ int wc[TB / 32][257];
   __shared__ int goff[256];
-  const Chunk c = ch[blockIdx.x];
+  constexpr int K = IPT / W;
+  Chunk c = ch[blockIdx.x / W];
+  c.first += static_cast<int>(blockIdx.x % W) * (K * TB);
+  c.count = min(max(c.count - static_cast<int>(blockIdx.x % W) * (K * TB), 0), K * TB);
   const int first = ch[c.cs].first, grid = gridDim.x, mine = blockIdx.x;
   int bars = 0;
   for (int pass = 0; pass < 8; ++pass) {
@@ -421,15 +428,15 @@ __global__ void __launch_bounds__(TB) k_sort(uint64_t* keyA, uint32_t* valA, uin
     const bool even = (pass & 1) == 0;
     for (int k = threadIdx.x; k < (TB / 32) * 257; k += TB) (&wc[0][0])[k] = 0;
     __syncthreads();
-    uint64_t kk[IPT];
-    uint32_t vv[IPT];
-    int rk[IPT];
+    uint64_t kk[K];
+    uint32_t vv[K];
+    int rk[K];
     cnt[256 * mine + threadIdx.x] =
-        chunk_ranks(even ? keyA : keyB, even ? valA : valB, c, shift, wc, kk, vv, rk);
+        chunk_ranks<K>(even ? keyA : keyB, even ? valA : valB, c, shift, wc, kk, vv, rk);
     if (!grid_barrier(&misc[M_BAR_SORT], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) return;
     int before = 0, total = 0;
 #pragma unroll 8
-    for (int j = c.cs; j < c.cs + c.nbs; ++j) {
+    for (int j = W * c.cs; j < W * (c.cs + c.nbs); ++j) {
       const int v = __ldcg(&cnt[256 * j + threadIdx.x]);
       total += v;
       before += j < mine ? v : 0;
@@ -440,8 +447,8 @@ __global__ void __launch_bounds__(TB) k_sort(uint64_t* keyA, uint32_t* valA, uin
     uint64_t* kout = even ? keyB : keyA;
     uint32_t* vout = even ? valB : valA;
 #pragma unroll
-    for (int r = 0; r < IPT; ++r) {
-      const int e = (threadIdx.x >> 5) * (32 * IPT) + r * 32 + (threadIdx.x & 31);
+    for (int r = 0; r < K; ++r) {
+      const int e = (threadIdx.x >> 5) * (32 * K) + r * 32 + (threadIdx.x & 31);
       if (e < c.count) {
         const int d = static_cast<int>((kk[r] >> shift) & 255);
         const int dst = goff[d] + wc[threadIdx.x >> 5][d] + rk[r];
@@ -1518,9 +1525,11 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
   k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, dch, part, misc);
   k_root<<<a.n_sys, TB, 0, st>>>(part, dchunk0, sg);
   k_morton<<<SUB * nch, TB, 0, st>>>(a.pos, dch, sg, keyA, valA);
-  if (nch <= SORT_CHUNKS && resident_blocks(k_sort, TB, nch) == nch) {
-    const Chunk* chunks = dch;
-    OG_TRY(launch_cooperative(k_sort, nch, TB, 0, st, keyA, valA, keyB, valB, chunks, cnt, misc));
+  const Chunk* chunks = dch;
+  if (nch <= SORT_CHUNKS4 && resident_blocks(k_sort<4>, TB, 4 * nch) == 4 * nch) {
+    OG_TRY(launch_cooperative(k_sort<4>, 4 * nch, TB, 0, st, keyA, valA, keyB, valB, chunks, cnt, misc));
+  } else if (nch <= SORT_CHUNKS2 && resident_blocks(k_sort<2>, TB, 2 * nch) == 2 * nch) {
+    OG_TRY(launch_cooperative(k_sort<2>, 2 * nch, TB, 0, st, keyA, valA, keyB, valB, chunks, cnt, misc));
   } else {
     int* dtot = at<int>(S, Lo.dtot);
     const int segblocks = (256 * a.n_sys + TB / 32 - 1) / (TB / 32);

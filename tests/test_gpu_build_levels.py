@@ -69,14 +69,15 @@ def test_more_nodes_on_a_level_than_eight_lane_groups_take():
     assert max(int(np.sum((depth == d) & (counts > 1))) for d in range(22)) > 4 * 4 * 608
 
 
-@pytest.mark.parametrize("n", [64 * 4096, 64 * 4096 + 1])
+@pytest.mark.parametrize("n", [1023, 1025, 3073, 8 * 4096, 8 * 4096 + 1, 64 * 4096, 64 * 4096 + 1])
 def test_sort_in_one_launch_and_in_passes(n):
-    """The last size that one launch sorts and the first that it does not."""
+    """The last sizes that one launch sorts with four and with two blocks a chunk
+    and the first that they do not, and chunks whose last blocks are empty."""
     rng = np.random.default_rng(n)
     _same(rng.random((n, 3)) ** 3, rng.random(n), 16, 64)
 
 
-@pytest.mark.parametrize("sizes", [[1, 4096, 4097, 2, 9000], [64] * 64, [64] * 65])
+@pytest.mark.parametrize("sizes", [[1, 4096, 4097, 2, 9000], [1, 1, 4096, 4097, 2], [64] * 64, [64] * 65])
 def test_sort_of_several_systems(sizes):
     """Every system is sorted by itself, whatever its number of chunks; 64 chunks
     take the one launch and 65 do not."""
