@@ -1025,7 +1025,13 @@ __global__ void __launch_bounds__(TB) k_leaf_scatter(Cells C, const int* __restr
   }
 }
 
-__global__ void __launch_bounds__(TB) k_leaf_props(Cells C, const int* __restrict__ lorder,
+// Bound by the FP64 instructions of a warp (see k_nodes), a lane per leaf. Four
+// warps a block, one per scheduler of an SM: with eight, trees of up to a few
+// hundred thousand particles left most SMs idle. 27 -> 22 us at 5000 particles,
+// 31 -> 22 at 65,536, 39 -> 31 at 262,144; 82 at 1M either way.
+constexpr int LT_LEAF = 128;
+
+__global__ void __launch_bounds__(LT_LEAF) k_leaf_props(Cells C, const int* __restrict__ lorder,
                                                    const int* __restrict__ misc, const int* __restrict__ ni,
                                                    const double* __restrict__ xs, const double* __restrict__ ms,
                                                    Props P) {
@@ -1578,7 +1584,7 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
   int* lhist = at<int>(S, Lo.lhist);
   k_leaf_hist<<<gc, TB, 0, st>>>(C, lvl, lhist, misc, a.n_sys > 1 ? nullptr : a.cell_off);
   k_leaf_scatter<<<gc, TB, 0, st>>>(C, lvl, lhist, lhist + LBINS, lorder);
-  k_leaf_props<<<gc, TB, 0, st>>>(C, lorder, misc, ni, xs, ms, P);
+  k_leaf_props<<<grid_for(a.cap, LT_LEAF), LT_LEAF, 0, st>>>(C, lorder, misc, ni, xs, ms, P);
   OG_TRY(cudaGetLastError());
   OG_TRY(enqueue_nodes(a, Lo, C, ni, P, st));
 
@@ -1607,7 +1613,7 @@ cudaError_t gpu_refit(const GpuBuild& a, cudaStream_t st) {
   k_bbox<<<BSUB * nch, TB, 0, st>>>(a.pos, a.mass, at<Chunk>(S, Lo.chunks), at<double>(S, Lo.part), misc);
   k_gather<<<grid_for(a.n, TB), TB, 0, st>>>(at<uint32_t>(S, Lo.valA), a.pos, a.mass, a.n, at<double>(S, Lo.xs),
                                              at<double>(S, Lo.ms), a.parts, a.perm, nullptr);
-  k_leaf_props<<<gc, TB, 0, st>>>(C, at<int>(S, Lo.lorder), misc, ni, at<double>(S, Lo.xs), at<double>(S, Lo.ms), P);
+  k_leaf_props<<<grid_for(a.cap, LT_LEAF), LT_LEAF, 0, st>>>(C, at<int>(S, Lo.lorder), misc, ni, at<double>(S, Lo.xs), at<double>(S, Lo.ms), P);
   if ((e = enqueue_nodes(a, Lo, C, ni, P, st)) != cudaSuccess) return e;
   k_items<<<grid_for(a.n, TB), TB, 0, st>>>(&misc[M_NGROUPS], a.group_cell, a.group_sys, at<int>(S, Lo.ioff), P,
                                             item_args(a));
