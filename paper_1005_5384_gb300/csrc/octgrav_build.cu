@@ -578,7 +578,7 @@ __device__ void no_cells(int* lvl) {
 // barriers (5 us; the levels with tens of thousands of cells up to 20 us, where
 // a warp's cells are all split). As three launches per level for 21 levels (4096
 // blocks each, most of them empty) the levels took 425 us at 1M particles and
-// 270 us at 5000 (sum of the launches); 327 us and 84 us now.
+// 270 us at 5000 (sum of the launches); 300 us and 77 us now.
 __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ code, Cells C, int n_leaf, int* lvl,
                                                   int* spl, int* lpre, int* nlist, int* bsum, int cap, int* misc) {
   constexpr int W = LT / 32;

@@ -629,7 +629,7 @@ std::vector<int64_t> build_key(const og::GpuBuild& a) {
 
 // Enqueue a GPU build on st. The kernels are captured once into a graph and
 // replayed on the device's own stream (ordered after and before st by
-// events) while the arguments stay the same: ~125 small launches become one.
+// events) while the arguments stay the same: 13 to 35 launches become one.
 int run_build(Device& D, const og::GpuBuild& a, cudaStream_t st, bool use_graph) {
   cudaError_t e;
   if (!use_graph) {  // a one-off build: capturing would cost more than it saves
