@@ -336,7 +336,7 @@ struct Device {
 // Buffer sets of freed trees, kept for the next tree of the same device (a
 // step of a user's loop frees one tree and builds another: some 20 cudaMalloc
 // and as many cudaFree, which took 1.5 of the 6.95 ms of such a step at 1M
-// particles). give_idle waits for the device, as cudaFree does, so nothing
+// particles). give_idle waits for the device (cudaFree does), so nothing
 // uses the buffers any more whatever streams the tree ran on, and take_idle
 // hands them out once, so threads never share a set. At most two sets of at
 // most 1 GiB each are kept; they go back to the device when an allocation fails.
