@@ -9,16 +9,19 @@ namespace ogh {
 
 namespace {
 
-constexpr size_t kIdleSets = 2, kIdleBytes = size_t{1} << 30;
+constexpr int kIdleSets = 2, kIdleSlots = 16;  // sets of one context; sets of all contexts
+constexpr size_t kIdleBytes = size_t{1} << 30;
 
 struct IdleSet {
-  unsigned long long context;
+  unsigned long long context = 0;  // 0: an empty slot
+  unsigned long long age = 0;
   Device D;
 };
 std::mutex idle_mu;
-// never destroyed: the driver may be gone before static destructors run
-std::vector<IdleSet>& idle_sets() {
-  static std::vector<IdleSet>& v = *new std::vector<IdleSet>();
+unsigned long long idle_age = 0;
+// never destroyed: a tree may be freed after static destructors have run
+IdleSet* idle_sets() {
+  static IdleSet* const v = new IdleSet[kIdleSlots];
   return v;
 }
 
@@ -40,36 +43,32 @@ unsigned long long context_id() {
 
 }  // namespace
 
+// A set of the current device's current context (context id `id`), taken out
+// of its slot; false when there is none.
+static bool take_set(int device, unsigned long long id, Device& got) {
+  std::lock_guard<std::mutex> g(idle_mu);
+  IdleSet* best = nullptr;
+  for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s)
+    if (s->context == id && s->D.device == device && (!best || s->age > best->age)) best = s;
+  if (!best) return false;
+  got = std::move(best->D);
+  *best = IdleSet();
+  return true;
+}
+
 bool release_idle() {
-  std::vector<IdleSet> sets;
-  {
-    std::lock_guard<std::mutex> g(idle_mu);
-    sets.swap(idle_sets());
-  }
-  const unsigned long long id = sets.empty() ? 0 : context_id();
+  int device = -1;
+  const unsigned long long id = context_id();
+  if (!id || cudaGetDevice(&device) != cudaSuccess) return false;
   bool any = false;
-  for (IdleSet& s : sets)
-    if (s.context == id) {  // others went with their context
-      s.D.release();
-      any = true;
-    }
+  for (Device D; take_set(device, id, D); any = true) D.release();
   return any;
 }
 
 void take_idle(int device, Device& D) {
   const unsigned long long id = context_id();
   Device got;
-  {
-    std::lock_guard<std::mutex> g(idle_mu);
-    std::vector<IdleSet>& sets = idle_sets();
-    for (size_t k = sets.size(); k-- > 0;)
-      if (sets[k].D.device == device && sets[k].context == id && id) {
-        got = std::move(sets[k].D);
-        sets.erase(sets.begin() + k);
-        break;
-      }
-  }
-  if (got.device < 0) return;
+  if (!id || !take_set(device, id, got)) return;
   std::vector<DevBuf*> mine;  // what D already holds stays (a criterion set before the upload)
   D.for_each([&](DevBuf& b) { mine.push_back(&b); });
   size_t k = 0;
@@ -100,13 +99,23 @@ void give_idle(Device& D) {
   const unsigned long long id = keep ? context_id() : 0;
   if (id) {
     std::lock_guard<std::mutex> g(idle_mu);
-    std::vector<IdleSet>& sets = idle_sets();
-    for (size_t k = sets.size(); k-- > 0;)  // sets of a context that is gone
-      if (sets[k].D.device == cur && sets[k].context != id) sets.erase(sets.begin() + k);
-    if (sets.size() < kIdleSets) {
+    // a free slot, or the oldest of those that another context of the device
+    // has left (a context that is gone took its buffers with it, and only then
+    // do so many sets remain)
+    IdleSet *slot = nullptr, *other = nullptr;
+    int mine = 0;
+    for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
+      if (!s->context) slot = s;
+      else if (s->D.device == cur && s->context == id) ++mine;
+      else if (s->D.device == cur && (!other || s->age < other->age)) other = s;
+    }
+    if (!slot) slot = other;
+    if (slot && mine < kIdleSets) {
       D.release_graph();
       D.cell_cap = 0;
-      sets.push_back({id, std::move(D)});
+      slot->context = id;
+      slot->age = ++idle_age;
+      slot->D = std::move(D);
       D = Device();
       return;
     }

@@ -261,8 +261,8 @@ int build_system(const double* pos, const double* mass, int64_t n, int n_leaf, i
 
 // ---------------------------------------------------------------- device buffers
 
-// Gives the idle buffer sets (take_idle) back to the device; false when there
-// were none.
+// Gives the idle buffer sets (take_idle) of the current context back to its
+// device; false when there were none. Those of other devices and contexts stay.
 bool release_idle();
 
 struct DevBuf {

@@ -84,3 +84,54 @@ def test_freeing_a_tree_leaves_captures_alone(fake):
     T.free()
     assert fake.fake_end_capture() == 0
     assert fake.fake_frees() > frees        # the wait that stands before any reuse
+
+
+def _one_tree(n=3000, seed=1):
+    T = _upload(_tree(n, seed))
+    T.free()
+
+
+def test_a_failed_allocation_leaves_other_devices_buffers(fake):
+    """Buffers kept from a tree of device 1 survive an allocation that fails on
+    device 0, and serve device 1's next tree."""
+    fake.fake_set_device(1)
+    _one_tree()
+    kept = fake.fake_used(1)
+    assert kept > 0
+    fake.fake_set_device(0)
+    fake.fake_set_limit(0, 1 << 10)
+    T = _tree(20000)
+    assert fake.octgrav_tree_upload(T._h, None) == G.ERR_OOM
+    fake.fake_set_device(1)
+    _upload(_tree(3000))
+    assert fake.fake_used(1) <= kept + 256          # the smallest buffer had been given back
+
+
+def test_a_failed_allocation_gives_back_its_own_contexts_buffers_only(fake):
+    """Two contexts of one device."""
+    first = 1 << 20
+    fake.fake_set_context(0, first)
+    _one_tree()
+    kept = fake.fake_used(0)
+    fake.fake_set_context(0, first + 1)
+    both = [_upload(_tree(3000, seed)) for seed in (1, 2)]
+    for T in both:
+        T.free()
+    fake.fake_set_limit(0, fake.fake_used(0) + (1 << 10))
+    T = _tree(20000)                                # takes one set, needs more: the other one goes back
+    assert fake.octgrav_tree_upload(T._h, None) == G.ERR_OOM
+    assert fake.fake_used(0) < 3 * kept
+    fake.fake_set_limit(0, 1 << 40)
+    fake.fake_set_context(0, first)
+    before = fake.fake_used(0)
+    _upload(_tree(3000))
+    assert fake.fake_used(0) <= before + 256
+
+
+def test_contexts_that_are_gone_do_not_use_up_the_places(fake):
+    for k in range(40):                             # as after 40 device resets
+        fake.fake_set_context(0, (1 << 21) + k)
+        _one_tree()
+    before = fake.fake_used(0)
+    _one_tree()
+    assert fake.fake_used(0) == before
