@@ -17,6 +17,13 @@
  *    acc[3*i+k] = a_k of particle i, pot[i] = its potential.
  *  - Plummer softening eps > 0, gravitational constant G (1 by default);
  *    the self term is excluded; potentials are negative.
+ *  - Units: forces are evaluated in FP32, so choose units in which the system's
+ *    mass and size are not far from 1. For unit mass, potentials, and
+ *    accelerations at one particle per lane (octgrav_set_launch), keep FP32
+ *    accuracy for distances (softened by eps) from 1e-7 to 1e8; accelerations at
+ *    two particles per lane (the default), which go through r^-5, for distances
+ *    from 1e-7 to 1e7. Outside, terms are lost or results become infinite or NaN
+ *    without an error status.
  *  - Opening test (Sec. 2.2): a cell whose boundary-cube side l satisfies
  *    l < theta * d, with d the distance between the group's tight box and
  *    the cell's cube, is accepted as a multipole; otherwise it is opened.

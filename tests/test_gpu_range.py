@@ -44,3 +44,15 @@ def _close(a, b):
 @pytest.mark.parametrize("k", [-20, -12, 12, 24, 28])
 def test_potentials(torch, k, ppl, split):
     assert _close(_scaled(torch, k, ppl, split)[1], _scaled(torch, 0, ppl, split)[1])
+
+
+@pytest.mark.parametrize("split", [1, 4])
+@pytest.mark.parametrize("k", [-20, -12, 12, 24, 28])
+def test_accelerations_with_one_particle_per_lane(torch, k, split):
+    assert _close(_scaled(torch, k, 1, split)[0], _scaled(torch, 0, 1, split)[0])
+
+
+@pytest.mark.parametrize("k", [-16, 16])
+def test_accelerations_with_two_particles_per_lane(torch, k):
+    """The stated range of this layout: softened distances from 1e-7 up, 1e7 at most."""
+    assert _close(_scaled(torch, k, 2, 1)[0], _scaled(torch, 0, 2, 1)[0])
