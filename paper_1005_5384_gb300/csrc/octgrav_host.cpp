@@ -10,11 +10,12 @@ namespace ogh {
 namespace {
 
 constexpr int kIdleSets = 2, kIdleSlots = 16;  // sets of one context; sets of all contexts
-constexpr size_t kIdleBytes = size_t{1} << 30;
+constexpr size_t kIdleBytes = size_t{1} << 30;   // of one context's sets together
 
 struct IdleSet {
   unsigned long long context = 0;  // 0: an empty slot
   unsigned long long age = 0;
+  size_t bytes = 0;
   Device D;
 };
 std::mutex idle_mu;
@@ -95,7 +96,10 @@ void give_idle(Device& D) {
   // mode. 3.2 us with the next tree's cudaMalloc, 1.1 us for the other.
   const bool keep = least && bytes <= kIdleBytes && cudaGetDevice(&cur) == cudaSuccess && cur == D.device &&
                     cudaFree(least->p) == cudaSuccess;
-  if (keep) *least = DevBuf();
+  if (keep) {
+    bytes -= least->cap;
+    *least = DevBuf();
+  }
   const unsigned long long id = keep ? context_id() : 0;
   if (id) {
     std::lock_guard<std::mutex> g(idle_mu);
@@ -104,17 +108,19 @@ void give_idle(Device& D) {
     // do so many sets remain)
     IdleSet *slot = nullptr, *other = nullptr;
     int mine = 0;
+    size_t sum = bytes;
     for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
       if (!s->context) slot = s;
-      else if (s->D.device == cur && s->context == id) ++mine;
+      else if (s->D.device == cur && s->context == id) ++mine, sum += s->bytes;
       else if (s->D.device == cur && (!other || s->age < other->age)) other = s;
     }
     if (!slot) slot = other;
-    if (slot && mine < kIdleSets) {
+    if (slot && mine < kIdleSets && sum <= kIdleBytes) {
       D.release_graph();
       D.cell_cap = 0;
       slot->context = id;
       slot->age = ++idle_age;
+      slot->bytes = bytes;
       slot->D = std::move(D);
       D = Device();
       return;
@@ -1759,6 +1765,11 @@ int octgrav_set_staging(octgrav_tree* t, int mode) {
   if (!t) return fail(OCTGRAV_ERR_ARG, "tree is NULL");
   if (mode < og::STAGING_BULK || mode > og::STAGING_GATHER4) return fail(OCTGRAV_ERR_ARG, "staging mode must be 0, 1 or 2");
   t->stage = mode;
+  return OCTGRAV_OK;
+}
+
+int octgrav_release_buffers(void) {
+  release_idle();
   return OCTGRAV_OK;
 }
 

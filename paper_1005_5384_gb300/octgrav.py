@@ -92,6 +92,7 @@ _SIGS = {
     "octgrav_autotune_ex": (C.c_int, [C.c_int, _i64, _f64, _f64, C.c_int, C.c_double, C.c_double, _vp, C.c_int,
                                       _vp, C.c_int, _vp, _vp]),
     "octgrav_free_tree": (None, [_vp]),
+    "octgrav_release_buffers": (C.c_int, []),
     "octgrav_forces_noalloc": (C.c_int, [_vp, _vp, C.POINTER(C.c_size_t), C.c_double, C.c_double, C.c_double,
                                          _vp, _vp]),
 }
@@ -466,6 +467,12 @@ def forces(pos, mass, eps: float, theta: float, n_leaf: int = 16, n_group: int |
 ONESHOT_PHASES = ("bbox_check", "morton", "sort", "gather_records", "levels", "cell_props", "groups",
                   "records_items", "host_build", "device_upload", "device_walk_eval", "device_unpermute_copy_out",
                   "call")
+
+
+def release_buffers():
+    """Give the device buffers that the library keeps from freed trees (up to
+    1 GiB) back to the current device."""
+    _check(load().octgrav_release_buffers())
 
 
 def oneshot_phases() -> dict:

@@ -135,3 +135,22 @@ def test_contexts_that_are_gone_do_not_use_up_the_places(fake):
     before = fake.fake_used(0)
     _one_tree()
     assert fake.fake_used(0) == before
+
+
+def test_kept_buffers_are_bounded_and_given_back(fake):
+    """Two trees of about 0.6 GiB each (256 bytes a particle are the parts'
+    outputs of a launch split over 16 warps; nothing writes them here)."""
+    both = [_upload(_tree(1900000, n_group=256)) for _ in range(2)]
+    for T in both:
+        T.set_split(16)
+        _forces(T)
+    assert fake.fake_used(0) > 1 << 30
+    for T in both:
+        T.free()
+    assert 0 < fake.fake_used(0) <= 1 << 30
+    alive = _upload(_tree(3000))
+    G.release_buffers()
+    left = fake.fake_used(0)
+    alive.free()
+    G.release_buffers()
+    assert fake.fake_used(0) == 0 < left            # a tree in use had kept its own
