@@ -45,12 +45,18 @@ unsigned long long context_id() {
 }  // namespace
 
 // A set of the current device's current context (context id `id`), taken out
-// of its slot; false when there is none.
-static bool take_set(int device, unsigned long long id, Device& got) {
+// of its slot; false when there is none. With need > 0 a set that fits a tree
+// whose particle records take `need` bytes: the smallest that is large enough,
+// up to eight times as large (or 1 MiB more), so that a small tree does not hold
+// a large one's buffers while the next large one allocates again.
+static bool take_set(int device, unsigned long long id, size_t need, Device& got) {
   std::lock_guard<std::mutex> g(idle_mu);
   IdleSet* best = nullptr;
-  for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s)
-    if (s->context == id && s->D.device == device && (!best || s->age > best->age)) best = s;
+  for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
+    const size_t have = s->D.parts.cap;
+    if (s->context != id || s->D.device != device || (need && (have < need || have > 8 * need + (1 << 20)))) continue;
+    if (!best || have < best->D.parts.cap || (have == best->D.parts.cap && s->age > best->age)) best = s;
+  }
   if (!best) return false;
   got = std::move(best->D);
   *best = IdleSet();
@@ -62,14 +68,14 @@ bool release_idle() {
   const unsigned long long id = context_id();
   if (!id || cudaGetDevice(&device) != cudaSuccess) return false;
   bool any = false;
-  for (Device D; take_set(device, id, D); any = true) D.release();
+  for (Device D; take_set(device, id, 0, D); any = true) D.release();
   return any;
 }
 
-void take_idle(int device, Device& D) {
+void take_idle(int device, int64_t n, Device& D) {
   const unsigned long long id = context_id();
   Device got;
-  if (!id || !take_set(device, id, got)) return;
+  if (!id || !take_set(device, id, 2 * sizeof(float4) * static_cast<size_t>(n), got)) return;
   std::vector<DevBuf*> mine;  // what D already holds stays (a criterion set before the upload)
   D.for_each([&](DevBuf& b) { mine.push_back(&b); });
   size_t k = 0;
@@ -101,30 +107,45 @@ void give_idle(Device& D) {
     *least = DevBuf();
   }
   const unsigned long long id = keep ? context_id() : 0;
-  if (id) {
-    std::lock_guard<std::mutex> g(idle_mu);
-    // a free slot, or the oldest of those that another context of the device
-    // has left (a context that is gone took its buffers with it, and only then
-    // do so many sets remain)
-    IdleSet *slot = nullptr, *other = nullptr;
-    int mine = 0;
-    size_t sum = bytes;
-    for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
-      if (!s->context) slot = s;
-      else if (s->D.device == cur && s->context == id) ++mine, sum += s->bytes;
-      else if (s->D.device == cur && (!other || s->age < other->age)) other = s;
+  for (bool again = id != 0; again;) {
+    Device old;  // the context's oldest set makes room
+    {
+      std::lock_guard<std::mutex> g(idle_mu);
+      // a free slot, or the oldest of those that another context of the device
+      // has left (a context that is gone took its buffers with it, and only then
+      // do so many sets remain)
+      IdleSet *slot = nullptr, *other = nullptr, *oldest = nullptr;
+      int mine = 0;
+      size_t sum = bytes;
+      for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
+        if (!s->context) {
+          slot = s;
+        } else if (s->D.device == cur && s->context == id) {
+          ++mine;
+          sum += s->bytes;
+          if (!oldest || s->age < oldest->age) oldest = s;
+        } else if (s->D.device == cur && (!other || s->age < other->age)) {
+          other = s;
+        }
+      }
+      if (!slot) slot = other;
+      if (slot && mine < kIdleSets && sum <= kIdleBytes) {
+        D.release_graph();
+        D.cell_cap = 0;
+        slot->context = id;
+        slot->age = ++idle_age;
+        slot->bytes = bytes;
+        slot->D = std::move(D);
+        D = Device();
+        return;
+      }
+      again = oldest != nullptr;
+      if (again) {
+        old = std::move(oldest->D);
+        *oldest = IdleSet();
+      }
     }
-    if (!slot) slot = other;
-    if (slot && mine < kIdleSets && sum <= kIdleBytes) {
-      D.release_graph();
-      D.cell_cap = 0;
-      slot->context = id;
-      slot->age = ++idle_age;
-      slot->bytes = bytes;
-      slot->D = std::move(D);
-      D = Device();
-      return;
-    }
+    old.release();
   }
   D.release();
 }
@@ -365,7 +386,7 @@ int upload(octgrav_tree* t, cudaStream_t st) {
   if (D.device >= 0 && D.device != dev) {
     D.release();
   }
-  if (D.device < 0 && t->dev == &t->own) take_idle(dev, D);
+  if (D.device < 0 && t->dev == &t->own) take_idle(dev, t->n, D);
   D.device = dev;
   int rc;
   if (!t->gpu) {  // a GPU-built tree already lives in these arrays
@@ -542,7 +563,7 @@ int forces_host(octgrav_tree* t, double eps, double theta, double G, double* acc
   if (D.device < 0 && t->dev == &t->own) {
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
-    take_idle(dev, D);
+    take_idle(dev, t->n, D);
     D.device = dev;
   }
   if ((rc = D.acc64.reserve(24 * t->n)) || (rc = D.pot64.reserve(8 * t->n))) return rc;
@@ -735,7 +756,7 @@ int build_gpu_common(int n_sys, const int64_t* offsets, const double* pos, const
   int cur = 0;
   CUDA_TRY(cudaGetDevice(&cur));
   if (D.device >= 0 && D.device != cur) D.release();
-  if (!dev) take_idle(cur, D);
+  if (!dev) take_idle(cur, n, D);
   D.device = cur;
   // every level holds at most n cells (they are disjoint and non-empty)
   const int64_t bound = std::min<int64_t>(22 * n + n_sys, (1ll << 28) - 1);

@@ -338,11 +338,12 @@ struct Device {
 // and as many cudaFree, which took 1.5 of the 6.95 ms of such a step at 1M
 // particles). give_idle waits for the device (cudaFree does), so nothing
 // uses the buffers any more whatever streams the tree ran on, and take_idle
-// hands them out once, so threads never share a set. At most two sets, 1 GiB
-// together, are kept per context; they go back to the device when an allocation
+// hands them out once, to a tree of n particles that the set fits, so threads never
+// share a set. At most two sets, 1 GiB
+// together, are kept per context, the newest; they go back to the device when an allocation
 // fails and by octgrav_release_buffers. A set is only taken in the context it was
 // allocated in.
-void take_idle(int device, Device& D);
+void take_idle(int device, int64_t n, Device& D);
 void give_idle(Device& D);
 
 }  // namespace ogh

@@ -154,3 +154,28 @@ def test_kept_buffers_are_bounded_and_given_back(fake):
     alive.free()
     G.release_buffers()
     assert fake.fake_used(0) == 0 < left            # a tree in use had kept its own
+
+
+def test_a_set_goes_to_a_tree_that_it_fits(fake):
+    """A small tree leaves a large one's buffers alone, so that the next large
+    tree allocates nothing; sets that fit no more make room for new ones."""
+    _one_tree(200000)
+    large = fake.fake_used(0)
+    small = _upload(_tree(2000))
+    own = fake.fake_used(0) - large
+    assert 0 < own < large // 8
+    T = _upload(_tree(200000))
+    assert fake.fake_used(0) <= large + own + 256   # the smallest buffer had been given back
+    T.free()
+    small.free()
+    for n in (2000, 200000, 2000, 150000):          # both sets serve again
+        before = fake.fake_used(0)
+        T = _upload(_tree(n))
+        assert fake.fake_used(0) <= before + 512
+        T.free()
+    for n in (10000, 11000, 12000, 13000):          # each too large for the last
+        _one_tree(n)
+    assert fake.fake_used(0) < large // 2           # the newest two
+    before = fake.fake_used(0)
+    _upload(_tree(13000))
+    assert fake.fake_used(0) <= before + 256
