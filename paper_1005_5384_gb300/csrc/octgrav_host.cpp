@@ -91,6 +91,7 @@ void give_idle(Device& D) {
   size_t bytes = 0;
   DevBuf* least = nullptr;
   D.dbg.release();
+  for (DevBuf& b : D.outgrown) b.release();
   D.for_each([&](DevBuf& b) {
     bytes += b.cap;
     if (b.p && (!least || b.cap < least->cap)) least = &b;
@@ -372,11 +373,32 @@ int split_parts(const octgrav_tree* t, bool capture) {
   return t->nparts > 0 ? t->nparts : auto_parts(t);
 }
 
+// Room for the outputs of `parts` parts. Launches that octgrav_graph_capture or
+// the caller has captured hold the buffer's address, so one that is too small
+// stays until its tree is freed. A tree has at most 16 sizes of it (one per
+// number of parts); the sets of the one-shot calls and of the integrator, whose
+// trees nobody captures, keep the last one only.
+int reserve_split(octgrav_tree* t, int parts) {
+  Device& D = *t->dev;
+  const size_t bytes = sizeof(float4) * parts * static_cast<size_t>(t->n);
+  if (t->dev == &t->own && D.split.p && bytes > D.split.cap) {
+    DevBuf* const end = D.outgrown + sizeof(D.outgrown) / sizeof(D.outgrown[0]);
+    DevBuf* const place = std::find_if(D.outgrown, end, [](const DevBuf& b) { return !b.p; });
+    if (place == end) return fail(OCTGRAV_ERR_STATE, "no place for another size of the parts' outputs");
+    DevBuf larger;
+    if (int rc = larger.reserve(bytes)) return rc;
+    *place = D.split;
+    D.split = larger;
+    return OCTGRAV_OK;
+  }
+  return D.split.reserve(bytes);
+}
+
 // The parts' outputs, reserved where the work items are made, so that a launch
 // (which may be in a stream capture) allocates nothing.
 int reserve_parts(octgrav_tree* t) {
   const int parts = split_parts(t, false);
-  return parts > 1 ? t->dev->split.reserve(sizeof(float4) * parts * static_cast<size_t>(t->n)) : OCTGRAV_OK;
+  return parts > 1 ? reserve_split(t, parts) : OCTGRAV_OK;
 }
 
 int upload(octgrav_tree* t, cudaStream_t st) {
@@ -489,7 +511,7 @@ int launch(octgrav_tree* t, double eps, double theta, double G, float4* out, cud
   CUDA_TRY(cudaMemsetAsync(t->dev->ctl.p, 0, 8, st));
   const int nparts = split_parts(t, capture);
   if (nparts > 1) {  // the parts' outputs are summed into out below; counts are accumulated
-    if ((rc = t->dev->split.reserve(sizeof(float4) * nparts * static_cast<size_t>(t->n)))) return rc;
+    if ((rc = reserve_split(t, nparts))) return rc;
     p.nparts = nparts;
     p.n = static_cast<int>(t->n);
     p.part_out = static_cast<float4*>(t->dev->split.p);
@@ -1562,7 +1584,7 @@ int octgrav_graph_capture(octgrav_tree* t, double eps, double theta, double G, f
   }
   CUDA_TRY(cudaStreamSynchronize(st));  // uploads from pageable memory cannot be captured
   if (const int np = split_parts(t, false); np > 1) {  // allocate outside the capture
-    if ((rc = t->dev->split.reserve(sizeof(float4) * np * static_cast<size_t>(t->n)))) return rc;
+    if ((rc = reserve_split(t, np))) return rc;
   }
   og::LaunchInfo li;
   cudaError_t e = og::prepare_walk_eval(t->ppl, t->stage, split_parts(t, false), t->ctas_per_sm, &li);

@@ -299,7 +299,9 @@ struct Device {
   // GPU build: tree arrays beyond the walk's, scratch, inputs and FP64 outputs
   DevBuf perm, key, props, pcount, cfirst, groups, ikey, celloff, result, scratch, in_pos, in_mass, acc64, pot64;
   DevBuf order;  // work-item processing order (octgrav_balance)
-  DevBuf split;  // per-part outputs of a list-split launch (octgrav_set_split)
+  DevBuf split;  // per-part outputs of a list-split launch (reserve_split)
+  // earlier ones that were too small for more parts: captured launches write them
+  DevBuf outgrown[16];
   int device = -1;
   int pageable = -1;     // kernels may read pageable host memory (-1: not asked yet)
   int64_t cell_cap = 0;  // cell capacity that last sufficed for a GPU build
@@ -322,6 +324,7 @@ struct Device {
     gstream = nullptr;
     ev_in = ev_out = nullptr;
     for_each([](DevBuf& b) { b.release(); });
+    for (DevBuf& b : outgrown) b.release();
     cell_cap = 0;
   }
   template <class F>

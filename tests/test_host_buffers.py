@@ -179,3 +179,32 @@ def test_a_set_goes_to_a_tree_that_it_fits(fake):
     before = fake.fake_used(0)
     _upload(_tree(13000))
     assert fake.fake_used(0) <= before + 256
+
+
+@pytest.mark.parametrize("own", [False, True])
+def test_captured_launches_keep_the_buffer_they_write(fake, own):
+    """A launch captured with the parts that a small tree chooses itself, by
+    octgrav_graph_capture or by the caller, writes a buffer that is still there
+    after launches with more parts."""
+    T = _upload(_tree(3000))
+    _forces(T)
+    auto = _last(fake)["nparts"]
+    assert auto > 1
+    if own:
+        fake.fake_begin_capture()
+        _forces(T)
+        fake.fake_end_capture()
+    else:
+        G._check(fake.octgrav_graph_capture(T._h, 0.01, 0.5, 1.0, C.c_void_p(256), C.c_void_p(1)))
+    for parts in range(1, 17):
+        T.set_split(parts)
+        _forces(T)
+        assert _last(fake)["nparts"] == parts
+        if own:
+            assert fake.fake_replay() == 0
+        else:
+            G._check(fake.octgrav_graph_launch(T._h, None))
+    assert fake.fake_dangling() == 0
+    T.free()
+    G.release_buffers()
+    assert fake.fake_used(0) == 0
