@@ -493,9 +493,10 @@ int octgrav_set_fault(octgrav_tree *t, int stack_cap, int64_t drop_item);
  * in part order by a second kernel, so a launch is deterministic but rounds
  * differently from an unsplit one (a sum of nparts FP32 results). Until this is
  * called a tree of at most 3200 work items is split over 2, 4 or 8 warps by
- * their number and the particles in each. Applies to launches with the plain
- * opening test that capture no lists; others run unsplit. A captured graph keeps
- * the split it was captured with. Errors: ERR_ARG. */
+ * their number and the particles in each, with any staging mode. Applies to
+ * launches with the plain opening test and staging mode 1 that capture no lists;
+ * others run unsplit. A captured graph keeps the split it was captured with.
+ * Errors: ERR_ARG. */
 int octgrav_set_split(octgrav_tree *t, int nparts);
 
 /* Free a tree. Waits until the current device has finished with its buffers. */

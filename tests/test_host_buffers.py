@@ -208,3 +208,14 @@ def test_captured_launches_keep_the_buffer_they_write(fake, own):
     T.free()
     G.release_buffers()
     assert fake.fake_used(0) == 0
+
+
+@pytest.mark.parametrize("stage", [0, 1, 2])
+def test_a_split_that_was_asked_for_runs_with_staging_mode_1(fake, stage):
+    T = _upload(_tree(3000))
+    T.set_staging(stage)
+    _forces(T)
+    assert _last(fake) == dict(nparts=8, stage=stage, ppl=2)      # the automatic split: any mode
+    T.set_split(4)
+    _forces(T)
+    assert _last(fake) == dict(nparts=4 if stage == 1 else 1, stage=stage, ppl=2)
