@@ -1495,8 +1495,9 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   const bool from_device = t->gpu;
   const size_t n = static_cast<size_t>(t->n), nc = static_cast<size_t>(t->n_cells),
                ni = static_cast<size_t>(t->n_items);
-  // a few work items run split, as a launch does until octgrav_set_split is called
-  const int nparts = t->learned ? 1 : auto_parts(t);
+  // a few work items run split, as a launch does until octgrav_set_split is called,
+  // unless that call has turned the split off
+  const int nparts = t->learned || t->nparts == 1 ? 1 : auto_parts(t);
   // arena layout: the device arrays, each starting on a 256-byte boundary
   const size_t sizes[8] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
                            4 * nc * sizeof(float4), ni * sizeof(int4),      4 * ni * sizeof(float4),

@@ -219,3 +219,29 @@ def test_a_split_that_was_asked_for_runs_with_staging_mode_1(fake, stage):
     T.set_split(4)
     _forces(T)
     assert _last(fake) == dict(nparts=4 if stage == 1 else 1, stage=stage, ppl=2)
+
+
+def _noalloc(lib, T, size=None):
+    """Runs octgrav_forces_noalloc in an arena of `size` bytes (default: what it
+    asks for) and returns its status."""
+    need = C.c_size_t(0)
+    G._check(lib.octgrav_forces_noalloc(T._h, None, C.byref(need), 1.0, 0.5, 1.0, None, None))
+    arena = np.empty(need.value + 256, np.uint8)
+    start = -arena.ctypes.data % 256
+    have = C.c_size_t(need.value if size is None else size)
+    return lib.octgrav_forces_noalloc(T._h, C.c_void_p(arena.ctypes.data + start), C.byref(have), 0.01, 0.5, 1.0,
+                                      C.c_void_p(256), None)
+
+
+def test_noalloc_runs_as_a_launch_does(fake):
+    """Split as a launch of the same tree chooses itself, unsplit where that was
+    turned off."""
+    T = _upload(_tree(3000))
+    _forces(T)
+    auto = _last(fake)["nparts"]
+    assert auto > 1
+    for asked, runs in ((None, auto), (4, auto), (1, 1)):
+        if asked:
+            T.set_split(asked)
+        assert _noalloc(fake, T) == G.OK
+        assert _last(fake)["nparts"] == runs
