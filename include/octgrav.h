@@ -525,12 +525,11 @@ int octgrav_release_buffers(void);
  * particles per lane, per-system parameters and the learned criterion (whose
  * network stays in the tree's device memory; set it on the current device) --
  * except a list split over two or more warps asked for with octgrav_set_split:
- * these launches run as octgrav_forces_device does where that was not called
- * (the parts' outputs of a small tree are in the arena). With
- * octgrav_set_split(t, 1) both run unsplit.
- * The status word, work-queue counter and per-item counts live in a
- * fixed-size array inside the library (2 MiB + 256 B per GPU, kept until the
- * process exits), so the tree may have at most OCTGRAV_NOALLOC_MAX_ITEMS work
+ * these launches run as octgrav_forces_device does where that was not called.
+ * With octgrav_set_split(t, 1) both run unsplit.
+ * The status word, work-queue counter, per-item counts and the parts' outputs of
+ * a small tree's split live in a fixed-size array inside the library (8.7 MB per
+ * GPU, kept until the process exits), so the tree may have at most OCTGRAV_NOALLOC_MAX_ITEMS work
  * items (octgrav_tree_stats out[4]); larger trees get ERR_ARG. The first call
  * on a device looks up that array's address with the device current; make it
  * before any stream capture. All calls share the array: calls that overlap on

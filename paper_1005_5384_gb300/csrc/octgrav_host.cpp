@@ -362,7 +362,7 @@ int auto_parts(const octgrav_tree* t) {
   if (t->n < 6 * items || t->n < 1000 * static_cast<int64_t>(t->n_sys)) return 1;
   const double fill = std::min(1.0, static_cast<double>(t->n) / (19.0 * static_cast<double>(items)));
   const auto fits = [&](int parts, int most) { return static_cast<double>(items * parts) <= fill * most; };
-  return fits(8, 4640) ? 8 : fits(4, 5200) ? 4 : fits(2, 6400) ? 2 : 1;
+  return fits(8, 4640) ? 8 : fits(4, 5200) ? 4 : fits(2, og::AUTO_SPLIT_MOST) ? 2 : 1;
 }
 
 // Parts of a list-split launch of t (1: no split): launches with the plain
@@ -1499,11 +1499,11 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   // unless that call has turned the split off
   const int nparts = t->learned || t->nparts == 1 ? 1 : auto_parts(t);
   // arena layout: the device arrays, each starting on a 256-byte boundary
-  const size_t sizes[8] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
+  const size_t sizes[7] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
                            4 * nc * sizeof(float4), ni * sizeof(int4),      4 * ni * sizeof(float4),
-                           t->sysp.size() * sizeof(float4), nparts > 1 ? nparts * n * sizeof(float4) : 0};
-  size_t offs[8], total = 0;
-  for (int k = 0; k < 8; ++k) {
+                           t->sysp.size() * sizeof(float4)};
+  size_t offs[7], total = 0;
+  for (int k = 0; k < 7; ++k) {
     offs[k] = total;
     total += (sizes[k] + 255) & ~static_cast<size_t>(255);
   }
@@ -1556,7 +1556,6 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
   p.n_group = t->n_group;
   p.nparts = nparts;
   p.n = static_cast<int>(n);
-  p.part_out = reinterpret_cast<float4*>(a + offs[7]);
   if (t->learned) {  // the network stays in the tree's own device memory (set_criterion)
     p.mlp = static_cast<const og::MlpDevice*>(t->dev->mlp.p);
     p.theta_lo2 = static_cast<float>(static_cast<double>(t->theta_lo) * t->theta_lo);

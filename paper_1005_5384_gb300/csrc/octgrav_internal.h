@@ -181,12 +181,16 @@ cudaError_t mlp_train_steps(float* w, float* m, float* v, const float* X, const 
 // used by the gather4 staging. Returns cudaSuccess or an error.
 cudaError_t encode_mp_map(CUtensorMap* map, const void* mp, int n_cells);
 
+// Work items x parts of a launch that chooses its list split itself (auto_parts
+// in octgrav_host.cpp), at most.
+constexpr int AUTO_SPLIT_MOST = 6400;
+
 // Allocation-free launch: like launch_walk_eval, but the status word, the
-// work-queue counter and the per-item counts live in a file-scope device
-// array (no cudaMalloc). p.status, p.work and p.counts are ignored (a list
-// split's part_out is the caller's); p.n_items
-// must not exceed OCTGRAV_NOALLOC_MAX_ITEMS. Waits for the stream and returns
-// the device status bits in *status_bits.
+// work-queue counter, the per-item counts and the parts' outputs of a list split
+// live in a file-scope device array (no cudaMalloc). p.status, p.work, p.counts
+// and p.part_out are ignored; p.n_items must not exceed OCTGRAV_NOALLOC_MAX_ITEMS,
+// and p.nparts x p.n OCTGRAV_MAX_ITEM x AUTO_SPLIT_MOST where p.nparts > 1.
+// Waits for the stream and returns the device status bits in *status_bits.
 cudaError_t launch_walk_eval_noalloc(KParams p, int ppl, int ctas_per_sm, cudaStream_t stream,
                                      int* status_bits);
 

@@ -1357,13 +1357,17 @@ cudaError_t prepare_walk_eval(int ppl, int stage, int nparts, int ctas_per_sm, L
 // Scratch of octgrav_forces_noalloc, for callers that must not allocate device
 // memory themselves or have the library do it (see include/octgrav.h).
 // Layout: bytes 0..3 status word, 4..7 work-queue counter, 256.. per-item
-// interaction counts (int2) for at most OCTGRAV_NOALLOC_MAX_ITEMS items
-// (2 MiB + 256 B in total). Every GPU that loads the library keeps this array
+// interaction counts (int2) for at most OCTGRAV_NOALLOC_MAX_ITEMS items, then the
+// parts' outputs (float4) of the largest automatic list split, which so takes
+// no room in the caller's arena (8.7 MB in total). Every GPU that loads the library keeps this array
 // until the process exits. All calls share it: calls that overlap on the GPU
 // (two streams, or two threads) race on it and give wrong results.
 namespace {
 constexpr size_t kNoAllocHeader = 256;
-constexpr size_t kNoAllocBytes = kNoAllocHeader + sizeof(int2) * OCTGRAV_NOALLOC_MAX_ITEMS;
+constexpr size_t kNoAllocParts = kNoAllocHeader + sizeof(int2) * OCTGRAV_NOALLOC_MAX_ITEMS;
+constexpr int64_t kNoAllocOutputs = int64_t{OCTGRAV_MAX_ITEM} * AUTO_SPLIT_MOST;
+constexpr size_t kNoAllocBytes = kNoAllocParts + sizeof(float4) * kNoAllocOutputs;
+static_assert(kNoAllocParts % sizeof(float4) == 0, "the parts' outputs are aligned");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 constexpr int kMaxDevices = 64;
@@ -1414,6 +1418,7 @@ cudaError_t noalloc_scratch(void** out) {
 cudaError_t launch_walk_eval_noalloc(KParams p, int ppl, int ctas_per_sm, cudaStream_t stream,
                                      int* status_bits) {
   if (p.n_items < 0 || p.n_items > OCTGRAV_NOALLOC_MAX_ITEMS) return cudaErrorInvalidValue;
+  if (p.nparts > 1 && static_cast<int64_t>(p.nparts) * p.n > kNoAllocOutputs) return cudaErrorInvalidValue;
   void* base = nullptr;
   cudaError_t e = noalloc_scratch(&base);
   if (e != cudaSuccess) return e;
@@ -1421,6 +1426,7 @@ cudaError_t launch_walk_eval_noalloc(KParams p, int ppl, int ctas_per_sm, cudaSt
   p.status = reinterpret_cast<int*>(b);
   p.work = reinterpret_cast<unsigned*>(b + 4);
   p.counts = reinterpret_cast<int2*>(b + kNoAllocHeader);
+  p.part_out = reinterpret_cast<float4*>(b + kNoAllocParts);
   // the array keeps the previous call's contents: the status word and the
   // work counter must start at zero
   if ((e = cudaMemsetAsync(b, 0, 8, stream)) != cudaSuccess) return e;

@@ -233,6 +233,18 @@ def _noalloc(lib, T, size=None):
                                       C.c_void_p(256), None)
 
 
+def test_noalloc_arena_holds_the_tree_alone(fake):
+    """The arena's size depends on the tree, not on the split that it runs with,
+    so one sized for a tree of as many cells and items serves."""
+    T = _upload(_tree(3000))
+    need = T.noalloc_arena_bytes()
+    T.set_split(1)
+    assert T.noalloc_arena_bytes() == need
+    s = T.stats
+    arrays = [32 * s["n"], 16 * s["n_cells"], 8 * s["n_cells"], 64 * s["n_cells"], 16 * s["n_items"], 64 * s["n_items"]]
+    assert need == sum(-(-a // 256) * 256 for a in arrays)
+
+
 def test_noalloc_runs_as_a_launch_does(fake):
     """Split as a launch of the same tree chooses itself, unsplit where that was
     turned off."""
