@@ -1737,7 +1737,8 @@ static int autotune_common(int n_sys, const int64_t* offsets, const double* pos,
   // keeps per-lane cp.async staging)
   if (rc == OCTGRAV_OK && tune_staging && bng >= 0 && bsplit == 1) {
     octgrav_tree* t = nullptr;
-    if (!(rc = build_common(n_sys, offsets, pos, mass, n_leaf, bng, &t)) && !(rc = octgrav_set_launch(t, bppl, 0))) {
+    if (!(rc = build_common(n_sys, offsets, pos, mass, n_leaf, bng, &t)) && !(rc = octgrav_set_launch(t, bppl, 0)) &&
+        !(rc = octgrav_set_split(t, bsplit))) {
       for (int stage : {og::STAGING_BULK, og::STAGING_GATHER4}) {
         double ms = 0;
         if ((rc = octgrav_set_staging(t, stage)) || (rc = time_tree(t, &ms))) break;

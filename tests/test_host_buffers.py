@@ -257,3 +257,15 @@ def test_noalloc_runs_as_a_launch_does(fake):
             T.set_split(asked)
         assert _noalloc(fake, T) == G.OK
         assert _last(fake)["nparts"] == runs
+
+
+def test_autotuner_times_the_staging_modes_unsplit(fake):
+    """An unsplit winner's staging modes are tried as it runs: unsplit. (By the
+    stand-in clock unsplit launches are the fastest with mode 1, and split ones
+    would be faster still with mode 0.)"""
+    for stage in (0, 1, 2):
+        fake.fake_set_time(1, stage, 0.5 if stage == 1 else 0.75)
+        for parts in (2, 4, 8):
+            fake.fake_set_time(parts, stage, 0.125 if stage == 0 else 1.0)
+    best = G.autotune([W.plummer(3000, seed=5)], 16, 0.01, 0.5, candidates=(64,))
+    assert best == dict(n_group=64, particles_per_lane=1, split=1, staging=1, ms=0.5)
