@@ -493,10 +493,11 @@ int octgrav_set_fault(octgrav_tree *t, int stack_cap, int64_t drop_item);
  * in part order by a second kernel, so a launch is deterministic but rounds
  * differently from an unsplit one (a sum of nparts FP32 results). Until this is
  * called a tree of at most 3200 work items is split over 2, 4 or 8 warps by
- * their number and the particles in each, with any staging mode. Applies to
- * launches with the plain opening test and staging mode 1 that capture no lists;
- * others run unsplit. A captured graph keeps the split it was captured with.
- * Errors: ERR_ARG. */
+ * their number, the particles in each, the particles per lane and theta, with any
+ * staging mode; with fewer than 6 particles an item (more beyond theta = 0.6) or
+ * 1000 a system it is not. A split that was asked for applies to staging mode 1.
+ * Launches with the learned criterion and those that capture lists run unsplit. A
+ * captured graph keeps the split it was captured with. Errors: ERR_ARG. */
 int octgrav_set_split(octgrav_tree *t, int nparts);
 
 /* Free a tree. Waits until the current device has finished with its buffers. */

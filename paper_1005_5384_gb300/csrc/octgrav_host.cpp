@@ -346,7 +346,7 @@ int build_oneshot(const double* pos, const double* mass, int64_t n, int n_leaf, 
 // Parts that fill the GPU's 2432 warp slots for a tree of few work items. Every
 // part repeats the item's walk, so a split pays where the evaluation outweighs
 // it: with many particles per item and long lists. Times of 1 / 2 / 4 / 8 parts
-// (us, theta 0.6):
+// (us, theta 0.6, two particles per lane):
 //   26 particles an item   92 items  69 / 51 / 39 / 34    652 222 / 162 / 148 / 161
 //                        1253 315 / 281 / 239 / 332      2770 521 / 432 / 558 / 824
 //   15                    318 142 / 96 / 74 / 62         2317 283 / 257 / 344 / 517
@@ -357,21 +357,44 @@ int build_oneshot(const double* pos, const double* mass, int64_t n, int n_leaf, 
 // 3236 items two parts gain 1.10x, at 3550 they lose 3 %); with fewer they fall
 // in proportion, and below 6 particles an item or 1000 a system there is no
 // split (550 particles in 79 items: 23 us alone, 28 in eight parts).
-int auto_parts(const octgrav_tree* t) {
+// A wider opening angle shortens the lists and not the walk as much, so beyond
+// theta = 0.6 an item needs more particles to be worth a split; so it does with
+// one particle per lane, whose items are walked as often for half the
+// particles. Without these two terms, drawn from 855 and 642 trees and
+// angles (8 sizes, 4 distributions, N_group 16 to 256, theta 0.3 to 2.5):
+//   928 items of 6.5, 1 / 2 parts   theta 0.6: 49 / 50   1.0: 31 / 37   2.5: 23 / 31
+//   2442 items of 16.4              theta 0.6: 300 / 277 1.0: 130 / 135 2.0: 78 / 87
+//   2550 of 15.7, one per lane      theta 0.5: 358 / 364 1.0: 130 / 147 2.0: 78 / 92
+// the choice lost more than 1.5 % to an unsplit launch in 50 and 86 of them, by
+// 25 and 18 % at worst; with them in 5 and 15, by 8 and 7 %. On other particles
+// and sizes (620 and 610): 44 and 73 before, 9 and 13 now, the worst (17 %) 949
+// items of 6.3 in star clusters, whose lists are short at any angle. The gain over
+// unsplit launches is 1.3x and 1.18x in the mean either way.
+int auto_parts(const octgrav_tree* t, double theta) {
   const int64_t items = t->n_items;
-  if (t->n < 6 * items || t->n < 1000 * static_cast<int64_t>(t->n_sys)) return 1;
-  const double fill = std::min(1.0, static_cast<double>(t->n) / (19.0 * static_cast<double>(items)));
+  const double n = static_cast<double>(t->n), wide = theta > 0.6001 ? 0.6 / theta : 1.0;
+  if (n * std::pow(wide, 0.75) < static_cast<double>(6 * items) || t->n < 1000 * static_cast<int64_t>(t->n_sys)) return 1;
+  double fill = std::min(1.0, std::sqrt(wide) * n / (19.0 * static_cast<double>(items)));
+  if (t->ppl == 1 && theta > 0.5001) fill *= std::pow(0.5 / theta, 0.7);
   const auto fits = [&](int parts, int most) { return static_cast<double>(items * parts) <= fill * most; };
   return fits(8, 4640) ? 8 : fits(4, 5200) ? 4 : fits(2, og::AUTO_SPLIT_MOST) ? 2 : 1;
+}
+
+// The widest opening angle of a launch of t with the scalar argument theta.
+double widest(const octgrav_tree* t, double theta) {
+  if (t->sysp.empty()) return theta;
+  float theta2 = 0.f;
+  for (const float4& s : t->sysp) theta2 = std::max(theta2, s.x);
+  return std::sqrt(static_cast<double>(theta2));
 }
 
 // Parts of a list-split launch of t (1: no split): launches with the plain
 // criterion that capture no lists split, by auto_parts or as octgrav_set_split
 // said; the latter with staging mode 1 only, as it always did (65,537 particles in
 // 2527 items asked for in 16 parts: 0.65 ms unsplit with mode 0, 1.65 ms split).
-int split_parts(const octgrav_tree* t, bool capture) {
+int split_parts(const octgrav_tree* t, bool capture, double theta) {
   if (capture || t->learned) return 1;
-  if (t->nparts == 0) return auto_parts(t);
+  if (t->nparts == 0) return auto_parts(t, widest(t, theta));
   return t->stage == og::STAGING_ASYNC ? t->nparts : 1;
 }
 
@@ -397,9 +420,10 @@ int reserve_split(octgrav_tree* t, int parts) {
 }
 
 // The parts' outputs, reserved where the work items are made, so that a launch
-// (which may be in a stream capture) allocates nothing.
+// (which may be in a stream capture) allocates nothing; for theta = 0, which takes
+// the most parts.
 int reserve_parts(octgrav_tree* t) {
-  const int parts = split_parts(t, false);
+  const int parts = t->nparts == 0 && !t->learned ? auto_parts(t, 0.0) : split_parts(t, false, 0.0);
   return parts > 1 ? reserve_split(t, parts) : OCTGRAV_OK;
 }
 
@@ -511,7 +535,7 @@ int launch(octgrav_tree* t, double eps, double theta, double G, float4* out, cud
     p.dbg_net_cap = cap->net_cap;
   }
   CUDA_TRY(cudaMemsetAsync(t->dev->ctl.p, 0, 8, st));
-  const int nparts = split_parts(t, capture);
+  const int nparts = split_parts(t, capture, theta);
   if (nparts > 1) {  // the parts' outputs are summed into out below; counts are accumulated
     if ((rc = reserve_split(t, nparts))) return rc;
     p.nparts = nparts;
@@ -1497,7 +1521,7 @@ int octgrav_forces_noalloc(octgrav_tree* t, void* arena, size_t* arena_bytes, do
                ni = static_cast<size_t>(t->n_items);
   // a few work items run split, as a launch does until octgrav_set_split is called,
   // unless that call has turned the split off
-  const int nparts = t->learned || t->nparts == 1 ? 1 : auto_parts(t);
+  const int nparts = t->learned || t->nparts == 1 ? 1 : auto_parts(t, widest(t, theta));
   // arena layout: the device arrays, each starting on a 256-byte boundary
   const size_t sizes[7] = {2 * n * sizeof(float4), nc * sizeof(float4),     nc * sizeof(int2),
                            4 * nc * sizeof(float4), ni * sizeof(int4),      4 * ni * sizeof(float4),
@@ -1585,11 +1609,11 @@ int octgrav_graph_capture(octgrav_tree* t, double eps, double theta, double G, f
     if ((rc = upload(t, st))) return rc;
   }
   CUDA_TRY(cudaStreamSynchronize(st));  // uploads from pageable memory cannot be captured
-  if (const int np = split_parts(t, false); np > 1) {  // allocate outside the capture
+  if (const int np = split_parts(t, false, theta); np > 1) {  // allocate outside the capture
     if ((rc = reserve_split(t, np))) return rc;
   }
   og::LaunchInfo li;
-  cudaError_t e = og::prepare_walk_eval(t->ppl, t->stage, split_parts(t, false), t->ctas_per_sm, &li);
+  cudaError_t e = og::prepare_walk_eval(t->ppl, t->stage, split_parts(t, false, theta), t->ctas_per_sm, &li);
   if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "kernel preparation failed: %s", cudaGetErrorString(e));
   CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   rc = launch(t, eps, theta, G, reinterpret_cast<float4*>(acc4_dev), st);

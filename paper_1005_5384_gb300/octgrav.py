@@ -290,7 +290,8 @@ class Tree:
     def set_split(self, nparts: int = 1):
         """Walk every work item with nparts warps, each evaluating a share of the
         lists (small systems; 1 = off). Until this is called launches choose by
-        the number of work items (up to 3200: 2, 4 or 8 warps) and their size."""
+        the number of work items (up to 3200: 2, 4 or 8 warps), their size, the
+        particles per lane and theta."""
         _check(load().octgrav_set_split(self._h, int(nparts)))
 
     def set_fault(self, stack_cap: int = 0, drop_item: int = -1):

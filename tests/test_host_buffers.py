@@ -221,15 +221,14 @@ def test_a_split_that_was_asked_for_runs_with_staging_mode_1(fake, stage):
     assert _last(fake) == dict(nparts=4 if stage == 1 else 1, stage=stage, ppl=2)
 
 
-def _noalloc(lib, T, size=None):
-    """Runs octgrav_forces_noalloc in an arena of `size` bytes (default: what it
-    asks for) and returns its status."""
+def _noalloc(lib, T, theta=0.5):
+    """Runs octgrav_forces_noalloc in an arena of the size it asks for and returns
+    its status."""
     need = C.c_size_t(0)
     G._check(lib.octgrav_forces_noalloc(T._h, None, C.byref(need), 1.0, 0.5, 1.0, None, None))
     arena = np.empty(need.value + 256, np.uint8)
     start = -arena.ctypes.data % 256
-    have = C.c_size_t(need.value if size is None else size)
-    return lib.octgrav_forces_noalloc(T._h, C.c_void_p(arena.ctypes.data + start), C.byref(have), 0.01, 0.5, 1.0,
+    return lib.octgrav_forces_noalloc(T._h, C.c_void_p(arena.ctypes.data + start), C.byref(need), 0.01, theta, 1.0,
                                       C.c_void_p(256), None)
 
 
@@ -269,3 +268,48 @@ def test_autotuner_times_the_staging_modes_unsplit(fake):
             fake.fake_set_time(parts, stage, 0.125 if stage == 0 else 1.0)
     best = G.autotune([W.plummer(3000, seed=5)], 16, 0.01, 0.5, candidates=(64,))
     assert best == dict(n_group=64, particles_per_lane=1, split=1, staging=1, ms=0.5)
+
+
+def _parts(items, n, theta, ppl):
+    """The rule of the automatic split, restated."""
+    wide = min(1.0, 0.6 / theta) if theta else 1.0
+    if n * wide ** 0.75 < 6 * items or n < 1000:
+        return 1
+    fill = min(1.0, n / items * wide ** 0.5 / 19)
+    if ppl == 1 and theta > 0.5:
+        fill *= (0.5 / theta) ** 0.7
+    return next((p for p, most in ((8, 4640), (4, 5200), (2, 6400)) if items * p <= fill * most), 1)
+
+
+@pytest.mark.parametrize("n,n_group,ppl", [(5003, 32, 2), (40000, 64, 2), (40000, 64, 1), (20000, 256, 1), (3000, 64, 2),
+                                           (1100, 32, 1)])
+def test_parts_by_opening_angle(fake, n, n_group, ppl):
+    """The parts that launches choose as theta grows; all of them are reserved with
+    the upload, so that a launch in a capture allocates nothing."""
+    T = _tree(n, n_group=n_group)
+    T.set_launch(ppl)
+    _upload(T)
+    used = fake.fake_used(0)
+    items = T._stats()["n_items"]
+    seen = []
+    for theta in (2.5, 1.6, 1.2, 1.0, 0.9, 0.8, 0.7, 0.6, 0.5, 0.3, 0.0):
+        _forces(T, theta)
+        seen.append(_last(fake)["nparts"])
+        assert seen[-1] == _parts(items, n, theta, ppl)
+        assert _noalloc(fake, T, theta=theta) == G.OK and _last(fake)["nparts"] == seen[-1]
+    assert seen == sorted(seen) and fake.fake_used(0) == used
+    if n in (5003, 40000):
+        assert seen[0] == 1 < seen[-1]              # 8 and 16 particles an item: not split at wide angles
+
+
+def test_parts_of_a_batch_follow_its_widest_angle(fake):
+    systems = [W.plummer(4000, seed=k) for k in (1, 2)]
+    _made.append(G.Tree.build_batch(systems, 16, 32))
+    T = _upload(_made[-1])
+    _forces(T, 0.5)
+    narrow = _last(fake)["nparts"]
+    for theta, parts in (([0.5, 0.5], narrow), ([0.5, 2.5], 1)):
+        T.set_system_params([0.01, 0.01], theta)
+        _forces(T, 0.3)
+        assert _last(fake)["nparts"] == parts
+    assert narrow > 1
