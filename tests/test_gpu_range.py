@@ -56,3 +56,23 @@ def test_accelerations_with_one_particle_per_lane(torch, k, split):
 def test_accelerations_with_two_particles_per_lane(torch, k):
     """The stated range of this layout: softened distances from 1e-7 up, 1e7 at most."""
     assert _close(_scaled(torch, k, 2, 1)[0], _scaled(torch, 0, 2, 1)[0])
+
+
+@pytest.mark.parametrize("split", [2, 4, 16])
+def test_results_beyond_the_largest_number_are_infinite(torch, split):
+    """G (finite in FP32: the mass is 16) times a potential that overflows, and
+    parts whose sum does."""
+    pos, m = W.plummer(5000, seed=3)
+    T = G.Tree.build(pos, 16.0 * m, 16, 64)
+    T.set_split(1)
+    out = torch.empty((T.n, 4), dtype=torch.float32, device="cuda")
+    T.forces_device(0.01, 0.5, out)
+    phi = out[:, 3].double().cpu().numpy()
+    big = 3.4028235e38
+    g = 1.2 * big / float(np.abs(phi).max())        # some potentials beyond the range, their parts mostly within
+    T.set_split(split)
+    T.forces_device(0.01, 0.5, out, G=g)
+    got = out[:, 3].cpu().numpy()
+    beyond = g * np.abs(phi) > 1.00001 * big
+    within = g * np.abs(phi) < 0.99999 * big
+    assert g < big and beyond.any() and np.isneginf(got[beyond]).all() and np.isfinite(got[within]).all()
