@@ -26,6 +26,8 @@ IdleSet* idle_sets() {
   return v;
 }
 
+}  // namespace
+
 // Identity of the current context, never used twice (0: unknown). A context
 // made anew after cudaDeviceReset has another one.
 unsigned long long context_id() {
@@ -41,8 +43,6 @@ unsigned long long context_id() {
   unsigned long long id = 0;
   return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;  // NULL: the calling thread's current context
 }
-
-}  // namespace
 
 // A set of the current device's current context (context id `id`), taken out
 // of its slot; false when there is none. With need > 0 a set that fits a tree
@@ -1840,6 +1840,7 @@ int octgrav_set_staging(octgrav_tree* t, int mode) {
 
 int octgrav_release_buffers(void) {
   release_idle();
+  release_training_scratch();
   return OCTGRAV_OK;
 }
 

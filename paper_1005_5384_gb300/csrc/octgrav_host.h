@@ -261,6 +261,11 @@ int build_system(const double* pos, const double* mass, int64_t n, int n_leaf, i
 
 // ---------------------------------------------------------------- device buffers
 
+// Identity of the current context, never used twice (0: unknown).
+unsigned long long context_id();
+// Gives the scratch that the calling thread keeps for the training calls back.
+void release_training_scratch();
+
 // Gives the idle buffer sets (take_idle) of the current context back to its
 // device; false when there were none. Those of other devices and contexts stay.
 bool release_idle();

@@ -214,20 +214,58 @@ namespace {
 
 constexpr int kTrainSteps = 512;  // training steps of one launch
 
-// One allocation for a call's device arrays, given back when the call ends.
-struct Scratch {
+// The training scratch that a thread keeps from call to call, at most kKeep
+// bytes (a gradient over 65,536 samples takes 10 MB), in the context it was made in.
+// Allocated and freed by each call it took 0.1 ms of a gradient over 5000 samples
+// (160 us by a call that never freed, 250 us freeing, 80 us kept).
+constexpr size_t kKeep = size_t{32} << 20;
+struct Kept {
   DevBuf buf;
+  unsigned long long context = 0;
+  void release() {
+    if (context && context == context_id()) buf.release();  // another context's stay with it
+    else if (context) return;
+    context = 0;
+  }
+  ~Kept() { release(); }
+};
+thread_local Kept kept;
+
+// One buffer for a call's device arrays: the thread's kept one, or for a large
+// call or in another context one of its own, given back when the call ends.
+struct Scratch {
+  explicit Scratch(cudaStream_t s) : stream(s) {}
+  cudaStream_t stream;
+  DevBuf own;
+  char* base = nullptr;
   size_t used = 0;
-  ~Scratch() { buf.release(); }
+  bool waited = false;  // the call has waited for its stream
+  ~Scratch() {
+    if (own.p) own.release();
+    else if (base && !waited) cudaStreamSynchronize(stream);  // an error: the next call may use another stream
+  }
+  int reserve(size_t bytes) {
+    const unsigned long long id = context_id();
+    const bool keep = id && bytes <= kKeep && (!kept.context || kept.context == id);
+    DevBuf& b = keep ? kept.buf : own;
+    if (int rc = b.reserve(bytes)) return rc;
+    if (keep) kept.context = id;
+    base = static_cast<char*>(b.p);
+    return OCTGRAV_OK;
+  }
   static size_t room(size_t floats) { return (4 * floats + 255) & ~static_cast<size_t>(255); }
   float* take(size_t floats) {
-    float* at = reinterpret_cast<float*>(static_cast<char*>(buf.p) + used);
+    float* at = reinterpret_cast<float*>(base + used);
     used += room(floats);
     return at;
   }
 };
 
 }  // namespace
+
+namespace ogh {
+void release_training_scratch() { kept.release(); }
+}  // namespace ogh
 
 extern "C" {
 
@@ -237,9 +275,9 @@ int octgrav_mlp_grad(const float* params, const float* x, const float* target, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int B = static_cast<int>(n);
   const size_t nx = static_cast<size_t>(og::MLP_NF) * B, np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
-  Scratch S;
-  int rc = S.buf.reserve(2 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + Scratch::room(B) + Scratch::room(np) +
-                         Scratch::room(1));
+  Scratch S(st);
+  int rc = S.reserve(2 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + Scratch::room(B) + Scratch::room(np) +
+                     Scratch::room(1));
   if (rc) return rc;
   float *w = S.take(og::MLP_NPARAM), *g = S.take(og::MLP_NPARAM), *dx = S.take(nx), *dt = S.take(B), *part = S.take(np),
         *dl = S.take(1);
@@ -252,6 +290,7 @@ int octgrav_mlp_grad(const float* params, const float* x, const float* target, i
   CUDA_TRY(cudaMemcpyAsync(grad, g, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(&l, dl, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
+  S.waited = true;
   if (loss) *loss = l;
   return OCTGRAV_OK;
 }
@@ -274,10 +313,10 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   const int B = static_cast<int>(std::min<int64_t>(batch, n));
   const size_t np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
   const size_t nx = static_cast<size_t>(F) * n;
-  Scratch S;
-  int rc = S.buf.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + 2 * Scratch::room(n) +
-                         Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) +
-                         Scratch::room(2 * kTrainSteps) + Scratch::room(2) + Scratch::room(1));
+  Scratch S(st);
+  int rc = S.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + 2 * Scratch::room(n) +
+                     Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) +
+                     Scratch::room(2 * kTrainSteps) + Scratch::room(2) + Scratch::room(1));
   if (rc) return rc;
   float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(nx),
         *dlab = S.take(n), *dy = S.take(n), *part = S.take(np), *dstd = S.take(og::MLP_STD_FLOATS), *drec = S.take(4 * F),
@@ -312,6 +351,7 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   CUDA_TRY(cudaMemcpyAsync(w.data(), dw, 4 * og::MLP_NPARAM, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaMemcpyAsync(&l, dl, 4, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
+  S.waited = true;
   // The range limits are the training extremes widened by kRangeMargin standard
   // deviations: an input equal to an extreme is in range however it is
   // rounded (several inputs take discrete values -- counts, cell sizes -- that

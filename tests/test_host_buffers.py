@@ -313,3 +313,30 @@ def test_parts_of_a_batch_follow_its_widest_angle(fake):
         _forces(T, 0.3)
         assert _last(fake)["nparts"] == parts
     assert narrow > 1
+
+
+def _grad(lib, n):
+    x, t, g = np.zeros((n, 12), np.float32), np.zeros(n, np.float32), np.zeros(5057, np.float32)
+    return lib.octgrav_mlp_grad(g.ctypes.data, x.ctypes.data, t.ctypes.data, n, g.ctypes.data, None, None)
+
+
+def test_training_scratch_is_kept_and_bounded(fake):
+    """A thread's gradient and training calls allocate once; large ones give their
+    buffer back; another context gets its own. (The gradient kernel is not imitated,
+    so every call ends with an error here.)"""
+    G.release_buffers()
+    _grad(fake, 5000)
+    kept, frees = fake.fake_used(0), fake.fake_frees()
+    assert 0 < kept <= 32 << 20
+    for n in (5000, 1, 700):
+        assert _grad(fake, n) == G.ERR_CUDA
+    assert fake.fake_used(0) == kept and fake.fake_frees() == frees
+    _grad(fake, 1000000)
+    assert fake.fake_used(0) == kept                # 52 MB, given back
+    fake.fake_set_context(0, 1 << 22)
+    _grad(fake, 5000)
+    G.release_buffers()
+    assert fake.fake_used(0) == kept                # the first context's is not touched
+    fake.fake_set_context(0, (1 << 22) + 1)
+    _grad(fake, 700)
+    assert fake.fake_used(0) == kept
