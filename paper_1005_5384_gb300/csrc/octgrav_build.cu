@@ -32,6 +32,8 @@ constexpr int SUB = 8;            // blocks per chunk in the key pass
 constexpr int BSUB = 2;           // blocks per chunk in the box pass
 constexpr int LT = 512;           // threads of the level kernel (16 warps) ...
 constexpr int LBMAX = 1024;       // ... and the most blocks it may have
+constexpr int LROUNDS = 16;       // most rounds in which its warps take a level ...
+constexpr int64_t LROUNDS_N = 4000000;  // ... of a tree of at least so many particles
 constexpr int NT = 128;           // threads of the node kernel
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int LBINS = 32;  // leaf size bins of the moment pass (32 = "32 or more")
@@ -94,7 +96,7 @@ Layout layout(int64_t n, int n_sys, int64_t n_chunks, int64_t cap) {
   L.spl = take(4 * 9 * std::min<int64_t>(n, cap));
   L.lpre = take(4 * std::min<int64_t>(n, cap));
   L.nlist = take(4 * cap);
-  L.bsum = take(4 * LBMAX);
+  L.bsum = take(4 * LBMAX * LROUNDS);
   L.lvl = take(4 * (NLEV + 2));
   L.misc = take(4 * MISC);
   L.sstart = take(4 * static_cast<size_t>(n_sys) * NLEV);
@@ -511,25 +513,37 @@ __global__ void k_roots(int n_sys, const int64_t* __restrict__ offs, Cells C, in
 // Split points of a cell holding particles [f, f + cnt): sp[o] = the first
 // position whose child octant at depth D is >= o, sp[0] = f, sp[8] = f + cnt
 // (octants ascend inside a cell). One warp; every lane returns the same sp.
-// The seven boundaries are searched together: a round probes 32 positions a
-// power of two apart of each one's interval, seven independent loads per lane,
-// so a cell of a million particles takes four rounds of load latency, one of at
-// most 1024 two and one of at most 32 a single load. (One boundary after the
-// other took seven times as many rounds; probes at 33rds of the intervals
-// spent 10 us of a level on their 64-bit divisions.)
+// A cell of at most 128 particles has all its keys loaded at once, four a lane,
+// and the particles of the octants below o are counted.
+__device__ __forceinline__ void load_keys(const uint64_t* __restrict__ code, int f, int cnt, int lane, uint64_t* v) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = lane + 32 * j < cnt ? code[f + lane + 32 * j] : 0;
+}
+__device__ __forceinline__ void small_split(const uint64_t* v, int f, int cnt, int D, int lane, int* sp) {
+  const int bit = 3 * (MAXD - D);
+  sp[0] = f;
+  sp[8] = f + cnt;
+#pragma unroll
+  for (int o = 1; o < 8; ++o) sp[o] = f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (32 * j >= cnt) break;
+    const int oc = lane + 32 * j < cnt ? static_cast<int>(v[j] >> bit) & 7 : 8;
+#pragma unroll
+    for (int o = 1; o < 8; ++o) sp[o] += __popc(__ballot_sync(FULL, oc < o));
+  }
+}
+
+// The same for a larger cell. The seven boundaries are searched together: a round
+// probes 32 positions a power of two apart of each one's interval, seven
+// independent loads per lane, so a cell of a million particles takes four rounds
+// of load latency and one of at most 1024 two. (One boundary after the other took
+// seven times as many rounds; probes at 33rds of the intervals spent 10 us of a
+// level on their 64-bit divisions.)
 __device__ void warp_split(const uint64_t* __restrict__ code, int f, int cnt, int D, int lane, int* sp) {
   const int bit = 3 * (MAXD - D);
   sp[0] = f;
   sp[8] = f + cnt;
-  if (cnt <= 32) {  // one probe per particle
-    const int oc = lane < cnt ? static_cast<int>(code[f + lane] >> bit) & 7 : 8;
-#pragma unroll
-    for (int o = 1; o < 8; ++o) {
-      const unsigned m = __ballot_sync(FULL, oc >= o);
-      sp[o] = m ? f + __ffs(m) - 1 : f + cnt;
-    }
-    return;
-  }
   // invariant: boundary o lies in [a[o], b[o]], and b[o] is the end or a known hit
   int a[8], b[8];
 #pragma unroll
@@ -565,8 +579,104 @@ __device__ void no_cells(int* lvl) {
   if (threadIdx.x <= NLEV + 1) lvl[threadIdx.x] = 0;
 }
 
+// Split points of the cells [c0, c1) of the level from lb on that hold more than
+// n_leaf particles, a warp per cell; the keys of the next cell are loaded while one is
+// worked on. Returns the children of all of them.
+__device__ __forceinline__ int split_cells(int c0, int c1, int lb, int L, const uint64_t* __restrict__ code, const Cells& C,
+                                           int n_leaf, int* spl, int* lpre, int* nlist, int* misc) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int mine = 0;
+  for (int base = c0; base < c1; base += 32) {
+    const int c = base + lane;
+    const int cnt = c < c1 ? C.pc[c] : 0;
+    const int f = c < c1 ? C.pf[c] : 0;
+    unsigned todo = __ballot_sync(FULL, cnt > n_leaf);
+    const unsigned nodes = todo;
+    int nch = 0;
+    int kf = 0, kc = 0;  // the cell that is split next: its first particle and their number ...
+    uint64_t v[4];       // ... and its keys, where there are at most 128
+    const auto next = [&]() {
+      const int k = todo ? __ffs(todo) - 1 : 0;
+      kf = __shfl_sync(FULL, f, k);
+      kc = todo ? __shfl_sync(FULL, cnt, k) : 0;
+      if (kc <= 128) load_keys(code, kf, kc, lane, v);
+    };
+    next();
+    while (todo) {
+      const int k = __ffs(todo) - 1, f0 = kf, n0 = kc;
+      todo &= todo - 1;
+      uint64_t u[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) u[j] = v[j];
+      next();
+      int sp[9];
+      if (n0 <= 128) small_split(u, f0, n0, L + 1, lane, sp);
+      else warp_split(code, f0, n0, L + 1, lane, sp);
+      int n = 0, own = sp[0];
+#pragma unroll
+      for (int o = 0; o < 8; ++o) {
+        n += sp[o + 1] > sp[o];
+        own = lane == o + 1 ? sp[o + 1] : own;
+      }
+      if (lane < 9) spl[9 * static_cast<int64_t>(base + k - lb) + lane] = own;
+      if (lane == k) nch = n;
+    }
+    int x = nch;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(FULL, x, d);
+      if (lane >= d) x += y;
+    }
+    int at = 0;
+    if (lane == 0 && nodes) at = atomicAdd(&misc[M_NODES + L], __popc(nodes));
+    at = __shfl_sync(FULL, at, 0);
+    if (nch) {
+      C.nc[c] = nch;
+      lpre[c - lb] = mine + x - nch;
+      nlist[lb + at + __popc(nodes & lt)] = c;
+    }
+    mine += __shfl_sync(FULL, x, 31);
+  }
+  return mine;
+}
+
+// Their children, numbered from `first` on: of the cells that were split four at a
+// time, lane (k, o) writing child o of the k-th.
+__device__ __forceinline__ void emit_cells(int c0, int c1, int lb, int first, const Cells& C, const int* spl, const int* lpre) {
+  const int lane = threadIdx.x & 31, o = lane & 7, sub = lane >> 3;
+  for (int base = c0; base < c1; base += 32) {
+    unsigned nodes = __ballot_sync(FULL, base + lane < c1 && C.nc[base + lane] > 0);
+    while (nodes) {
+      int c = -1;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (nodes && sub == k) c = base + __ffs(nodes) - 1;
+        nodes &= nodes - 1;
+      }
+      int f = 0, e = 0;
+      if (c >= 0) {
+        f = spl[9 * static_cast<int64_t>(c - lb) + o];
+        e = spl[9 * static_cast<int64_t>(c - lb) + o + 1];
+      }
+      const unsigned m = __ballot_sync(FULL, e > f) >> (8 * sub) & 255u;
+      if (e > f) {
+        const int k0 = first + lpre[c - lb], k = k0 + __popc(m & ((1u << o) - 1u));
+        if ((m & ((1u << o) - 1u)) == 0) C.fc[c] = k0;
+        C.key[k] = (C.key[c] << 3) | static_cast<uint64_t>(o);
+        C.par[k] = c;
+        C.pf[k] = f;
+        C.pc[k] = e - f;
+        C.sys[k] = C.sys[c];
+        C.fc[k] = -1;
+        C.nc[k] = 0;
+      }
+    }
+  }
+}
+
 // All levels of the tree in one cooperative launch. Per level: every block
-// takes a contiguous range of the level's cells and finds the split points of
+// takes contiguous ranges of the level's cells and finds the split points of
 // those that hold more than n_leaf particles (a warp per cell); after a
 // barrier every block adds the blocks' children counts up to its own, which
 // places its children in the host's breadth-first order, and writes them;
@@ -577,15 +687,22 @@ __device__ void no_cells(int* lvl) {
 // Latency bounds it: a level is a few dependent rounds of loads and two
 // barriers (5 us; the levels with tens of thousands of cells up to 20 us, where
 // a warp's cells are all split). As three launches per level for 21 levels (4096
-// blocks each, most of them empty) the levels took 425 us at 1M particles and
-// 270 us at 5000 (sum of the launches); 300 us and 77 us now.
+// blocks each, most of them empty) the levels took 412 us at 1M particles and
+// 229 us at 5000 (sum of the launches); 301 us and 79 us now.
+//
+// The cells that are split lie together, so with one range a block a large level
+// waits for the blocks in the dense part. From LROUNDS_N particles on a warp takes
+// up to 16 ranges of at least 32 cells, spread over the level: 4.2M particles 627 ->
+// 590 us, 16M 2100 -> 1210 us, where the three launches a level took 636 and 1460;
+// at 3M 503 us with one range, 540 with several.
+template <int ROUNDS>
 __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ code, Cells C, int n_leaf, int* lvl,
                                                   int* spl, int* lpre, int* nlist, int* bsum, int cap, int* misc) {
   constexpr int W = LT / 32;
-  __shared__ int wsum[W];
-  __shared__ int sh_before, sh_total;
+  static_assert(W >= ROUNDS, "a warp per round");
+  __shared__ int wsum[ROUNDS * W];
+  __shared__ int before[ROUNDS], all[ROUNDS];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, grid = gridDim.x;
-  const unsigned lt = (1u << lane) - 1u;
   int lb = lvl[0], le = lvl[1], bars = 0;
   if (__ldcg(&misc[M_STATUS]) & GPU_BUILD_STUCK) {  // the sort did not finish
     no_cells(lvl);
@@ -593,86 +710,60 @@ __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ c
   }
   for (int L = 0; L < MAXD; ++L) {
     const int nl = le - lb;
-    // cells per warp; block b's warps take consecutive ranges of its range
-    const int per = (nl + grid * W - 1) / (grid * W);
-    const int b0 = lb + static_cast<int>(min(static_cast<int64_t>(blockIdx.x) * per * W, static_cast<int64_t>(nl)));
-    const int c0 = min(le, b0 + w * per), c1 = min(le, c0 + per);
-    int mine = 0;  // children of this warp's cells
-    for (int base = c0; base < c1; base += 32) {
-      const int c = base + lane;
-      const int cnt = c < c1 ? C.pc[c] : 0;
-      const int f = c < c1 ? C.pf[c] : 0;
-      unsigned todo = __ballot_sync(FULL, cnt > n_leaf);
-      const unsigned nodes = todo;
-      int nch = 0;
-      while (todo) {
-        const int k = __ffs(todo) - 1;
-        todo &= todo - 1;
-        int sp[9];
-        warp_split(code, __shfl_sync(FULL, f, k), __shfl_sync(FULL, cnt, k), L + 1, lane, sp);
-        int n = 0, own = sp[0];
-#pragma unroll
-        for (int o = 0; o < 8; ++o) {
-          n += sp[o + 1] > sp[o];
-          own = lane == o + 1 ? sp[o + 1] : own;
-        }
-        if (lane < 9) spl[9 * static_cast<int64_t>(base + k - lb) + lane] = own;
-        if (lane == k) nch = n;
-      }
-      int x = nch;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(FULL, x, d);
-        if (lane >= d) x += y;
-      }
-      int at = 0;
-      if (lane == 0 && nodes) at = atomicAdd(&misc[M_NODES + L], __popc(nodes));
-      at = __shfl_sync(FULL, at, 0);
-      if (nch) {
-        C.nc[c] = nch;
-        lpre[c - lb] = mine + x - nch;
-        nlist[lb + at + __popc(nodes & lt)] = c;
-      }
-      mine += __shfl_sync(FULL, x, 31);
+    // a round gives every warp `per` consecutive cells, a block's warps one after the other
+    const int rounds = ROUNDS == 1 || nl <= 32 * grid * W ? 1 : min(ROUNDS, (nl + grid * W * 32 - 1) / (grid * W * 32));
+    const int per = (nl + grid * W * rounds - 1) / (grid * W * rounds);
+    const auto range = [&](int r) {  // this warp's cells of round r
+      const int c0 = lb + min(((r * grid + static_cast<int>(blockIdx.x)) * W + w) * per, nl);
+      return make_int2(c0, min(le, c0 + per));
+    };
+    const int2 first_range = range(0);
+    for (int r = 0; r < rounds; ++r) {
+      const int2 cells = ROUNDS == 1 ? first_range : range(r);
+      const int c0 = cells.x, c1 = cells.y;
+      const int mine = split_cells(c0, c1, lb, L, code, C, n_leaf, spl, lpre, nlist, misc);
+      if (lane == 0) wsum[r * W + w] = mine;
     }
-    if (lane == 0) wsum[w] = mine;
     __syncthreads();
-    if (w == 0) {  // children before each warp, and the block's
-      const int v = lane < W ? wsum[lane] : 0;
+    if (w < rounds) {  // children before each warp, and the block's, in round w
+      const int v = lane < W ? wsum[w * W + lane] : 0;
       int x = v;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
         const int y = __shfl_up_sync(FULL, x, d);
         if (lane >= d) x += y;
       }
-      if (lane < W) wsum[lane] = x - v;
-      if (lane == 31) bsum[blockIdx.x] = x;
+      if (lane < W) wsum[w * W + lane] = x - v;
+      if (lane == 31) bsum[w * grid + blockIdx.x] = x;
+      if (lane == 0) before[w] = all[w] = 0;
     }
     if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) {
       no_cells(lvl);
       return;
     }
-    {  // children of the blocks before this one, and of all
-      int before = 0, all = 0;
-      for (int b = threadIdx.x; b < grid; b += LT) {
-        const int v = __ldcg(&bsum[b]);
-        all += v;
-        before += b < static_cast<int>(blockIdx.x) ? v : 0;
-      }
+    {  // per round: children of the blocks before this one, and of all
+      const int warps = rounds == 1 ? W : W / rounds, r = rounds == 1 ? 0 : w / warps;
+      if (r < rounds) {
+        int bef = 0, sum = 0;
+        for (int b = 32 * (w - r * warps) + lane; b < grid; b += 32 * warps) {
+          const int v = __ldcg(&bsum[r * grid + b]);
+          sum += v;
+          bef += b < static_cast<int>(blockIdx.x) ? v : 0;
+        }
 #pragma unroll
-      for (int d = 16; d; d >>= 1) {
-        before += __shfl_xor_sync(FULL, before, d);
-        all += __shfl_xor_sync(FULL, all, d);
+        for (int d = 16; d; d >>= 1) {
+          bef += __shfl_xor_sync(FULL, bef, d);
+          sum += __shfl_xor_sync(FULL, sum, d);
+        }
+        if (lane == 0) {
+          atomicAdd(&before[r], bef);
+          atomicAdd(&all[r], sum);
+        }
       }
-      if (threadIdx.x == 0) sh_before = sh_total = 0;
-      __syncthreads();
-      if (lane == 0) {
-        atomicAdd(&sh_before, before);
-        atomicAdd(&sh_total, all);
-      }
-      __syncthreads();
     }
-    const int total = sh_total;
+    __syncthreads();
+    int total = 0;
+    for (int r = 0; r < rounds; ++r) total += all[r];
     const int64_t next = static_cast<int64_t>(le) + total;
     if (total == 0 || next > cap) {  // the same in every block
       if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -683,40 +774,18 @@ __global__ void __launch_bounds__(LT, 2) k_levels(const uint64_t* __restrict__ c
         }
       }
       if (next > cap)  // the unsplit cells are no nodes
-        for (int c = c0 + lane; c < c1; c += 32) C.nc[c] = 0;
+        for (int r = 0; r < rounds; ++r) {
+          const int2 cells = ROUNDS == 1 ? first_range : range(r);
+          for (int c = cells.x + lane; c < cells.y; c += 32) C.nc[c] = 0;
+        }
       return;
     }
-    // emit: of the cells that were split four at a time, lane (k, o) writing
-    // child o of the k-th
-    const int first = le + sh_before + wsum[w];
-    const int o = lane & 7, sub = lane >> 3;
-    for (int base = c0; base < c1; base += 32) {
-      unsigned nodes = __ballot_sync(FULL, base + lane < c1 && C.nc[base + lane] > 0);
-      while (nodes) {
-        int c = -1;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (nodes && sub == k) c = base + __ffs(nodes) - 1;
-          nodes &= nodes - 1;
-        }
-        int f = 0, e = 0;
-        if (c >= 0) {
-          f = spl[9 * static_cast<int64_t>(c - lb) + o];
-          e = spl[9 * static_cast<int64_t>(c - lb) + o + 1];
-        }
-        const unsigned m = __ballot_sync(FULL, e > f) >> (8 * sub) & 255u;
-        if (e > f) {
-          const int k0 = first + lpre[c - lb], k = k0 + __popc(m & ((1u << o) - 1u));
-          if ((m & ((1u << o) - 1u)) == 0) C.fc[c] = k0;
-          C.key[k] = (C.key[c] << 3) | static_cast<uint64_t>(o);
-          C.par[k] = c;
-          C.pf[k] = f;
-          C.pc[k] = e - f;
-          C.sys[k] = C.sys[c];
-          C.fc[k] = -1;
-          C.nc[k] = 0;
-        }
-      }
+    int done = le;  // the rounds before
+    for (int r = 0; r < rounds; done += all[r], ++r) {
+      const int2 cells = ROUNDS == 1 ? first_range : range(r);
+      const int c0 = cells.x, c1 = cells.y;
+      const int first = done + before[r] + wsum[r * W + w];
+      emit_cells(c0, c1, lb, first, C, spl, lpre);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) lvl[L + 2] = static_cast<int>(next);
     if (!grid_barrier(&misc[M_BAR_LEVELS], ++bars * grid, &misc[M_STATUS], GPU_BUILD_STUCK)) {
@@ -1419,6 +1488,7 @@ int grid_for(int64_t n, int per_block) {
   return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16)));
 }
 
+
 // The node kernel: a warp per 4 nodes of a level (a level holds at most n /
 // (n_leaf + 1) nodes) and at most one block per SM: its four warps have a
 // scheduler each, and fewer blocks make cheaper barriers.
@@ -1560,7 +1630,8 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
     // few blocks, whose barriers are cheaper
     const int64_t want = std::max<int64_t>(1, a.n / (16 * (LT / 32)));
     const int most = static_cast<int>(std::min<int64_t>(want, LBMAX));
-    OG_TRY(launch_cooperative(k_levels, resident_blocks(k_levels, LT, most), LT, 0, st, static_cast<const uint64_t*>(keyA), C,
+    const auto kernel = a.n < LROUNDS_N ? k_levels<1> : k_levels<LROUNDS>;
+    OG_TRY(launch_cooperative(kernel, resident_blocks(kernel, LT, most), LT, 0, st, static_cast<const uint64_t*>(keyA), C,
                               a.n_leaf, lvl, spl, lpre, at<int>(S, Lo.nlist), bsum, static_cast<int>(a.cap), misc));
   }
 
