@@ -40,6 +40,11 @@
  *  - Thread safety: distinct trees may be used from distinct threads; one tree
  *    must not be used by two threads at once. The one-shot calls keep their
  *    buffers per calling thread and may run concurrently.
+ *  - Other streams: tree builds on the GPU and the training calls contain
+ *    cooperative launches, which start once all their blocks find room. They take
+ *    at most 11/12 of the SMs' places (half of them in builds of up to 200,000
+ *    particles) and so run beside a kernel on another stream that leaves those
+ *    free; beside one that takes more they wait until it ends.
  *  - Environment (read at first use): OCTGRAV_THREADS = host build threads (default:
  *    all hardware threads); OCTGRAV_HOST_PULL=0 makes a thread's one-shot host-build
  *    call upload with cudaMemcpyAsync only (no copy kernel reading pageable

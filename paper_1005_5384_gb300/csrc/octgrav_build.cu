@@ -1627,9 +1627,11 @@ cudaError_t gpu_build_kernels(const GpuBuild& a, cudaStream_t st) {
                                                                                  at<int>(S, Lo.lhist));
   {
     // about a warp per cell that is split on the widest level; a small tree gets
-    // few blocks, whose barriers are cheaper
+    // few blocks, whose barriers are cheaper; up to 200,000 particles one an SM, half
+    // of the places (65,536 particles 115 us, 119 with two; 131,072 130 and 134; 262,144
+    // 164 and 155)
     const int64_t want = std::max<int64_t>(1, a.n / (16 * (LT / 32)));
-    const int most = static_cast<int>(std::min<int64_t>(want, LBMAX));
+    const int most = static_cast<int>(std::min<int64_t>(want, a.n <= 200000 ? 152 : LBMAX));
     const auto kernel = a.n < LROUNDS_N ? k_levels<1> : k_levels<LROUNDS>;
     OG_TRY(launch_cooperative(kernel, resident_blocks(kernel, LT, most), LT, 0, st, static_cast<const uint64_t*>(keyA), C,
                               a.n_leaf, lvl, spl, lpre, at<int>(S, Lo.nlist), bsum, static_cast<int>(a.cap), misc));
