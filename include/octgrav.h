@@ -506,6 +506,11 @@ int octgrav_set_fault(octgrav_tree *t, int stack_cap, int64_t drop_item);
  * captured graph keeps the split it was captured with. Errors: ERR_ARG. */
 int octgrav_set_split(octgrav_tree *t, int nparts);
 
+/* Let launches of t choose their list split again, as before the first
+ * octgrav_set_split (the next one may allocate the parts' buffer).
+ * Errors: ERR_ARG. */
+int octgrav_auto_split(octgrav_tree *t);
+
 /* Free a tree. Waits until the current device has finished with its buffers. */
 void octgrav_free_tree(octgrav_tree *t);
 

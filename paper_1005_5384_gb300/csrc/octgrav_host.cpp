@@ -1822,6 +1822,12 @@ int octgrav_set_split(octgrav_tree* t, int nparts) {
   return OCTGRAV_OK;
 }
 
+int octgrav_auto_split(octgrav_tree* t) {
+  if (!t) return fail(OCTGRAV_ERR_ARG, "tree is NULL");
+  t->nparts = 0;
+  return OCTGRAV_OK;
+}
+
 int octgrav_set_fault(octgrav_tree* t, int stack_cap, int64_t drop_item) {
   if (!t) return fail(OCTGRAV_ERR_ARG, "tree is NULL");
   if (stack_cap < 0 || drop_item < -1 || drop_item >= t->n_items)

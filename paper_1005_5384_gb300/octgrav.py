@@ -78,6 +78,7 @@ _SIGS = {
     "octgrav_set_staging": (C.c_int, [_vp, C.c_int]),
     "octgrav_set_fault": (C.c_int, [_vp, C.c_int, C.c_int64]),
     "octgrav_set_split": (C.c_int, [_vp, C.c_int]),
+    "octgrav_auto_split": (C.c_int, [_vp]),
     "octgrav_oneshot_phases": (C.c_int, [_vp, C.c_int]),
     "octgrav_mlp_samples": (C.c_int, [_vp, _i64, C.c_int64, C.c_double, C.c_double, _vp, _vp, _vp, C.c_int64,
                                       C.POINTER(C.c_int64), _vp]),
@@ -293,6 +294,10 @@ class Tree:
         the number of work items (up to 3200: 2, 4 or 8 warps), their size, the
         particles per lane and theta."""
         _check(load().octgrav_set_split(self._h, int(nparts)))
+
+    def auto_split(self):
+        """Let launches choose their split again (after set_split)."""
+        _check(load().octgrav_auto_split(self._h))
 
     def set_fault(self, stack_cap: int = 0, drop_item: int = -1):
         """Failure injection for tests: a node stack of stack_cap entries (0 = all),

@@ -340,3 +340,17 @@ def test_training_scratch_is_kept_and_bounded(fake):
     fake.fake_set_context(0, (1 << 22) + 1)
     _grad(fake, 700)
     assert fake.fake_used(0) == kept
+
+
+def test_the_automatic_split_can_be_had_back(fake):
+    T = _upload(_tree(3000))
+    _forces(T)
+    auto, used = _last(fake)["nparts"], fake.fake_used(0)
+    T.set_split(1)
+    _forces(T)
+    assert _last(fake)["nparts"] == 1 < auto
+    T.auto_split()
+    _forces(T)
+    assert _last(fake)["nparts"] == auto and fake.fake_used(0) == used
+    with pytest.raises(G.OctgravError):
+        T.set_split(0)                              # no number of parts
