@@ -20,10 +20,16 @@ struct IdleSet {
 };
 std::mutex idle_mu;
 unsigned long long idle_age = 0;
-// never destroyed: a tree may be freed after static destructors have run
-IdleSet* idle_sets() {
-  static IdleSet* const v = new IdleSet[kIdleSlots];
-  return v;
+// The slots (empty if the host has no memory for them: the calls that use them do
+// not throw); never destroyed, as a tree may be freed after static destructors have run.
+struct IdleSets {
+  IdleSet* v = new (std::nothrow) IdleSet[kIdleSlots];
+  IdleSet* begin() const { return v; }
+  IdleSet* end() const { return v ? v + kIdleSlots : v; }
+};
+const IdleSets& idle_sets() {
+  static const IdleSets s;
+  return s;
 }
 
 }  // namespace
@@ -52,10 +58,10 @@ unsigned long long context_id() {
 static bool take_set(int device, unsigned long long id, size_t need, Device& got) {
   std::lock_guard<std::mutex> g(idle_mu);
   IdleSet* best = nullptr;
-  for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
-    const size_t have = s->D.parts.cap;
-    if (s->context != id || s->D.device != device || (need && (have < need || have > 8 * need + (1 << 20)))) continue;
-    if (!best || have < best->D.parts.cap || (have == best->D.parts.cap && s->age > best->age)) best = s;
+  for (IdleSet& s : idle_sets()) {
+    const size_t have = s.D.parts.cap;
+    if (s.context != id || s.D.device != device || (need && (have < need || have > 8 * need + (1 << 20)))) continue;
+    if (!best || have < best->D.parts.cap || (have == best->D.parts.cap && s.age > best->age)) best = &s;
   }
   if (!best) return false;
   got = std::move(best->D);
@@ -76,9 +82,10 @@ void take_idle(int device, int64_t n, Device& D) {
   const unsigned long long id = context_id();
   Device got;
   if (!id || !take_set(device, id, 2 * sizeof(float4) * static_cast<size_t>(n), got)) return;
-  std::vector<DevBuf*> mine;  // what D already holds stays (a criterion set before the upload)
-  D.for_each([&](DevBuf& b) { mine.push_back(&b); });
+  DevBuf* mine[Device::kBuffers];  // what D already holds stays (a criterion set before the upload)
   size_t k = 0;
+  D.for_each([&](DevBuf& b) { mine[k++] = &b; });
+  k = 0;
   got.for_each([&](DevBuf& b) {
     if (!mine[k]->p) std::swap(*mine[k], b);
     ++k;
@@ -118,15 +125,15 @@ void give_idle(Device& D) {
       IdleSet *slot = nullptr, *other = nullptr, *oldest = nullptr;
       int mine = 0;
       size_t sum = bytes;
-      for (IdleSet* s = idle_sets(); s < idle_sets() + kIdleSlots; ++s) {
-        if (!s->context) {
-          slot = s;
-        } else if (s->D.device == cur && s->context == id) {
+      for (IdleSet& s : idle_sets()) {
+        if (!s.context) {
+          slot = &s;
+        } else if (s.D.device == cur && s.context == id) {
           ++mine;
-          sum += s->bytes;
-          if (!oldest || s->age < oldest->age) oldest = s;
-        } else if (s->D.device == cur && (!other || s->age < other->age)) {
-          other = s;
+          sum += s.bytes;
+          if (!oldest || s.age < oldest->age) oldest = &s;
+        } else if (s.D.device == cur && (!other || s.age < other->age)) {
+          other = &s;
         }
       }
       if (!slot) slot = other;

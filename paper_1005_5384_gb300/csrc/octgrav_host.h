@@ -332,12 +332,14 @@ struct Device {
     for (DevBuf& b : outgrown) b.release();
     cell_cap = 0;
   }
+  static constexpr size_t kBuffers = 28;
   template <class F>
   void for_each(F f) {
-    for (DevBuf* b : {&parts, &geo, &link, &mp, &items, &ibox, &sysp, &out, &counts, &ctl, &dbg, &mlp, &perm, &key,
-                      &props, &pcount, &cfirst, &groups, &ikey, &celloff, &result, &scratch, &in_pos, &in_mass,
-                      &acc64, &pot64, &order, &split})
-      f(*b);
+    DevBuf* const all[] = {&parts, &geo, &link, &mp, &items, &ibox, &sysp, &out, &counts, &ctl, &dbg, &mlp, &perm, &key,
+                           &props, &pcount, &cfirst, &groups, &ikey, &celloff, &result, &scratch, &in_pos, &in_mass,
+                           &acc64, &pot64, &order, &split};
+    static_assert(sizeof(all) / sizeof(all[0]) == kBuffers, "every buffer once");
+    for (DevBuf* b : all) f(*b);
   }
 };
 

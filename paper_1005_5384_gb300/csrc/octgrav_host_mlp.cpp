@@ -217,7 +217,7 @@ constexpr int kTrainSteps = 512;  // training steps of one launch
 // The training scratch that a thread keeps from call to call, at most kKeep
 // bytes (a gradient over 65,536 samples takes 10 MB), in the context it was made in.
 // Allocated and freed by each call it took 0.1 ms of a gradient over 5000 samples
-// (160 us by a call that never freed, 250 us freeing, 80 us kept).
+// (150 us by a call that never freed, 250 us freeing, 90 us kept).
 constexpr size_t kKeep = size_t{32} << 20;
 struct Kept {
   DevBuf buf;
