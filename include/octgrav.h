@@ -34,9 +34,9 @@
  *    default stream). Device memory owned by a tree is allocated by the
  *    library (cudaMalloc) on the current CUDA device and given up by
  *    octgrav_free_tree. The library keeps the buffers of up to two freed trees,
- *    1 GiB together, per device for the next trees, and each thread's training
- *    calls keep up to 32 MiB; octgrav_release_buffers gives them back, as does (the
- *    trees') an allocation of the library's own that fails.
+ *    1 GiB together, per device for the next trees, and each thread up to 32 MiB
+ *    of its last octgrav_direct or training call; octgrav_release_buffers gives
+ *    them back, as does (the trees') an allocation of the library's own that fails.
  *  - Thread safety: distinct trees may be used from distinct threads; one tree
  *    must not be used by two threads at once. The one-shot calls keep their
  *    buffers per calling thread and may run concurrently.
@@ -514,9 +514,9 @@ int octgrav_auto_split(octgrav_tree *t);
 /* Free a tree. Waits until the current device has finished with its buffers. */
 void octgrav_free_tree(octgrav_tree *t);
 
-/* Give the buffers kept from freed trees, and by the calling thread's training
- * calls, back to the current device, for another allocator of the process (trees
- * in use keep theirs). Returns OK. */
+/* Give the buffers kept from freed trees, and the calling thread's scratch of
+ * direct sums and training calls, back to the current device, for another
+ * allocator of the process (trees in use keep theirs). Returns OK. */
 int octgrav_release_buffers(void);
 
 #define OCTGRAV_NOALLOC_MAX_ITEMS 262144 /* work items accepted by octgrav_forces_noalloc */

@@ -158,6 +158,40 @@ void give_idle(Device& D) {
   D.release();
 }
 
+namespace {
+
+constexpr size_t kScratchKept = size_t{32} << 20;
+struct KeptScratch {
+  DevBuf buf;
+  unsigned long long context = 0;
+  void release() {
+    if (!context || context != context_id()) return;  // another context's stays with it
+    buf.release();
+    context = 0;
+  }
+  ~KeptScratch() { release(); }
+};
+thread_local KeptScratch kept;
+
+}  // namespace
+
+void release_scratch() { kept.release(); }
+
+int Scratch::reserve(size_t bytes) {
+  const unsigned long long id = context_id();
+  const bool keep = id && bytes <= kScratchKept && (!kept.context || kept.context == id);
+  DevBuf& b = keep ? kept.buf : own;
+  if (int rc = b.reserve(bytes)) return rc;
+  if (keep) kept.context = id;
+  base = static_cast<char*>(b.p);
+  return OCTGRAV_OK;
+}
+
+Scratch::~Scratch() {
+  if (own.p) own.release();
+  else if (base && !waited) cudaStreamSynchronize(stream);  // an error: the next call may use another stream
+}
+
 // Host memory reused by a thread's one-shot calls: the per-system build
 // arrays and the tree's host images keep their pages from call to call (at
 // N = 1M a call otherwise touches ~200 MB of fresh memory).
@@ -1147,23 +1181,24 @@ int octgrav_direct(const double* pos, const double* mass, int64_t n, const int64
       if (targets[k] < 0 || targets[k] >= n) return fail(OCTGRAV_ERR_ARG, "target %lld out of range", (long long)k);
   if (nt == 0) return OCTGRAV_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  DevBuf dp, dm, dt, dpart, da, dpot;
-  int rc;
-  if ((rc = dp.reserve(24 * n)) || (rc = dm.reserve(8 * n)) || (rc = dt.reserve(targets ? 8 * nt : 8)) ||
-      (rc = dpart.reserve(32 * og::direct_chunks(n, nt) * nt)) || (rc = da.reserve(24 * nt)) || (rc = dpot.reserve(8 * nt)))
+  const size_t zn = static_cast<size_t>(n), zt = static_cast<size_t>(nt);
+  const size_t np = 4 * static_cast<size_t>(og::direct_chunks(n, nt)) * zt;
+  Scratch S(st);
+  if (int rc = S.reserve(Scratch::room(24 * zn) + Scratch::room(8 * zn) + 2 * Scratch::room(8 * zt) + Scratch::room(8 * np) +
+                         Scratch::room(24 * zt)))
     return rc;
-  CUDA_TRY(cudaMemcpyAsync(dp.p, pos, 24 * n, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemcpyAsync(dm.p, mass, 8 * n, cudaMemcpyHostToDevice, st));
-  if (targets) CUDA_TRY(cudaMemcpyAsync(dt.p, targets, 8 * nt, cudaMemcpyHostToDevice, st));
-  cudaError_t e = og::direct_sum(static_cast<const double*>(dp.p), static_cast<const double*>(dm.p), n,
-                                 targets ? static_cast<const int64_t*>(dt.p) : nullptr, nt, eps, G,
-                                 static_cast<double*>(dpart.p), static_cast<double*>(da.p),
-                                 static_cast<double*>(dpot.p), st);
+  double *dp = S.take<double>(3 * zn), *dm = S.take<double>(zn), *part = S.take<double>(np), *da = S.take<double>(3 * zt),
+         *dpot = S.take<double>(zt);
+  int64_t* dt = S.take<int64_t>(zt);
+  CUDA_TRY(cudaMemcpyAsync(dp, pos, 24 * n, cudaMemcpyHostToDevice, st));
+  CUDA_TRY(cudaMemcpyAsync(dm, mass, 8 * n, cudaMemcpyHostToDevice, st));
+  if (targets) CUDA_TRY(cudaMemcpyAsync(dt, targets, 8 * nt, cudaMemcpyHostToDevice, st));
+  cudaError_t e = og::direct_sum(dp, dm, n, targets ? dt : nullptr, nt, eps, G, part, da, dpot, st);
   if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "direct-sum launch failed: %s", cudaGetErrorString(e));
-  CUDA_TRY(cudaMemcpyAsync(acc, da.p, 24 * nt, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(pot, dpot.p, 8 * nt, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(acc, da, 24 * nt, cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(pot, dpot, 8 * nt, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
-  for (DevBuf* b : {&dp, &dm, &dt, &dpart, &da, &dpot}) b->release();
+  S.waited = true;
   return OCTGRAV_OK;
 }
 
@@ -1853,7 +1888,7 @@ int octgrav_set_staging(octgrav_tree* t, int mode) {
 
 int octgrav_release_buffers(void) {
   release_idle();
-  release_training_scratch();
+  release_scratch();
   return OCTGRAV_OK;
 }
 

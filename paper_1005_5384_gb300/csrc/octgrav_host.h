@@ -263,8 +263,8 @@ int build_system(const double* pos, const double* mass, int64_t n, int n_leaf, i
 
 // Identity of the current context, never used twice (0: unknown).
 unsigned long long context_id();
-// Gives the scratch that the calling thread keeps for the training calls back.
-void release_training_scratch();
+// Gives the calling thread's kept scratch back (Scratch).
+void release_scratch();
 
 // Gives the idle buffer sets (take_idle) of the current context back to its
 // device; false when there were none. Those of other devices and contexts stay.
@@ -297,6 +297,33 @@ struct DevBuf {
     p = nullptr;
     cap = 0;
   }
+};
+
+// One device buffer for the arrays of a call that waits for its stream (direct sums,
+// gradients, training): the one that the calling thread keeps from call to call
+// (at most 32 MiB, in the context it was made in), or for a larger call or in another
+// context one of its own, given back when the call ends. An allocation and its
+// cudaFree take 70 us where no small ones are alive: a gradient over 5000 samples
+// 250 us with, 90 us kept.
+struct Scratch {
+  explicit Scratch(cudaStream_t s) : stream(s) {}
+  ~Scratch();
+  Scratch(const Scratch&) = delete;
+  int reserve(size_t bytes);
+  static size_t room(size_t bytes) { return (bytes + 255) & ~static_cast<size_t>(255); }
+  template <class T>
+  T* take(size_t count) {  // the next array; `room` bytes of what was reserved
+    T* const at = reinterpret_cast<T*>(base + used);
+    used += room(sizeof(T) * count);
+    return at;
+  }
+  bool waited = false;  // set once the call has waited for its stream
+
+ private:
+  cudaStream_t stream;
+  DevBuf own;
+  char* base = nullptr;
+  size_t used = 0;
 };
 
 struct Device {

@@ -214,58 +214,10 @@ namespace {
 
 constexpr int kTrainSteps = 512;  // training steps of one launch
 
-// The training scratch that a thread keeps from call to call, at most kKeep
-// bytes (a gradient over 65,536 samples takes 10 MB), in the context it was made in.
-// Allocated and freed by each call it took 0.1 ms of a gradient over 5000 samples
-// (150 us by a call that never freed, 250 us freeing, 90 us kept).
-constexpr size_t kKeep = size_t{32} << 20;
-struct Kept {
-  DevBuf buf;
-  unsigned long long context = 0;
-  void release() {
-    if (context && context == context_id()) buf.release();  // another context's stay with it
-    else if (context) return;
-    context = 0;
-  }
-  ~Kept() { release(); }
-};
-thread_local Kept kept;
-
-// One buffer for a call's device arrays: the thread's kept one, or for a large
-// call or in another context one of its own, given back when the call ends.
-struct Scratch {
-  explicit Scratch(cudaStream_t s) : stream(s) {}
-  cudaStream_t stream;
-  DevBuf own;
-  char* base = nullptr;
-  size_t used = 0;
-  bool waited = false;  // the call has waited for its stream
-  ~Scratch() {
-    if (own.p) own.release();
-    else if (base && !waited) cudaStreamSynchronize(stream);  // an error: the next call may use another stream
-  }
-  int reserve(size_t bytes) {
-    const unsigned long long id = context_id();
-    const bool keep = id && bytes <= kKeep && (!kept.context || kept.context == id);
-    DevBuf& b = keep ? kept.buf : own;
-    if (int rc = b.reserve(bytes)) return rc;
-    if (keep) kept.context = id;
-    base = static_cast<char*>(b.p);
-    return OCTGRAV_OK;
-  }
-  static size_t room(size_t floats) { return (4 * floats + 255) & ~static_cast<size_t>(255); }
-  float* take(size_t floats) {
-    float* at = reinterpret_cast<float*>(base + used);
-    used += room(floats);
-    return at;
-  }
-};
+// Bytes of an array of floats in a call's scratch.
+size_t room(size_t floats) { return Scratch::room(4 * floats); }
 
 }  // namespace
-
-namespace ogh {
-void release_training_scratch() { kept.release(); }
-}  // namespace ogh
 
 extern "C" {
 
@@ -276,11 +228,11 @@ int octgrav_mlp_grad(const float* params, const float* x, const float* target, i
   const int B = static_cast<int>(n);
   const size_t nx = static_cast<size_t>(og::MLP_NF) * B, np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
   Scratch S(st);
-  int rc = S.reserve(2 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + Scratch::room(B) + Scratch::room(np) +
-                     Scratch::room(1));
+  int rc = S.reserve(2 * room(og::MLP_NPARAM) + room(nx) + room(B) + room(np) +
+                     room(1));
   if (rc) return rc;
-  float *w = S.take(og::MLP_NPARAM), *g = S.take(og::MLP_NPARAM), *dx = S.take(nx), *dt = S.take(B), *part = S.take(np),
-        *dl = S.take(1);
+  float *w = S.take<float>(og::MLP_NPARAM), *g = S.take<float>(og::MLP_NPARAM), *dx = S.take<float>(nx), *dt = S.take<float>(B), *part = S.take<float>(np),
+        *dl = S.take<float>(1);
   CUDA_TRY(cudaMemcpyAsync(w, params, 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dx, x, 4 * nx, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dt, target, 4 * n, cudaMemcpyHostToDevice, st));
@@ -314,17 +266,17 @@ int octgrav_mlp_train(const float* features, const float* labels, int64_t n, int
   const size_t np = og::MLP_PART * static_cast<size_t>(og::mlp_blocks(B));
   const size_t nx = static_cast<size_t>(F) * n;
   Scratch S(st);
-  int rc = S.reserve(3 * Scratch::room(og::MLP_NPARAM) + Scratch::room(nx) + 2 * Scratch::room(n) +
-                     Scratch::room(np) + Scratch::room(og::MLP_STD_FLOATS) + Scratch::room(4 * F) +
-                     Scratch::room(2 * kTrainSteps) + Scratch::room(2) + Scratch::room(1));
+  int rc = S.reserve(3 * room(og::MLP_NPARAM) + room(nx) + 2 * room(n) +
+                     room(np) + room(og::MLP_STD_FLOATS) + room(4 * F) +
+                     room(2 * kTrainSteps) + room(2) + room(1));
   if (rc) return rc;
-  float *dw = S.take(og::MLP_NPARAM), *dm = S.take(og::MLP_NPARAM), *dv = S.take(og::MLP_NPARAM), *dx = S.take(nx),
-        *dlab = S.take(n), *dy = S.take(n), *part = S.take(np), *dstd = S.take(og::MLP_STD_FLOATS), *drec = S.take(4 * F),
-        *dcoef = S.take(2 * kTrainSteps), *dbar = S.take(2), *dl = S.take(1);
+  float *dw = S.take<float>(og::MLP_NPARAM), *dm = S.take<float>(og::MLP_NPARAM), *dv = S.take<float>(og::MLP_NPARAM), *dx = S.take<float>(nx),
+        *dlab = S.take<float>(n), *dy = S.take<float>(n), *part = S.take<float>(np), *dstd = S.take<float>(og::MLP_STD_FLOATS), *drec = S.take<float>(4 * F),
+        *dcoef = S.take<float>(2 * kTrainSteps), *dbar = S.take<float>(2), *dl = S.take<float>(1);
   CUDA_TRY(cudaMemcpyAsync(dx, features, 4 * nx, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dlab, labels, 4 * n, cudaMemcpyHostToDevice, st));
   CUDA_TRY(cudaMemcpyAsync(dw, w.data(), 4 * og::MLP_NPARAM, cudaMemcpyHostToDevice, st));
-  CUDA_TRY(cudaMemsetAsync(dm, 0, 2 * Scratch::room(og::MLP_NPARAM), st));  // dm and dv follow each other
+  CUDA_TRY(cudaMemsetAsync(dm, 0, 2 * room(og::MLP_NPARAM), st));  // dm and dv follow each other
   {  // targets: log10 of the error label; inputs standardised per feature
     const cudaError_t e = og::mlp_standardise(dx, dlab, n, dstd, dy, drec, st);
     if (e != cudaSuccess) return fail(OCTGRAV_ERR_CUDA, "standardisation failed: %s", cudaGetErrorString(e));

@@ -320,19 +320,25 @@ def _grad(lib, n):
     return lib.octgrav_mlp_grad(g.ctypes.data, x.ctypes.data, t.ctypes.data, n, g.ctypes.data, None, None)
 
 
-def test_training_scratch_is_kept_and_bounded(fake):
-    """A thread's gradient and training calls allocate once; large ones give their
-    buffer back; another context gets its own. (The gradient kernel is not imitated,
-    so every call ends with an error here.)"""
+def _direct(lib, n):
+    x, m, a, p = np.zeros((n, 3)), np.zeros(n), np.zeros((2, 3)), np.zeros(2)
+    return lib.octgrav_direct(x.ctypes.data, m.ctypes.data, n, None, 2, 0.01, 1.0, a.ctypes.data, p.ctypes.data, None)
+
+
+def test_scratch_is_kept_and_bounded(fake):
+    """A thread's direct sums, gradients and training calls allocate once; large ones
+    give their buffer back; another context gets its own. (The kernels are not
+    imitated, so every call ends with an error here.)"""
     G.release_buffers()
     _grad(fake, 5000)
     kept, frees = fake.fake_used(0), fake.fake_frees()
     assert 0 < kept <= 32 << 20
     for n in (5000, 1, 700):
-        assert _grad(fake, n) == G.ERR_CUDA
+        assert _grad(fake, n) == G.ERR_CUDA and _direct(fake, n + 1) == G.ERR_CUDA
     assert fake.fake_used(0) == kept and fake.fake_frees() == frees
     _grad(fake, 1000000)
-    assert fake.fake_used(0) == kept                # 52 MB, given back
+    _direct(fake, 1200000)
+    assert fake.fake_used(0) == kept                # 52 and 38 MB, given back
     fake.fake_set_context(0, 1 << 22)
     _grad(fake, 5000)
     G.release_buffers()
