@@ -477,7 +477,8 @@ ONESHOT_PHASES = ("bbox_check", "morton", "sort", "gather_records", "levels", "c
 
 def release_buffers():
     """Give the device buffers that the library keeps from freed trees (up to
-    1 GiB) back to the current device."""
+    1 GiB), and the calling thread's scratch of direct sums and training (up to
+    32 MiB), back to the current device."""
     _check(load().octgrav_release_buffers())
 
 
