@@ -42,9 +42,9 @@
  *    buffers per calling thread and may run concurrently.
  *  - Other streams: tree builds on the GPU and the training calls contain
  *    cooperative launches, which start once all their blocks find room. They take
- *    at most 11/12 of the SMs' places (half of them in builds of up to 200,000
- *    particles) and so run beside a kernel on another stream that leaves those
- *    free; beside one that takes more they wait until it ends.
+ *    at most eleven twelfths of what an idle GPU holds and so run beside a kernel
+ *    on another stream that leaves that room; beside one that takes more they wait
+ *    until it ends.
  *  - Environment (read at first use): OCTGRAV_THREADS = host build threads (default:
  *    all hardware threads); OCTGRAV_HOST_PULL=0 makes a thread's one-shot host-build
  *    call upload with cudaMemcpyAsync only (no copy kernel reading pageable
