@@ -379,9 +379,9 @@ static_assert(16 * 32 + 4 * 32 <= 32 * 32, "packed sources and indices must fit 
 // 1M particles (7.62 to 8.0 ms) this was the fastest; in place 7.67 ms, the same with
 // a packed potential 7.77. Other scalar splits were slower, as issue slots run
 // out. The learned kernel keeps the potential packed (1.72 against 1.74 ms).
-// The quadrupole's potential through r^-3 instead of r^-5: 7.66 ms either way at 1M
-// particles, 1.217 either way for the galaxy of 300k, 1.736 instead of 1.722 with the
-// learned criterion.
+// The quadrupole's potential through r^-3 instead of r^-5 costs nothing in this order
+// (y, z, x): 7.65 ms at 1M particles (7.66 with r^-5), 1.215 for the galaxy of 300k
+// (1.216), 1.724 with the learned criterion (1.722; 1.736 with z, x, y).
 template <bool SP>
 __device__ __forceinline__ void body_cellP(float2 X, float2 Y, float2 Z, float2 eps2, const CellRec& c,
                                            Acc2& a) {
@@ -403,9 +403,9 @@ __device__ __forceinline__ void body_cellP(float2 X, float2 Y, float2 Z, float2 
   const float2 q = fma2(sx, dx, fma2(dz, sz, fma2(dy, sy, f2(c.k))));
   const float2 t = mul2(rinv2, q);
   const float2 cb = fma2(f2(-2.5f), t, mul2(r2, f2(c.nM)));
+  a.y = fma2(fma2(cb, dy, sy), rinv5, a.y);
   a.z = fma2(fma2(cb, dz, sz), rinv5, a.z);
   a.x = fma2(fma2(dx, cb, sx), rinv5, a.x);
-  a.y = fma2(fma2(cb, dy, sy), rinv5, a.y);
   a.p = SP ? fma1(rinv, f2(c.M2), a.p) : fma2(rinv, f2(c.M2), a.p);
   a.w = fma2(t, rinv3, a.w);
 }
