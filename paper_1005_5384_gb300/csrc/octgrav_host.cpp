@@ -862,6 +862,9 @@ int build_gpu_common(int n_sys, const int64_t* offsets, const double* pos, const
     t->cell_cap = cap;
     og::GpuBuild a = gpu_args(t.get(), offsets, pos, mass);
     if ((rc = run_build(D, a, st, dev != nullptr))) return rc;  // cached buffers: replay a graph
+    // the buffer that give_idle frees, allocated while the build runs (3 us of a step of
+    // 5000 particles where upload did it, after the build)
+    if ((rc = D.ctl.reserve(64))) return rc;
     if ((rc = gpu_result(t.get(), st, res))) return rc;
     if (res[og::GB_STATUS] & og::GPU_BUILD_BADINPUT)
       return fail(OCTGRAV_ERR_NONFINITE, "non-finite position/mass or negative mass");
